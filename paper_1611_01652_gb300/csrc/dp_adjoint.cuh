@@ -56,7 +56,8 @@ __device__ void loss_reverse(const DevTopo& T, const BLaneT<RV>& B, const SL& X,
 // XB holds the adjoint of x_{t+1}; on return its p/R fields hold the adjoint of x_t's p/R,
 // its v/w fields are zero, and VB holds the adjoint of the solver's output velocities.
 // (bmask: the bodies to process, bit b)
-__device__ inline void integrate_reverse(const DevTopo& T, const GC& Xt, const SL& X, const SL& XB, const SL& VB,
+template <class XT>
+__device__ __forceinline__ void integrate_reverse(const DevTopo& T, const XT& Xt, const SL& X, const SL& XB, const SL& VB,
                                   uint32_t bmask = 0xffffffffu) {
   const float h = T.dt;
   for (int b = 0; b < T.nb; ++b) {
@@ -594,12 +595,13 @@ __device__ void servo_reverse(const DevTopo& T, const BLaneT<RV>& B, const AV& u
 }
 
 // One dense layer reversed on this lane: in_bar[i] (+)= sum_o W[o][i] out_bar[o], using the
-// [out][in_pad] weight copy; the ReLU mask of the input is applied when `mask` is set.
+// [out][in_pad] weight copy; the ReLU mask of the input is applied when `mask` is set (the passes
+// i_first, i_first + i_step, ... of 8 inputs only, so that several warps may share a layer).
 template <class AVD, class AVA, class AVI>
 __device__ void dense_bwd(const float* __restrict__ Wn, int ni, int no, const AVD& outb, const AVA& in_act,
-                          const AVI& inb, bool mask, bool accumulate) {
+                          const AVI& inb, bool mask, bool accumulate, int i_first = 0, int i_step = 8) {
   const int nip = (ni + 7) & ~7;
-  for (int i0 = 0; i0 < ni; i0 += 8) {
+  for (int i0 = i_first; i0 < ni; i0 += i_step) {
     float acc[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) acc[k] = 0.f;

@@ -235,6 +235,85 @@ void plan_smem(DevTopo& T, bool backward, int smem_floats_max, bool rows_on_chip
   T.sm_total = o;
 }
 
+// Shared-memory plans of the four-warp step (units of 32 floats). Forward; the first `keep` units stay
+// free (the reverse pass's segment recompute leaves its state adjoint there).
+void plan_smem_blk_fwd(DevTopo& T, int keep = 0) {
+  int o = keep;
+  auto take = [&](int n) { int r = o; o += std::max(n, 1); return r; };
+  T.sm_x = take(18 * T.nb);
+  T.sm_iinv = take(6 * T.nb);
+  T.sm_invm = take(T.nb);
+  T.sm_th = take(T.nj);
+  T.sm_thd = take(T.nj);
+  T.sm_ua = take(3 * T.nj);
+  T.sm_wst = take(T.nj);
+  T.sm_wbr = take(T.nj);
+  T.sm_lam = take(T.nslots);
+  T.sm_h = take(T.n_rec);
+  T.sm_ws = take(76 + T.n_wsg);  // learned start: features and outputs per warp, harvest row ids
+  T.sm_prog = take((T.blk_bytes_total + 127) / 128);
+  // controller activations and the records share one region: the records are assembled after the
+  // servo targets have consumed the controller output
+  const int region = o;
+  int acts = 0;
+  for (int l = 0; l <= DPK_MAXL; ++l) T.sm_act[l] = region;
+  if (T.ext_ctrl || T.mlp_tc) {
+    T.sm_act[0] = region;
+    T.sm_act[T.n_layers] = region + T.widths[0];
+    acts = T.widths[0] + T.widths[T.n_layers];
+    T.sm_hbuf = region + acts;
+    if (T.mlp_tc) acts += T.widths[1] + 8;  // two layers of [32][H + 8] bfloat16
+  } else if (T.n_layers > 0) {
+    for (int l = 0; l <= T.n_layers; ++l) { T.sm_act[l] = region + acts; acts += T.widths[l]; }
+  }
+  T.sm_rows = region;
+  T.rec_j = 64;
+  T.rec_c = 17;
+  T.rec_p = 50;
+  T.sm_total = region + std::max({acts, T.rec_j * T.nj + T.rec_c * T.ns + T.rec_p * T.np, 1});
+}
+// Reverse. Returns the units in front of the layout that outlive a step (state adjoint, h's adjoint).
+int plan_smem_blk_bwd(DevTopo& T) {
+  int o = 0;
+  auto take = [&](int n) { int r = o; o += std::max(n, 1); return r; };
+  T.sm_xb = take(18 * T.nb);
+  T.sm_hb = take(T.n_rec);
+  const int keep = o;
+  T.sm_x = take(18 * T.nb);
+  T.sm_vb = take(6 * T.nb);
+  T.sm_vw = take(6 * T.nb);
+  T.sm_iinv = take(6 * T.nb);
+  T.sm_invm = take(T.nb);
+  T.sm_iinvb = take(6 * T.nb);
+  T.sm_invmb = take(T.nb);
+  T.sm_th = take(T.nj);
+  T.sm_thd = take(T.nj);
+  T.sm_ua = take(3 * T.nj);
+  T.sm_wst = take(T.nj);
+  T.sm_wbr = take(T.nj);
+  T.sm_thb = take(T.nj);
+  T.sm_thdb = take(T.nj);
+  T.sm_uab = take(3 * T.nj);
+  T.sm_wstb = take(T.nj);
+  T.sm_lam = take(T.nslots);
+  T.sm_sbar = take(T.n_layers > 0 && !T.ext_ctrl ? T.widths[0] : 1);
+  T.sm_zb = take(T.n_layers > 0 ? std::max(T.widths[T.n_layers], 16) : 1);
+  T.sm_prog = take((T.blk_bytes_total + 127) / 128);
+  T.sm_rows = T.sm_hbuf = o;
+  T.rec_j = 58;
+  T.rec_c = 21;
+  T.rec_p = 64;
+  int buf = 1;  // the controller's buffers lie over the records
+  if (T.mlp_tc) buf = 2 * (T.widths[1] + 8);  // four planes of [32][H + 8] bfloat16
+  if (T.n_layers > 0 && !T.mlp_tc && !T.ext_ctrl) {
+    int maxw = 1;
+    for (int l = 0; l <= T.n_layers; ++l) maxw = std::max(maxw, T.widths[l]);
+    buf = 2 * maxw;
+  }
+  T.sm_total = o + std::max(buf, T.rec_j * T.nj + T.rec_c * T.ns + T.rec_p * T.np);
+  return keep;
+}
+
 void pack_param(std::vector<float>& h, int Bp, int B, int field0, int n, const float* src) {
   if (!src) return;
   for (int i = 0; i < Bp; ++i) {
@@ -482,6 +561,26 @@ dp_status dp_create_world(const dp_batch_desc* d, void* stream, dp_world** out) 
   CU(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   plan_smem(w->Tf, false, smem_max / (int)sizeof(float), d->rows_global == 0);
   plan_smem(w->Tb, true, smem_max / (int)sizeof(float));
+  // The four-warp step, unless the world asks for one warp per group or rows in global memory (or
+  // the environment forces the one-warp kernels, for comparison).
+  std::vector<int32_t> prog;
+  if (!T.one_warp && d->rows_global == 0 && plan_blocks(T, prog)) {
+    DevTopo f = T;
+    plan_smem_blk_fwd(f);
+    if ((size_t)f.sm_total * 128 <= (size_t)smem_max && !getenv("DP_SINGLE_WARP_FORWARD")) {
+      f.blk_fwd = 1;
+      w->Tf = f;
+    }
+    DevTopo b = T;
+    w->Ts = T;
+    plan_smem_blk_fwd(w->Ts, plan_smem_blk_bwd(b));
+    if ((size_t)std::max(b.sm_total, w->Ts.sm_total) * 128 <= (size_t)smem_max && !getenv("DP_SINGLE_WARP_BACKWARD")) {
+      b.blk_bwd = 1;
+      w->Tb = b;
+    }
+  }
+  // only the one-warp reverse reads the rows from the tape
+  w->Tf.rec_rows = w->Tb.rec_rows = w->Ts.rec_rows = T.rec_rows = !w->Tb.blk_bwd;
   size_t need = (size_t)std::max(w->Tf.sm_total, w->Tb.sm_total) * 32 * sizeof(float);
   if (need > (size_t)smem_max) {
     dp_status s = fail(DP_EINVAL, "robot too large: needs " + std::to_string(need) + " bytes of shared memory per warp, the device offers " +
@@ -494,10 +593,10 @@ dp_status dp_create_world(const dp_batch_desc* d, void* stream, dp_world** out) 
   const int nf = 18 * T.nb;
   w->nf = nf;
   const size_t state_bytes = (size_t)nf * Bp * sizeof(float);
-  // tape record of one (step, warp): rows, impulses, per-sweep velocities, post-impulse
+  // tape record of one (step, warp): rows (one-warp reverse only), impulses, per-sweep velocities, post-impulse
   // velocities, clamp branches; 32 lanes interleaved; 16-byte multiple for bulk prefetches
   {
-    long long o = (long long)T.nslots * RF_N * 32 * 4;
+    long long o = T.rec_rows ? (long long)T.nslots * RF_N * 32 * 4 : 0;
     T.rec_lam = o;
     o += (long long)T.iters * T.nslots * 32 * 4;
     T.rec_viter = o;
@@ -510,7 +609,7 @@ dp_status dp_create_world(const dp_batch_desc* d, void* stream, dp_world** out) 
     T.rec_lam0 = o;
     if (d->warmstart) o += (long long)T.nslots * 32 * 4;
     T.rec_bytes = (o + 255) / 256 * 256;
-    for (DevTopo* t2 : {&w->Tf, &w->Tb}) {
+    for (DevTopo* t2 : {&w->Tf, &w->Tb, &w->Ts}) {
       t2->rec_lam = T.rec_lam;
       t2->rec_viter = T.rec_viter;
       t2->rec_vminus = T.rec_vminus;
@@ -619,6 +718,16 @@ dp_status dp_create_world(const dp_batch_desc* d, void* stream, dp_world** out) 
     CU(cudaMemsetAsync(dummy, 0, 8 * sizeof(float), w->stream));
     D.Wt = D.Wn = D.bias = dummy;
     D.dump = dummy;
+  }
+  if (w->Tf.blk_fwd || w->Tb.blk_bwd) {
+    int* pb = nullptr;
+    float* ck = nullptr;
+    if (dalloc(w, &pb, prog.size()) || dalloc(w, &ck, 2 * (size_t)T.horizon)) return cleanup(DP_ENOMEM);
+    CU(cudaMemcpyAsync(pb, prog.data(), sizeof(int32_t) * prog.size(), cudaMemcpyHostToDevice, w->stream));
+    CU(cudaStreamSynchronize(w->stream));
+    CU(launch_clock(w->Tf, ck, w->stream));
+    D.blk = pb;
+    D.clk = ck;
   }
   // warm start (enabled later by dp_set_warmstart), residual sums, harvest counter
   w->ws_capable = d->warmstart != 0;
@@ -813,21 +922,21 @@ dp_status dp_set_warmstart(dp_world* w, const float* W, float alpha) {
   if (!w->ws_capable) return fail(DP_EINVAL, "the world was created without warm-start support (desc.warmstart = 0)");
   if (!(alpha >= 0.f && alpha <= 1.f)) return fail(DP_EINVAL, "alpha must lie in [0, 1]");
   if (w->have_rollout) w->have_rollout = false;  // the recorded tape belongs to the other solver
-  w->Tf.ws_alpha = w->Tb.ws_alpha = alpha;
+  w->Tf.ws_alpha = w->Tb.ws_alpha = w->Ts.ws_alpha = alpha;
   if (!W) {
-    w->Tf.ws = w->Tb.ws = 0;
+    w->Tf.ws = w->Tb.ws = w->Ts.ws = 0;
     return DP_OK;
   }
   CU(cudaMemcpyAsync(w->ws_master, W, sizeof(float) * WsTC::PARAMS, cudaMemcpyDefault, w->stream));
   CU(launch_ws_prep(w->ws_master, w->ws_tc, w->ws_b, w->stream));
-  w->Tf.ws = w->Tb.ws = 1;
+  w->Tf.ws = w->Tb.ws = w->Ts.ws = 1;
   {  // an identically zero network is the damped start: the kernels skip its evaluation
     std::vector<float> hw(WsTC::PARAMS);
     CU(cudaMemcpyAsync(hw.data(), w->ws_master, sizeof(float) * WsTC::PARAMS, cudaMemcpyDeviceToHost, w->stream));
     CU(cudaStreamSynchronize(w->stream));
     int nz = 0;
     for (float x : hw) nz |= x != 0.f;
-    w->Tf.ws_net = w->Tb.ws_net = nz;
+    w->Tf.ws_net = w->Tb.ws_net = w->Ts.ws_net = nz;
   }
   return DP_OK;
 }
@@ -943,7 +1052,7 @@ dp_status dp_backward(dp_world* w, const float* dloss, float* dW, float* dstate0
   if (T.ext_ctrl)
     CU(ext_backward(w, T, D));
   else
-    CU(launch_backward(T, D, w->stream));
+    CU(launch_backward(T, w->Ts, D, w->stream));
   CU(launch_check_grads(w->B, w->Bp, w->nf, T.n_pfields, D.grad_state0, D.grad_prm, D.status, w->stream));
   if (dstate0) {
     CU(launch_state_out(w->B, w->Bp, w->nf, D.grad_state0, w->stage, w->stream));

@@ -1,0 +1,7 @@
+// Launchers of the four-warp reverse kernels for every other robot.
+#include "dp_blk_bwd.cuh"
+#include "dp_kernels.h"
+
+cudaError_t launch_backward_blk_dyn(const DevTopo& T, const DevTopo& Ts, const DevPtrs& D, cudaStream_t s) {
+  return launch_backward_blk_t<BlkDyn>(T, Ts, D, s);
+}

@@ -102,6 +102,18 @@ struct DevTopo {
   // MW_SLOT_B (owns side b)
   int16_t mw_slot[4][DPK_MAXSLOT];
   int16_t mw_nslot[4];
+  // four-warp step (dp_blk.cuh; laid out by plan_blocks): blk = 1 when the robot's solver blocks
+  // are scheduled and its records fit on chip; byte offsets in the program's region of shared
+  // memory (sm_prog): level table, bodies' item lists (first index per body, entries), live flags,
+  // streams; slots of each joint's first linear row, limit row and servo row, and of the contacts
+  int blk, blk_nops, blk_nlev, blk_single, blk_words, blk_bytes_total;
+  int blk_lev, blk_inc0, blk_inc, blk_live, blk_stream, blk_stream_len, sm_prog;
+  int blk_fwd, blk_bwd;  // 1: rollouts and steps / reverse passes of this world run on the four-warp step
+  int rec_rows;          // 1: the tape records hold the constraint rows (read by the one-warp reverse)
+  int rec_j, rec_c, rec_p;  // strides of the joints', contacts' and pairs' records
+  int sm_hbuf;           // controller buffers over the records (bfloat16 activations or delta planes, or ping-pong)
+  int cslot;
+  int16_t jslot[DPK_MAXJ], jlim[DPK_MAXJ], jmot[DPK_MAXJ];
   // activation/delta dump offsets (rows of [feature][T*Bp]); act l = input of layer l
   int dump_act[DPK_MAXL + 1], dump_del[DPK_MAXL + 1], dump_rows;
   // tape record of one (step, warp), lanes interleaved ([field][32]): byte offsets
@@ -117,6 +129,8 @@ struct DevTopo {
 // Global buffers a kernel works on.
 struct DevPtrs {
   const float* prm;      // [n_pfields][Bp]
+  const int* blk;        // block program (DevTopo.blk_words)
+  const float* clk;      // controller clock features of the steps 0 .. horizon - 1 [horizon][2]
   const float* Wt;       // controller, fp32 copies of the bf16 weights, each layer [in][out]
   const float* Wn;       // same, each layer [out][in]
   const float* bias;     // controller biases, per layer [out] (then skip bias)

@@ -94,6 +94,13 @@ __device__ __forceinline__ int warp_horizon(const DevPtrs& D, int i) {
 
 __device__ __forceinline__ float qz(const DevTopo& T, float x) { return T.ctrl_round ? bf16r(x) : x; }
 
+// The controller's clock at step t: sine and cosine of its phase, in double precision.
+__device__ __forceinline__ void clock_features(const DevTopo& T, int t, float& s, float& c) {
+  const double ph = 2.0 * 3.14159265358979323846 * (double)T.clock_hz * ((double)t * (double)T.dt);
+  s = (float)sin(ph);
+  c = (float)cos(ph);
+}
+
 // Controller input vector s(x^t), rounded to bfloat16 (unless the fp32 controller mode is
 // selected), into act0 (padded with zeros).
 template <class RV, class AV>
@@ -105,9 +112,10 @@ __device__ void controller_features(const DevTopo& T, const LaneT<RV>& L, const 
   if (T.features & 2)
     for (int m = 0; m < T.n_motors; ++m) act0[k++] = qz(T, S[T.sm_thd + T.motor_joint[m]]);
   if (T.features & 4) {
-    double ph = 2.0 * 3.14159265358979323846 * (double)T.clock_hz * ((double)t * (double)T.dt);
-    act0[k++] = qz(T, (float)sin(ph));
-    act0[k++] = qz(T, (float)cos(ph));
+    float s, c;
+    clock_features(T, t, s, c);
+    act0[k++] = qz(T, s);
+    act0[k++] = qz(T, c);
   }
   if (T.features & 8) {
     int b = T.imu_body;
@@ -125,12 +133,14 @@ __device__ void controller_features(const DevTopo& T, const LaneT<RV>& L, const 
 }
 
 // One dense layer on this lane: out[o] = b[o] + sum_i W[o][i] in[i], weights from the
-// [in][out_pad] copy (8 outputs per pass, broadcast float4 loads).
+// [in][out_pad] copy (8 outputs per pass, broadcast float4 loads; the passes o_first, o_first +
+// o_step, ... only, so that several warps may share a layer).
 template <class AVI, class AVO>
 __device__ void dense_fwd(const float* __restrict__ Wt, const float* __restrict__ bias, int ni, int no, const AVI& in,
-                          const AVO& out, bool hidden, bool accumulate, bool round) {
+                          const AVO& out, bool hidden, bool accumulate, bool round, int o_first = 0,
+                          int o_step = 8) {
   const int nop = (no + 7) & ~7;
-  for (int o0 = 0; o0 < no; o0 += 8) {
+  for (int o0 = o_first; o0 < no; o0 += o_step) {
     float acc[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) acc[k] = (o0 + k < no) ? __ldg(bias + o0 + k) : 0.f;
@@ -812,7 +822,8 @@ __device__ float step_forward(const DevTopo& T, const DevPtrs& D, const LaneT<RV
   assemble_rows(T, L, X, active_out);
   // the rows go to the tape, unless they were assembled in it (segment recompute)
   if constexpr (TAPE && !std::is_same<RV, GS>::value) {
-    for (int f = 0; f < T.nslots * RF_N; ++f) tp.rows[f * 32] = L.rows[f];
+    if (T.rec_rows)
+      for (int f = 0; f < T.nslots * RF_N; ++f) tp.rows[f * 32] = L.rows[f];
   }
   if (T.ws || D.harvest) warm_start<TAPE>(T, D, L, X, tp);
   if constexpr (Q::id == 0)

@@ -1,0 +1,9 @@
+// Launcher of the four-warp rollout kernel k_forward_blk for every other robot.
+#include "dp_blk_fwd.cuh"
+#include "dp_kernels.h"
+
+cudaError_t launch_forward_blk_dyn(const DevTopo& T, const DevPtrs& D, const float* x0, int t0, int nsteps, int rollout,
+                                   int record, cudaStream_t s) {
+  return record ? launch_forward_blk_t<true, BlkDyn>(T, D, x0, t0, nsteps, rollout, s)
+                : launch_forward_blk_t<false, BlkDyn>(T, D, x0, t0, nsteps, rollout, s);
+}

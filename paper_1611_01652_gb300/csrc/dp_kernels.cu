@@ -67,6 +67,16 @@ __global__ void k_prep_weights_tc(const __grid_constant__ DevTopo T, const float
   Wc[p] = __float2bfloat16_rn(v);
 }
 
+// The controller's clock features of the steps 0 .. horizon - 1.
+__global__ void k_clock(const __grid_constant__ DevTopo T, float* clk) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < T.horizon) clock_features(T, t, clk[2 * t], clk[2 * t + 1]);
+}
+cudaError_t launch_clock(const DevTopo& T, float* clk, cudaStream_t s) {
+  k_clock<<<(T.horizon + 127) / 128, 128, 0, s>>>(T, clk);
+  return cudaGetLastError();
+}
+
 // ------------------------------------------------------------------------------ layouts
 // [B][nb*18] (user) -> [nb*18][Bp]; padded instances copy instance B-1.
 __global__ void k_state_in(int B, int Bp, int nf, const float* __restrict__ src, float* dst) {

@@ -3,6 +3,9 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <cstdint>
+#include <vector>
+
 #include "dp_device.cuh"
 
 cudaError_t launch_prep_weights(const DevTopo& T, const float* W, float* Wt, float* Wn, float* bias, cudaStream_t s);
@@ -16,13 +19,22 @@ cudaError_t launch_param_in(int B, int Bp, int o, int n, const float* src, float
 cudaError_t launch_pad_scalar(int B, int Bp, const float* src, float* dst, cudaStream_t s);
 cudaError_t launch_forward(const DevTopo& T, const DevPtrs& D, const float* x0, int t0, int nsteps, int rollout,
                            int record, cudaStream_t s);
-cudaError_t launch_forward_mw_quadruped(const DevTopo& T, const DevPtrs& D, const float* x0, int t0, int nsteps,
-                                        int rollout, cudaStream_t s);
-cudaError_t launch_forward_mw_arm(const DevTopo& T, const DevPtrs& D, const float* x0, int t0, int nsteps,
-                                  int rollout, cudaStream_t s);
-cudaError_t launch_backward(const DevTopo& T, const DevPtrs& D, cudaStream_t s);
-cudaError_t launch_backward_mw_quadruped(const DevTopo& T, const DevPtrs& D, cudaStream_t s);
-cudaError_t launch_backward_mw_arm(const DevTopo& T, const DevPtrs& D, cudaStream_t s);
+cudaError_t launch_forward_blk(const DevTopo& T, const DevPtrs& D, const float* x0, int t0, int nsteps, int rollout,
+                               int record, cudaStream_t s);
+cudaError_t launch_forward_blk_arm(const DevTopo& T, const DevPtrs& D, const float* x0, int t0, int nsteps, int rollout,
+                                   int record, cudaStream_t s);
+cudaError_t launch_forward_blk_dyn(const DevTopo& T, const DevPtrs& D, const float* x0, int t0, int nsteps, int rollout,
+                                   int record, cudaStream_t s);
+// Schedule of the solver's blocks (dp_plan.cu): fills T's block fields and the program's words.
+bool plan_blocks(DevTopo& T, std::vector<int32_t>& blob);
+cudaError_t launch_clock(const DevTopo& T, float* clk, cudaStream_t s);
+cudaError_t launch_backward(const DevTopo& T, const DevTopo& Ts, const DevPtrs& D, cudaStream_t s);
+// Ts: forward layout of the segments' recompute
+cudaError_t launch_backward_blk(const DevTopo& T, const DevTopo& Ts, const DevPtrs& D, cudaStream_t s);
+cudaError_t launch_backward_blk_quad(const DevTopo& T, const DevTopo& Ts, const DevPtrs& D, cudaStream_t s);
+cudaError_t launch_backward_blk_arm(const DevTopo& T, const DevTopo& Ts, const DevPtrs& D, cudaStream_t s);
+cudaError_t launch_backward_blk_dyn(const DevTopo& T, const DevTopo& Ts, const DevPtrs& D, cudaStream_t s);
+cudaError_t launch_backward_ext_blk(const DevTopo& T, const DevPtrs& D, int t, cudaStream_t s);
 cudaError_t launch_backward_ext(const DevTopo& T, const DevPtrs& D, int t, cudaStream_t s);
 cudaError_t launch_dw(const float* del, const float* act, int M, int C, size_t N, float* partial, int splits,
                       size_t chunk, cudaStream_t s);

@@ -76,7 +76,7 @@ extern "C" dp_status dp_backward_noalloc(dp_world* w, const float* dloss, float*
   CUN(cudaMemcpyAsync(w->stage, dloss, sizeof(float) * w->B, cudaMemcpyDefault, w->stream));
   CUN(launch_pad_scalar(w->B, w->Bp, w->stage, D.dloss, w->stream));
   CUN(cudaMemsetAsync(D.grad_prm, 0, sizeof(float) * (size_t)T.n_pfields * w->Bp, w->stream));
-  CUN(launch_backward(T, D, w->stream));
+  CUN(launch_backward(T, w->Ts, D, w->stream));
   const size_t N = (size_t)T.horizon * w->Bp;
   size_t off = 0;
   for (int l = 0; l < nl; ++l) {

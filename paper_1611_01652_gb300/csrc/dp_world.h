@@ -17,6 +17,7 @@ struct ExtLayout {
 
 struct dp_world {
   DevTopo Tf, Tb;  // same topology; forward / backward shared-memory layouts
+  DevTopo Ts;      // forward layout of the four-warp reverse pass's segment recompute
   DevPtrs D;
   cudaStream_t stream = nullptr;
   int device = 0;  // the CUDA device current at creation (the world's buffers live there)
