@@ -1164,7 +1164,10 @@ __device__ __forceinline__ void blk_reverse_step(const DevTopo& T, const DevPtrs
     // wide controller: the output adjoint goes to the batched products; the features' adjoint comes
     // back into the next launch
     float* ubx = D.ub_ext + (size_t)i * 16;
-    for (int o = warp; o < 16; o += 4) ubx[o] = o < nout ? zb[o] : 0.f;
+    for (int o = warp; o < 16; o += 4) {
+      ubx[o] = o < nout ? zb[o] : 0.f;
+      if (o < nout) D.dump[(size_t)(T.dump_del[T.n_layers - 1] + o) * N + n] = zb[o];  // output layer's delta
+    }
     cta_sync();
   } else if (T.n_layers > 0) {
     GW act[DPK_MAXL + 1], del[DPK_MAXL + 1];
