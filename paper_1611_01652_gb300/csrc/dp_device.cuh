@@ -21,14 +21,6 @@
 // non-finite state or parameter adjoint in the last reverse pass
 #define DPK_ST_NAN_STATE 1
 #define DPK_ST_NAN_GRAD 2
-// rows per chunk of the multi-warp reverse sweep's hand-off ring (dp_mw.cuh)
-#ifndef DPK_MW_CH
-#define DPK_MW_CH 20
-#endif
-
-// Flags of DevTopo.mw_slot entries (the slot index takes the low 12 bits).
-#define MW_SLOT_A 0x1000
-#define MW_SLOT_B 0x2000
 
 // Warm-start group types (feature 15 of a group).
 enum { WSG_GROUND = 0, WSG_PAIR = 1, WSG_JOINT = 2, WSG_HINGE = 3 };
@@ -93,15 +85,6 @@ struct DevTopo {
   int sm_x0, sm_x, sm_xb, sm_vb, sm_iinv, sm_invm, sm_th, sm_thd, sm_ua, sm_wst, sm_wbr, sm_lam, sm_u;
   int sm_thb, sm_thdb, sm_uab, sm_wstb, sm_iinvb, sm_invmb, sm_rc, sm_sbar, sm_vw, sm_zb, sm_act[DPK_MAXL + 1], sm_rows,
       sm_total;
-  int sm_ring;  // multi-warp reverse sweep: two buffers of DPK_MW_CH (j, p_bar) pairs (shares sm_vw's region)
-  // multi-warp reverse pass: the warp (0..3) that owns each body's adjoint accumulators in the
-  // stages outside the sweeps, and the matching body / joint (by child body) masks per warp
-  int8_t mw_own[DPK_MAXB];
-  uint32_t mw_bmask[4], mw_jmask[4];
-  // per warp, the slots with a side it owns in slot order: slot | MW_SLOT_A (owns side a) |
-  // MW_SLOT_B (owns side b)
-  int16_t mw_slot[4][DPK_MAXSLOT];
-  int16_t mw_nslot[4];
   // four-warp step (dp_blk.cuh; laid out by plan_blocks): blk = 1 when the robot's solver blocks
   // are scheduled and its records fit on chip; byte offsets in the program's region of shared
   // memory (sm_prog): level table, bodies' item lists (first index per body, entries), live flags,

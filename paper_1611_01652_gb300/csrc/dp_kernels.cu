@@ -1,6 +1,6 @@
 // Kernels of libdphys around the rollout: weight staging, layout transposes, the gradient check
 // and the controller-gradient reduction. The persistent rollout and reverse-mode kernels are in
-// dp_steps.cuh, instantiated by dp_fwd.cu, dp_bwd.cu, dp_bwd_mw.cu and dp_bwd_ext.cu (one
+// dp_blk_fwd.cuh, dp_blk_bwd.cuh and dp_steps.cuh, instantiated by the dp_fwd*.cu and dp_bwd*.cu (one
 // translation unit per kernel family, so that they compile in parallel).
 #include <cuda_runtime.h>
 

@@ -1,5 +1,5 @@
-// Host-side launchers of the kernels in dp_kernels.cu, dp_fwd.cu, dp_fwd_mw.cu, dp_bwd.cu,
-// dp_bwd_mw.cu and dp_bwd_ext.cu (internal to libdphys).
+// Host-side launchers of the kernels in dp_kernels.cu, dp_fwd.cu, dp_bwd.cu,
+// dp_bwd_blk*.cu, dp_fwd_blk*.cu and dp_bwd_ext.cu (internal to libdphys).
 #pragma once
 #include <cuda_runtime.h>
 

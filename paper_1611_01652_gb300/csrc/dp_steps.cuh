@@ -1,12 +1,13 @@
-// The persistent rollout (forward) and reverse-mode kernel templates (one warp = 32 instances for
-// the whole horizon; four warps per 32 instances for the compiled topology's reverse pass).
+// The persistent rollout (forward) and reverse-mode kernel templates on one warp per group of 32
+// instances: robots too large for the four-warp step, worlds that keep rows in global memory, and
+// those that ask for one warp.
 #pragma once
 #include <cuda_runtime.h>
 
 #include <cstdlib>
 #include <type_traits>
 
-#include "dp_mw.cuh"
+#include "dp_static.cuh"
 
 extern __shared__ float g_smem[];
 
@@ -108,165 +109,6 @@ __global__ void __launch_bounds__(32, 1) k_forward(const __grid_constant__ DevTo
   for (int f = 0; f < 18 * T.nb; ++f) bad |= !isfinite(X[f]);
   if (rollout) D.loss[i] = loss;
   if (bad && i < B) D.status[i] |= DPK_ST_NAN_STATE;
-}
-
-// The one-warp warm start with the solver tape, out of line (it runs on one warp of k_forward_mw
-// and keeps the network's registers out of that kernel's budget).
-static __device__ __noinline__ void warm_start_call(const DevTopo& T, const DevPtrs& D, const LaneT<SL>& L, const SL& X,
-                                             const TapeStep& tp) {
-  warm_start<true>(T, D, L, X, tp);
-}
-
-// Persistent rollout of the compiled topology with the solver tape, on four warps per group of
-// 32 instances (one CTA per group; a lane is an instance in every warp, as in k_forward). The
-// stages outside the sweeps are split: warp w takes the joints and bodies it owns
-// (DevTopo.mw_jmask, mw_bmask: kinematics, servo targets, external impulses, the warm start's
-// application, integration), every fourth constraint slot of the row assembly and every fourth
-// field of the tape and checkpoint copies; warps 0 and 1 take one 16-row tile each of the
-// tensor-core controller's products. The sweeps, the controller's features and the loss run on
-// warp 0. Each quantity is computed by the same arithmetic in the same order as in k_forward,
-// so the two kernels give identical results. For rollouts (rollout != 0) without the harvest or
-// gait noise; with the wide controller (one step per launch) the step's controller output comes
-// from the batched products and the next step's input features go back to them, as in
-// k_forward.
-template <class Q>
-__global__ void __launch_bounds__(128, 1) k_forward_mw(const __grid_constant__ DevTopo T, const __grid_constant__ DevPtrs D,
-                                                       const float* __restrict__ x0, int t0, int nsteps, int rollout) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int i = blockIdx.x * 32 + lane;
-  const int Bp = T.Bp, B = T.B, nf = 18 * T.nb;
-  float* sm = g_smem + lane;
-  LaneT<SL> L{SL{sm}, GC{D.prm + i, Bp}, SL{sm + T.sm_rows * 32}, i};
-  const SL X{sm + T.sm_x * 32};
-  SL act[DPK_MAXL + 1];
-  for (int l = 0; l <= DPK_MAXL; ++l) act[l] = SL{sm + T.sm_act[l] * 32};
-  const uint32_t bm = T.mw_bmask[warp], jm = T.mw_jmask[warp];
-  const bool fresh = rollout == 1 || (rollout == 2 && t0 == 0);
-  const float* xs = fresh ? x0 : D.state;
-  for (int f = warp; f < nf; f += 4) X[f] = xs[(size_t)f * Bp + i];
-  for (int s = warp; s < T.nslots; s += 4) L.S[T.sm_lam + s] = fresh ? 0.f : D.lam_prev[(size_t)s * Bp + i];
-  if (warp == 0)
-    for (int k = 0; k < T.n_rec; ++k) L.S[T.sm_h + k] = fresh ? 0.f : D.hrec[(size_t)k * Bp + i];
-  mw_barrier();
-  float loss = (rollout == 2 && !fresh) ? D.loss[i] : 0.f;  // warp 0's copy is the one kept
-  if (fresh && T.loss_kind == 3) loss = -dot3(L.P.v3(T.o_loss_target), loss_point(T, L, X));
-  const int nrun = max(0, min(nsteps, warp_horizon(D, i) - t0));
-  const size_t N = (size_t)T.horizon * Bp;
-  for (int k = 0; k < nrun; ++k) {
-    const int t = t0 + k;
-    if (t % D.ckpt_every == 0) {
-      const size_t c = (size_t)(t / D.ckpt_every);
-      for (int f = warp; f < nf; f += 4) D.ckpt[(c * nf + f) * Bp + i] = X[f];
-      if (D.ckpt_lam)
-        for (int s = warp; s < T.nslots; s += 4) D.ckpt_lam[(c * T.nslots + s) * Bp + i] = L.S[T.sm_lam + s];
-      if (D.ckpt_h && warp == 0)
-        for (int q = 0; q < T.n_rec; ++q) D.ckpt_h[(c * T.n_rec + q) * Bp + i] = L.S[T.sm_h + q];
-    }
-    if (D.traj && i < B)
-      for (int f = warp; f < nf; f += 4) D.traj[((size_t)t * B + i) * nf + f] = X[f];
-    uint8_t* ao = (D.active && i < B) ? D.active + ((size_t)t * B + i) * T.nslots : nullptr;
-    // joint kinematics, controller, servo targets
-    hinge_kinematics(T, L, X, jm);
-    mw_barrier();
-    if (T.ext_ctrl) {
-      // wide controller: its output for this step was computed between launches
-      if (warp == 0) {
-        const float* ue = D.u_ext + ((size_t)t * Bp + i) * T.ext_nop;
-        for (int m = 0; m < T.widths[T.n_layers]; ++m) act[T.n_layers][m] = ue[m];
-      }
-      mw_barrier();
-      servo_targets(T, L, act[T.n_layers], jm);
-    } else if (T.n_layers > 0) {
-      float* dump_col = D.dump + (size_t)t * Bp + i;
-      if (warp == 0) {
-        controller_features(T, L, X, t, act[0]);
-        if (T.n_rec) {  // recurrent state h^t: the last inputs
-          const int base = T.widths[0] - T.n_rec;
-          for (int q = 0; q < T.n_rec; ++q) act[0][base + q] = qz(T, L.S[T.sm_h + q]);
-        }
-      }
-      mw_barrier();
-      if (T.mlp_tc) {
-        if (warp < 2) ctrl_tc_forward_q<Q, SL>(T, D, act, dump_col, warp, warp + 1);
-      } else if (warp == 0) {
-        controller_forward(T, D, act);
-      }
-      mw_barrier();
-      if (warp == 0) {
-        if (T.n_rec) {  // h^{t+1} = tanh of the last outputs
-          const int base = T.widths[T.n_layers] - T.n_rec;
-          for (int q = 0; q < T.n_rec; ++q) L.S[T.sm_h + q] = tanhf(act[T.n_layers][base + q]);
-        }
-        for (int l = 0; l <= T.n_layers; ++l) {
-          if (T.mlp_tc && l > 0 && l < T.n_layers) continue;  // hidden layers went straight to the dump
-          for (int q = 0; q < T.widths[l]; ++q) dump_col[(size_t)(T.dump_act[l] + q) * N] = act[l][q];
-        }
-      }
-      servo_targets(T, L, act[T.n_layers], jm);
-    } else {
-      servo_targets(T, L, act[0], jm);
-    }
-    // external impulses and world inverse inertias; the tape's pre-solve velocities
-    external_impulses(T, L, X, bm);
-    const TapeStep tp = tape_step(T, D, t);
-    for (int b = 0; b < T.nb; ++b)
-      if ((bm >> b) & 1u)
-#pragma unroll
-        for (int q = 0; q < 6; ++q) tp.vminus[(6 * b + q) * 32] = X[18 * b + 12 + q];
-    mw_barrier();
-    assemble_rows(T, L, X, ao, warp, 4);
-    mw_barrier();
-    for (int f = warp; f < T.nslots * RF_N; f += 4) tp.rows[f * 32] = L.rows[f];
-    if (T.ws) {
-      if (T.ws_net) {
-        // a learned network's start: the one-warp stage (features, the network on the tensor
-        // cores, projection, application to every body) on warp 0, as in k_forward
-        if (warp == 0) warm_start_call(T, D, L, X, tp);
-      } else {
-        warm_start_mw<true>(T, L, X, tp, warp, bm);
-      }
-    }
-    mw_barrier();
-    if (warp == 0) {
-      pgs_solve_static<Q, true>(T, L, X, tp);
-      if (D.resid) D.resid[i] += solve_residual(T, L, X);
-    }
-    mw_barrier();
-    integrate(T, X, bm);
-    mw_barrier();
-    if (warp == 0) {
-      const float w = loss_weight(T, t + 1, D.hz[i]);
-      if (w != 0.f) loss += w * loss_value(T, L, X);
-    }
-  }
-  if (D.traj && i < B)
-    for (int f = warp; f < nf; f += 4) D.traj[((size_t)(t0 + nrun) * B + i) * nf + f] = X[f];
-  if (T.ext_ctrl && t0 + nrun < T.horizon && warp == 0) {
-    // wide controller: input features of the next step, bf16 for the products, and the
-    // activation dump column for the weight gradient
-    const int tn = t0 + nrun;
-    hinge_kinematics(T, L, X);
-    controller_features(T, L, X, tn, act[0]);
-    __nv_bfloat16* sx = D.s_ext + (size_t)i * T.ext_k0p;
-    for (int q = 0; q < T.ext_k0p; ++q) {
-      const float v = q < T.widths[0] ? act[0][q] : 0.f;
-      sx[q] = __float2bfloat16_rn(v);
-      if (q < T.widths[0]) D.dump[(size_t)(T.dump_act[0] + q) * N + (size_t)tn * Bp + i] = v;
-    }
-  }
-  for (int s = warp; s < T.nslots; s += 4) D.lam_prev[(size_t)s * Bp + i] = L.S[T.sm_lam + s];
-  if (warp == 0)
-    for (int q = 0; q < T.n_rec; ++q) D.hrec[(size_t)q * Bp + i] = L.S[T.sm_h + q];
-  bool bad = false;
-  for (int f = warp; f < nf; f += 4) {
-    D.state[(size_t)f * Bp + i] = X[f];
-    bad |= !isfinite(X[f]);
-  }
-  if (warp == 0) {
-    bad |= !isfinite(loss);
-    D.loss[i] = loss;
-  }
-  if (bad && i < B) atomicOr(D.status + i, DPK_ST_NAN_STATE);
 }
 
 // ------------------------------------------------------------------------------ backward
@@ -391,28 +233,6 @@ __device__ void reverse_step_ctrl(const DevTopo& T, const DevPtrs& D, const BwdC
   hinge_reverse(T, V.Bl, C.XB);
 }
 
-// reverse_step_ctrl on the four warps of k_backward_mw (called by every warp; ends after a CTA
-// barrier): warp 0 takes the servo, feature and hinge-kinematics reverse, warps 0 and 1 one
-// 16-row tile each of the tensor-core controller's reverse products.
-template <class Q, class RV>
-__device__ void reverse_step_ctrl_mw(const DevTopo& T, const DevPtrs& D, const BwdCtx& C, const RevStep<RV>& V,
-                                     int warp) {
-  if (T.ext_ctrl || T.n_layers == 0 || !T.mlp_tc) {
-    if (warp == 0) reverse_step_ctrl<Q>(T, D, C, V);
-    mw_barrier();
-    return;
-  }
-  if (warp == 0) ctrl_reverse_head(T, C, V);
-  mw_barrier();
-  if (warp < 2) controller_reverse_tc<Q>(T, D, V.act, V.del, V.zb0, C.sbar, warp, warp + 1);
-  mw_barrier();
-  if (warp == 0) {
-    ctrl_reverse_tail(T, C, V);
-    hinge_reverse(T, V.Bl, C.XB);
-  }
-  mw_barrier();
-}
-
 // Last part of the reverse of step t (after the solver's reverse sweeps): warm-start
 // application, row assembly, external impulses, then the stages above, down to the adjoint of x_t.
 template <class Q, class RV>
@@ -496,87 +316,6 @@ __global__ void __launch_bounds__(32, 1) k_backward(const __grid_constant__ DevT
   for (int f = 0; f < nf; ++f) D.grad_state0[(size_t)f * Bp + i] = C.XB[f];
 }
 
-// Reverse mode through the last rollout on four warps per group of 32 instances (compiled
-// topology, whole tape recorded by the rollout). Every warp runs every phase of a step on its
-// share: bodies and joints split by DevTopo.mw_own (state copies, integrator, hinge kinematics,
-// servo targets, inverse inertias, warm-start and row-assembly reverse, external impulses),
-// the solver's reverse sweeps split into the chain and three helpers (dp_mw.cuh); warp 0 alone
-// runs the servo, controller, feature and hinge reverse. The warps meet at CTA barrier 1
-// between phases; every warp executes the same barrier sequence. Same arithmetic as
-// k_backward up to the order of the row-adjoint sums, which is fixed.
-// One step of the four-warp reverse pass (called by every warp of the CTA; ends after a CTA
-// barrier): step t from its tape record and x_t from the checkpoints, with x_{t+1} on chip in
-// C.X (copied there first from x_t1 when load_x1 is set); the state adjoint in C.XB is that of
-// x_{t+1} on entry and that of x_t on exit.
-// Step t's state checkpoint and controller activations of this CTA's 32 instances into L2, one
-// 128-byte line per field, spread over the CTA's threads (the reverse of step t + 1 runs
-// meanwhile).
-__device__ __forceinline__ void mw_prefetch_step_l2(const DevTopo& T, const DevPtrs& D, int t) {
-  const int Bp = T.Bp, nf = 18 * T.nb, base = blockIdx.x * 32;
-  const float* x = D.ckpt + (size_t)t * nf * Bp + base;
-  for (int f = threadIdx.x; f < nf; f += blockDim.x) prefetch_l2(x + (size_t)f * Bp);
-  // the controller's activation rows (its delta rows are written, not read, by the reverse)
-  if (T.n_layers == 0 || T.ext_ctrl) return;
-  const size_t N = (size_t)T.horizon * Bp;
-  const float* d = D.dump + (size_t)t * Bp + base;
-  for (int l = 0; l <= T.n_layers; ++l)
-    for (int r = threadIdx.x; r < T.widths[l]; r += blockDim.x) prefetch_l2(d + (size_t)(T.dump_act[l] + r) * N);
-}
-
-template <class Q>
-__device__ void mw_reverse_step(const DevTopo& T, const DevPtrs& D, const BwdCtx& C, int t, const float* x_t1,
-                                bool load_x1, int warp, uint32_t bm, uint32_t jm) {
-  const int i = C.i, Bp = T.Bp, nf = 18 * T.nb;
-  const size_t sbytes = (size_t)nf * Bp;
-  const RevStep<GSR> V = rev_views<GSR>(T, D, C, t, t);
-  const float* x_t = D.ckpt + (size_t)t * sbytes;
-  if (load_x1)
-    for (int f = warp; f < nf; f += 4) C.X[f] = x_t1[(size_t)f * Bp + i];
-  if (t > 0) {  // the next step to reverse: its tape record, state checkpoint and controller columns
-    if (warp == 0) prefetch_record_l2(T, tape_step(T, D, t - 1).rec);
-    mw_prefetch_step_l2(T, D, t - 1);
-  }
-  if (T.grad_decay != 1.f) {  // section 3.2: the adjoint from later steps shrinks by alpha per step
-    for (int f = warp; f < nf; f += 4) C.XB[f] *= T.grad_decay;
-    if (warp == 0)
-      for (int k = 0; k < T.n_rec; ++k) C.S[T.sm_hb + k] *= T.grad_decay;  // and so does h's
-  }
-  mw_barrier();
-  // loss term (by the loss body's owner) and integrator, x_{t+1} on chip
-  if (T.mw_own[T.loss_body] == warp) loss_reverse(T, V.Bl, C.X, C.XB, loss_weight(T, t + 1, D.hz[i]) * C.dl);
-  integrate_reverse(T, GC{x_t + i, Bp}, C.X, C.XB, C.VB, bm);
-  mw_barrier();
-  // x_t on chip; accumulators zeroed
-  for (int f = warp; f < nf; f += 4) C.X[f] = x_t[(size_t)f * Bp + i];
-  for (int j = 0; j < T.nj; ++j) {
-    if (!((jm >> j) & 1u)) continue;
-    C.S[T.sm_thb + j] = 0.f; C.S[T.sm_thdb + j] = 0.f; C.S[T.sm_wstb + j] = 0.f;
-    C.S.s3(T.sm_uab + 3 * j, f3(0.f, 0.f, 0.f));
-  }
-  for (int b = 0; b < T.nb; ++b) {
-    if (!((bm >> b) & 1u)) continue;
-    C.S[T.sm_invmb + b] = 0.f;
-    for (int q = 0; q < 9; ++q) C.S[T.sm_iinvb + 9 * b + q] = 0.f;
-  }
-  for (int q = warp; q < T.nslots * RC_N; q += 4) C.RC[q] = 0.f;
-  mw_barrier();
-  // per-step forward quantities of x_t, recomputed bit-identically
-  hinge_kinematics(T, V.L, C.X, jm);
-  servo_targets(T, V.L, V.act[T.n_layers > 0 ? T.n_layers : 0], jm);
-  inverse_inertia(T, V.L, C.X, bm);
-  mw_barrier();
-  pgs_reverse_mw<Q>(T, V.L, V.tp, warp);
-  if (T.ws) {
-    ws_apply_reverse_own(T, V.L, C.VB, C.RC, V.tp, warp);
-    mw_barrier();
-  }
-  rows_reverse_own(T, V.Bl, C.XB, C.VB, C.RC, warp);
-  mw_barrier();
-  external_reverse(T, V.Bl, C.XB, C.VB, bm);
-  mw_barrier();
-  reverse_step_ctrl_mw<Q>(T, D, C, V, warp);
-}
-
 // Initial term -a.q(x_0) of the displacement loss (warp 0).
 __device__ __forceinline__ void loss_initial_reverse(const DevTopo& T, const DevPtrs& D, const BwdCtx& C) {
   copy_state_to_smem(T, D.ckpt, C.i, C.X);
@@ -588,80 +327,6 @@ __device__ __forceinline__ void loss_initial_reverse(const DevTopo& T, const Dev
   add_outer(C.XB, 18 * b + 3, gq, c);
   C.G.red3(T.o_loss_point, mtv(R, gq));
   C.G.red3(T.o_loss_target, -C.dl * (C.X.v3(18 * b) + mv(R, c)));
-}
-
-// Reverse mode through the last rollout on four warps per group of 32 instances (compiled
-// topology, whole tape): every step by mw_reverse_step, last first.
-template <class Q>
-__global__ void __launch_bounds__(128, 1) k_backward_mw(const __grid_constant__ DevTopo T, const __grid_constant__ DevPtrs D) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int i = blockIdx.x * 32 + lane;
-  const int Bp = T.Bp;
-  const int nf = 18 * T.nb;
-  float* sm = g_smem + lane;
-  BwdCtx C{SL{sm}, SL{sm + T.sm_x * 32}, SL{sm + T.sm_xb * 32}, SL{sm + T.sm_vb * 32}, SL{sm + T.sm_rc * 32},
-           SL{sm + T.sm_sbar * 32}, GC{D.prm + i, Bp}, GL{D.grad_prm + i, Bp}, i, D.dloss[i]};
-  const uint32_t bm = T.mw_bmask[warp], jm = T.mw_jmask[warp];
-  for (int f = warp; f < nf; f += 4) C.XB[f] = 0.f;
-  if (warp == 0)
-    for (int k = 0; k < T.n_rec; ++k) C.S[T.sm_hb + k] = 0.f;
-  const size_t sbytes = (size_t)nf * Bp;
-  const int Tw = warp_horizon(D, i);  // the same for the CTA's four warps (same instances)
-  for (int t = Tw - 1; t >= 0; --t) {
-    // x_{t+1} is on chip from the previous (later) step, except for the first one reversed
-    const float* x_t1 = t + 1 < Tw ? D.ckpt + (size_t)(t + 1) * sbytes : D.state;
-    mw_reverse_step<Q>(T, D, C, t, x_t1, t == Tw - 1, warp, bm, jm);
-  }
-  if (warp != 0) return;
-  if (T.loss_kind == 3) loss_initial_reverse(T, D, C);
-  for (int f = 0; f < nf; ++f) D.grad_state0[(size_t)f * Bp + i] = C.XB[f];
-}
-
-// The wide controller's per-step reverse launches (k_backward_ext) on four warps per group of 32
-// instances (compiled topology, whole tape): the feature adjoint of x_{t+1} (joint kinematics split
-// by joint owner, the features' and hinges' reverse on warp 0), then mw_reverse_step of step t.
-template <class Q>
-__global__ void __launch_bounds__(128, 1) k_backward_ext_mw(const __grid_constant__ DevTopo T,
-                                                           const __grid_constant__ DevPtrs D, int t) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int i = blockIdx.x * 32 + lane;
-  const int Bp = T.Bp;
-  const int nf = 18 * T.nb;
-  float* sm = g_smem + lane;
-  BwdCtx C{SL{sm}, SL{sm + T.sm_x * 32}, SL{sm + T.sm_xb * 32}, SL{sm + T.sm_vb * 32}, SL{sm + T.sm_rc * 32},
-           SL{sm + T.sm_sbar * 32}, GC{D.prm + i, Bp}, GL{D.grad_prm + i, Bp}, i, D.dloss[i]};
-  const uint32_t bm = T.mw_bmask[warp], jm = T.mw_jmask[warp];
-  const int Tw = warp_horizon(D, i);  // the same for the CTA's four warps
-  if (t >= Tw) return;                // this group's rollout ended before step t
-  const size_t sbytes = (size_t)nf * Bp;
-  for (int f = warp; f < nf; f += 4) C.XB[f] = D.grad_state0[(size_t)f * Bp + i];
-  const int tn = t + 1;
-  if (tn < Tw) {  // adjoint of the features of x_{t+1}
-    const float* xs = D.ckpt + (size_t)tn * sbytes;
-    for (int f = warp; f < nf; f += 4) C.X[f] = xs[(size_t)f * Bp + i];
-    mw_barrier();
-    LaneT<GSR> L{C.S, C.P, GSR{D.ckpt}, i};
-    BLaneT<GSR> Bl{L, C.X, C.G, GC{D.ckpt, 32}};
-    hinge_kinematics(T, L, C.X, jm);
-    for (int j = 0; j < T.nj; ++j) {
-      if (!((jm >> j) & 1u)) continue;
-      C.S[T.sm_thb + j] = 0.f; C.S[T.sm_thdb + j] = 0.f; C.S[T.sm_wstb + j] = 0.f;
-      C.S.s3(T.sm_uab + 3 * j, f3(0.f, 0.f, 0.f));
-    }
-    mw_barrier();
-    if (warp == 0) {
-      features_reverse(T, Bl, C.XB, GC{D.sbar_ext + (size_t)i * T.ext_k0p, 1});
-      hinge_reverse(T, Bl, C.XB);
-    }
-    mw_barrier();
-  }
-  if (t >= 0) {
-    mw_reverse_step<Q>(T, D, C, t, D.state, tn >= Tw, warp, bm, jm);
-  } else {
-    if (warp == 0 && T.loss_kind == 3) loss_initial_reverse(T, D, C);
-    mw_barrier();
-  }
-  for (int f = warp; f < nf; f += 4) D.grad_state0[(size_t)f * Bp + i] = C.XB[f];
 }
 
 // Wide controller, reverse mode one step per launch. Launch t adds the adjoint of the input
