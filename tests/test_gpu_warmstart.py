@@ -298,3 +298,25 @@ def test_learned_warm_start_training_and_acceptance_gate():
     print("acceptance gate", rep)
     assert not any(c["accepted"] for c in rep["candidates"] if c["name"] == "bad"), rep
     assert rep["accepted"] is not None and rep["accepted"][1] < 20, rep
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 256, 257, 8191, 70001])
+def test_weight_gradient_sums_over_splits(n):
+    """The gradient of n rows is the mean of the gradients of its rows: one launch over n rows against
+    launches over pieces of other lengths (around a tile of 32 columns and a split of 256). fp32 sums of
+    at most n terms in two orders, formed in pieces of 256: 1e-5 of the gradient's norm."""
+    g = torch.Generator().manual_seed(n)
+    rows = torch.randn(n, Bd.WS_ROW, generator=g).cuda()
+    W = (0.2 * torch.randn(Bd.WS_PARAMS, generator=g)).cuda()
+
+    def grad(r):
+        loss, dW = torch.zeros(1, device="cuda"), torch.zeros_like(W)
+        Bd.ws_loss_grad(W, r.contiguous(), loss, dW, Bd.ws_workspace(len(r)))
+        return loss.double() * len(r), dW.double() * len(r)
+
+    L, d = grad(rows)
+    step = max(1, min(n, 10007) * 3 // 5)
+    parts = [grad(rows[k:k + step]) for k in range(0, n, step)]
+    Ls, ds = sum(p[0] for p in parts), sum(p[1] for p in parts)
+    assert abs(L - Ls) <= 1e-5 * abs(Ls)
+    assert (d - ds).norm() <= 1e-5 * ds.norm()
