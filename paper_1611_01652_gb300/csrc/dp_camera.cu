@@ -371,13 +371,45 @@ __global__ void __launch_bounds__(kThreads, DPK_RENDER_BLOCKS) k_render(const __
   }
 }
 
+// Adds six consecutive values (two texels) at D + i, which starts at a multiple of four floats below
+// n: with 16-byte reductions over the aligned window of eight or twelve floats around them, the rest
+// of the window zeros; one by one where the window would leave the buffer (or it is not aligned).
+__device__ __forceinline__ void red_texels(float* D, size_t i, size_t n, bool vec, const float (&w)[6]) {
+  const size_t b = i & ~(size_t)3;
+  const int o = (int)(i - b);
+  if (!vec || b + 12 > n) {
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+      if (w[k] != 0.f) atomicAdd(D + i + k, w[k]);
+    return;
+  }
+  float v[12];
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    v[k] = 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (k - q >= 0 && k - q < 6 && o == q) v[k] = w[k - q];
+  }
+  atomicAdd(reinterpret_cast<float4*>(D + b), make_float4(v[0], v[1], v[2], v[3]));
+  atomicAdd(reinterpret_cast<float4*>(D + b + 4), make_float4(v[4], v[5], v[6], v[7]));
+  if (o == 3) atomicAdd(reinterpret_cast<float4*>(D + b + 8), make_float4(v[8], v[9], v[10], v[11]));
+}
+
 // Reverse mode: dstate[inst][body][0..11] (position, rotation entries) += the pixel's share of
 // d(sum dimage * image); dtex (optional) += the texel shares. A warp whose 32 pixels belong to one
 // instance sums its state shares per body with shuffles before one atomic per value.
+// Bound: the additions into the textures, which all instances share. One atomic per pixel, texel and
+// channel (12 a pixel) took 2998 us for 512 frames of 288 x 96 (six objects), the frames themselves
+// 240 us. A texture is usually stretched over several pixels, so the neighbouring pixels of a warp that
+// sample the same four texels are summed first (shuffles over each run of lanes), and the run's first
+// lane adds a texture row's two texels with 16-byte reductions: frames and gradients 3329 -> 890 us.
 __global__ void __launch_bounds__(kThreads) k_render_bwd(const __grid_constant__ CamArgs A, const float* __restrict__ state,
                                                          const float* __restrict__ tex, const float* __restrict__ dimage,
-                                                         float* __restrict__ dstate, float* __restrict__ dtex) {
+                                                         float* __restrict__ dstate, float* __restrict__ dtex,
+                                                         size_t ntex) {
   __shared__ BoxFrame sf[kMaxObj];
+  const bool vec = (reinterpret_cast<size_t>(dtex) & 15) == 0;
   int inst0s, pix0;
   const bool staged = stage_frames(A, state, sf, inst0s, pix0);
   const int npixi = A.W * A.H;
@@ -391,6 +423,12 @@ __global__ void __launch_bounds__(kThreads) k_render_bwd(const __grid_constant__
 #pragma unroll
   for (int k = 0; k < 12; ++k) g[k] = 0.f;
   int gb = -1;  // body receiving g (-1: none)
+  // texel shares: channels of (x0, x1) of row y0, then of row y1; the texels (y0, x0) of texture kt, and
+  // which of x1 = x0 + 1, y1 = y0 + 1 hold (at an edge both are clamped to one texel)
+  float tg[12];
+#pragma unroll
+  for (int k = 0; k < 12; ++k) tg[k] = 0.f;
+  int kt = -1, ky0 = 0, kx0 = 0, kdx = 0, kdy = 0;
   if (live) {
     int i, j;
     pixel_ij(A, pixr, i, j);
@@ -408,14 +446,18 @@ __global__ void __launch_bounds__(kThreads) k_render_bwd(const __grid_constant__
         const float t00 = __ldg(T + i00), t01 = __ldg(T + i01), t10 = __ldg(T + i10), t11 = __ldg(T + i11);
         dfx += gi * ((1.f - S.fy) * (t01 - t00) + S.fy * (t11 - t10));
         dfy += gi * (((1.f - S.fx) * t10 + S.fx * t11) - ((1.f - S.fx) * t00 + S.fx * t01));
-        if (dtex && gi != 0.f) {
-          float* D = dtex + (size_t)A.tex[h.obj] * A.th * A.tw * 3;
-          atomicAdd(D + i00, gi * (1.f - S.fx) * (1.f - S.fy));
-          atomicAdd(D + i01, gi * S.fx * (1.f - S.fy));
-          atomicAdd(D + i10, gi * (1.f - S.fx) * S.fy);
-          atomicAdd(D + i11, gi * S.fx * S.fy);
+        if (gi != 0.f) {
+          tg[ch] = gi * (1.f - S.fx) * (1.f - S.fy);
+          tg[3 + ch] = gi * S.fx * (1.f - S.fy);
+          tg[6 + ch] = gi * (1.f - S.fx) * S.fy;
+          tg[9 + ch] = gi * S.fx * S.fy;
+          kt = A.tex[h.obj];
         }
       }
+      ky0 = S.y0;
+      kx0 = S.x0;
+      kdx = S.x1 - S.x0;
+      kdy = S.y1 - S.y0;
       const int b = A.body[h.obj];
       if (b >= 0) {
         BoxFrame F;
@@ -492,6 +534,38 @@ __global__ void __launch_bounds__(kThreads) k_render_bwd(const __grid_constant__
     }
   }
   const unsigned full = 0xffffffffu;
+  if (dtex && __any_sync(full, kt >= 0)) {
+    const int lane = threadIdx.x & 31;
+    const int kxy = kx0 * 2 + kdx, kyy = ky0 * 2 + kdy;
+    // (every lane takes part in the three shuffles)
+    const int ut = __shfl_up_sync(full, kt, 1), ux = __shfl_up_sync(full, kxy, 1), uy = __shfl_up_sync(full, kyy, 1);
+    const bool head = lane == 0 || kt != ut || kxy != ux || kyy != uy;
+    const unsigned heads = __ballot_sync(full, head);
+    const unsigned above = lane == 31 ? 0u : heads >> (lane + 1);
+    const int last = above ? lane + __ffs(above) - 1 : 31;  // last lane of this lane's run
+    const int longest = __reduce_max_sync(full, (unsigned)(last - lane));
+    for (int off = 1; off <= longest; off <<= 1) {
+#pragma unroll
+      for (int k = 0; k < 12; ++k) {
+        const float v = __shfl_down_sync(full, tg[k], off);
+        if (lane + off <= last) tg[k] += v;
+      }
+    }
+    if (head && kt >= 0) {
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const size_t i0 = (((size_t)kt * A.th + ky0 + r * kdy) * A.tw + kx0) * 3;
+        float w[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) w[k] = tg[6 * r + k];
+        if (kdx == 0) {  // both texels are the same one
+#pragma unroll
+          for (int k = 0; k < 3; ++k) { w[k] += w[3 + k]; w[3 + k] = 0.f; }
+        }
+        red_texels(dtex, i0, ntex, vec && kdx != 0, w);
+      }
+    }
+  }
   const int inst0 = __shfl_sync(full, inst, 0);
   if (__all_sync(full, inst == inst0) && inst0 >= 0) {
     for (int b = 0; b < A.nb; ++b) {
@@ -593,7 +667,8 @@ dp_status dp_render_backward(const dp_camera* cam, const dp_scene* scene, int32_
     e = cudaMemsetAsync(dtextures, 0, sizeof(float) * (size_t)scene->n_tex * A.th * A.tw * 3, s);
   const size_t n = (size_t)A.W * A.H * A.B;
   if (e == cudaSuccess && n > 0) {
-    k_render_bwd<<<(unsigned)((n + kChunk - 1) / kChunk), kThreads, 0, s>>>(A, state, textures, dimage, dstate, dtextures);
+    k_render_bwd<<<(unsigned)((n + kChunk - 1) / kChunk), kThreads, 0, s>>>(A, state, textures, dimage, dstate, dtextures,
+                                                                                 (size_t)scene->n_tex * A.th * A.tw * 3);
     e = cudaGetLastError();
   }
   if (e != cudaSuccess) { g_cam_err = cudaGetErrorString(e); return DP_ECUDA; }

@@ -119,3 +119,26 @@ def test_screen_rectangles_change_nothing(monkeypatch, mixed):
     assert np.array_equal(ia, ib) and np.array_equal(ha, hb)
     assert np.abs(sa - sb).max() <= 1e-5 * max(1.0, np.abs(sb).max())
     assert np.abs(ta - tb).max() <= 1e-5 * max(1.0, np.abs(tb).max())
+
+
+@pytest.mark.parametrize("tex_size,W,H", [(1, 32, 16), (3, 144, 48), (5, 288, 96), (64, 64, 38)])
+def test_texture_gradient_at_any_alignment(tex_size, W, H):
+    """The texel gradient with 16-byte reductions (aligned buffer) and one value at a time (a buffer that
+    starts one float later), down to textures of one texel and of sizes that are no multiple of four
+    floats; nothing is written around the buffer. Sums of at most B W H terms in two orders: 1e-4."""
+    cs = WL.camera_scene(B=6, W=W, H=H, tex_size=tex_size, mixed=True)
+    rig = CameraRig(cs)
+    st = torch.tensor(np.asarray(cs.states, np.float32), device="cuda")
+    tex = torch.tensor(np.asarray(cs.textures, np.float32), device="cuda")
+    dimg = torch.randn(6, H, W, 3, device="cuda", generator=torch.Generator("cuda").manual_seed(3))
+    out = []
+    for shift in (0, 1):
+        buf = torch.full((tex.numel() + 16,), 7.0, device="cuda")
+        dtex = buf[shift:shift + tex.numel()].view(tex.shape)
+        ds = torch.zeros_like(st)
+        rig.render_backward(st, tex, dimg, ds, dtex)
+        torch.cuda.synchronize()
+        assert (buf[:shift] == 7.0).all() and (buf[shift + tex.numel():] == 7.0).all()
+        out.append((dtex.double().clone(), ds.double()))
+    for a, b in zip(*out):
+        assert torch.isfinite(a).all() and (a - b).norm() <= 1e-4 * b.norm()
