@@ -278,7 +278,9 @@ int plan_smem_blk_bwd(DevTopo& T) {
   const int keep = o;
   T.sm_x = take(18 * T.nb);
   T.sm_vb = take(6 * T.nb);
-  T.sm_vw = take(6 * T.nb);
+  T.sm_vw = take(2 * 6 * T.nb);                  // two sweeps
+  T.sm_rlam = take(3 * T.nslots);                // impulses after three sweeps
+  T.sm_rbr = take(2 * ((T.nslots + 3) / 4));     // clamp branches (bytes) of two
   T.sm_iinv = take(6 * T.nb);
   T.sm_invm = take(T.nb);
   T.sm_iinvb = take(6 * T.nb);

@@ -437,22 +437,28 @@ static __device__ __noinline__ RowRec blk_row(const DevTopo& T, const SL S, int 
 }
 
 // ------------------------------------------------------------------------------ forward sweeps
-// One projected row update: the new impulse, its tape entries, and the change dl.
-template <bool TAPE>
-__device__ __forceinline__ float row_solve(const DevTopo& T, const SL& S, const TapeStep& tp, int it, int slot, float Jv,
-                                           float meff, float bias, float lo, float hi, float& lam) {
+// One projected row update: lam becomes the new impulse, br its clamp branch (0 inside, 1 lower
+// bound, 2 upper bound); returns the change. A row without bounds (EQ) never clamps.
+template <bool EQ>
+__device__ __forceinline__ float row_solve(const DevTopo& T, float Jv, float meff, float bias, float lo, float hi, float& lam,
+                                           int& br) {
   const float l0 = lam;
   const float pre = fmaf(-meff, fmaf(T.gamma, l0, __fadd_rn(Jv, bias)), l0);
-  const int br = pre < lo ? 1 : (pre > hi ? 2 : 0);
-  const float ln = br == 1 ? lo : (br == 2 ? hi : pre);
-  lam = ln;
-  S[T.sm_lam + slot] = ln;
+  br = EQ ? 0 : (pre < lo ? 1 : (pre > hi ? 2 : 0));
+  lam = br == 1 ? lo : (br == 2 ? hi : pre);
+  return lam - l0;
+}
+// A row's new impulse on chip and, with TAPE, to the tape with its clamp branch (only the one-warp
+// reverse reads the branch of a row without bounds).
+template <bool TAPE, bool EQ>
+__device__ __forceinline__ void row_store(const DevTopo& T, const SL& S, const TapeStep& tp, int it, int slot, float lam,
+                                          int br) {
+  S[T.sm_lam + slot] = lam;
   if (TAPE) {
     const int o = (it * T.nslots + slot) * 32;
-    tp.lam[o] = ln;
-    tp.br[o] = (uint8_t)br;
+    tp.lam[o] = lam;
+    if (!EQ || T.rec_rows) tp.br[o] = (uint8_t)br;
   }
-  return ln - l0;
 }
 template <int AX>
 __device__ __forceinline__ float& axis_of(float3& v) {
@@ -475,41 +481,53 @@ __device__ __forceinline__ void lin_sub(float& v, float dl, float im) {
 }
 
 // The blocks' bodies: va, wa, vb, wb are the velocities of the parent and the child (zeros for the
-// world).
-template <bool TAPE, bool SEQ>
+// world). Everything a block reads from the record is loaded before its first row and every result
+// is stored after its last one: a store between the rows would keep the loads of the next row behind
+// it, and each row would wait for shared memory (some 30 cycles) besides its own chain of products.
+template <bool TAPE, bool SEQ, bool FULL>
 __device__ __forceinline__ void joint_rows(const DevTopo& T, const SL& S, const TapeStep& tp, int it, const BlkOp& op,
                                            const SL& R, float ima, float imb, float3& va, float3& wa, float3& vb,
                                            float3& wb) {
-  const float INF = __int_as_float(0x7f800000);
-  const int mask = op.mask(), s0 = op.slot();
+  const int mask = FULL ? 31 : op.mask(), s0 = op.slot();
   const float3 ra = R.v3(JF_RA), rb = R.v3(JF_RB);
+  float lam[5], me[5], bi[5];
+  float3 IA[5], IB[5], t[2];
+#pragma unroll
+  for (int k = 0; k < 5; ++k)
+    if (mask >> k & 1) {
+      lam[k] = S[T.sm_lam + s0 + k];
+      me[k] = R[JF_ME + k];
+      bi[k] = R[JF_BI + k];
+      IA[k] = R.v3(k < 3 ? JF_IAL + 3 * k : JF_IAT + 3 * (k - 3));
+      IB[k] = R.v3(k < 3 ? JF_IBL + 3 * k : JF_IBT + 3 * (k - 3));
+      if (k >= 3) t[k - 3] = R.v3(JF_T + 3 * (k - 3));
+    }
+  int br;
   auto lin = [&](auto KI) {
     constexpr int k = decltype(KI)::value;
     if (!(mask >> k & 1)) return;
     const float3 angA = cross_axis<k>(ra), angB = -cross_axis<k>(rb);
-    float lam = S[T.sm_lam + s0 + k];
     const float Jv = jv_lin<SEQ>(axis_of<k>(va), angA, wa) + (dotx(angB, wb) - axis_of<k>(vb));
-    const float dl = row_solve<TAPE>(T, S, tp, it, s0 + k, Jv, R[JF_ME + k], R[JF_BI + k], -INF, INF, lam);
-    const float3 IA = R.v3(JF_IAL + 3 * k), IB = R.v3(JF_IBL + 3 * k);
+    const float dl = row_solve<true>(T, Jv, me[k], bi[k], 0.f, 0.f, lam[k], br);
     lin_add<SEQ>(axis_of<k>(va), dl, ima);
-    wa = axpy3(dl, IA, wa);
+    wa = axpy3(dl, IA[k], wa);
     lin_sub<SEQ>(axis_of<k>(vb), dl, imb);
-    wb = axpy3(dl, IB, wb);
+    wb = axpy3(dl, IB[k], wb);
   };
   lin(std::integral_constant<int, 0>{});
   lin(std::integral_constant<int, 1>{});
   lin(std::integral_constant<int, 2>{});
 #pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    if (!(mask >> (3 + k) & 1)) continue;
-    const float3 t = R.v3(JF_T + 3 * k), angB = -t;
-    float lam = S[T.sm_lam + s0 + 3 + k];
-    const float Jv = dotx(t, wa) + dotx(angB, wb);
-    const float dl = row_solve<TAPE>(T, S, tp, it, s0 + 3 + k, Jv, R[JF_ME + 3 + k], R[JF_BI + 3 + k], -INF, INF, lam);
-    const float3 IA = R.v3(JF_IAT + 3 * k), IB = R.v3(JF_IBT + 3 * k);
-    wa = axpy3(dl, IA, wa);
-    wb = axpy3(dl, IB, wb);
+  for (int k = 3; k < 5; ++k) {
+    if (!(mask >> k & 1)) continue;
+    const float Jv = dotx(t[k - 3], wa) + dotx(-t[k - 3], wb);
+    const float dl = row_solve<true>(T, Jv, me[k], bi[k], 0.f, 0.f, lam[k], br);
+    wa = axpy3(dl, IA[k], wa);
+    wb = axpy3(dl, IB[k], wb);
   }
+#pragma unroll
+  for (int k = 0; k < 5; ++k)
+    if (mask >> k & 1) row_store<TAPE, true>(T, S, tp, it, s0 + k, lam[k], 0);
 }
 template <bool TAPE>
 __device__ __forceinline__ void hinge_row(const DevTopo& T, const SL& S, const TapeStep& tp, int it, const BlkOp& op,
@@ -520,43 +538,51 @@ __device__ __forceinline__ void hinge_row(const DevTopo& T, const SL& S, const T
   const int j = op.idx();
   const float3 angB = sg * S.v3(T.sm_ua + 3 * j), angA = -angB;
   float lam = S[T.sm_lam + s];
-  const float Jv = dotx(angA, wa) + dotx(angB, wb);
+  const float me = R[JF_ME + m], bi = R[JF_BI + m];
   const float hi = lim ? __int_as_float(0x7f800000) : R[JF_BND], lo = lim ? 0.f : -hi;
-  const float dl = row_solve<TAPE>(T, S, tp, it, s, Jv, R[JF_ME + m], R[JF_BI + m], lo, hi, lam);
   const float3 IA = -(sg * R.v3(JF_IAU)), IB = sg * R.v3(JF_IBU);
+  const float Jv = dotx(angA, wa) + dotx(angB, wb);
+  int br;
+  const float dl = row_solve<false>(T, Jv, me, bi, lo, hi, lam, br);
   wa = axpy3(dl, IA, wa);
   wb = axpy3(dl, IB, wb);
+  row_store<TAPE, false>(T, S, tp, it, s, lam, br);
 }
-template <bool TAPE, bool SEQ>
+template <bool TAPE, bool SEQ, bool FULL>
 __device__ __forceinline__ void contact_rows(const DevTopo& T, const SL& S, const TapeStep& tp, int it, const BlkOp& op,
                                              const SL& R, float ima, float3& va, float3& wa) {
-  const int mask = op.mask(), s0 = op.slot();
+  const int mask = FULL ? 7 : op.mask(), s0 = op.slot();
   const float3 ra = R.v3(CF_RA);
-  float ln = S[T.sm_lam + s0];
-  auto row = [&](auto MI, auto AI, float lo, float hi, float bias, float& lam) {
+  float lam[3], me[3];
+  float3 IA[3];
+  int br[3];
+  lam[0] = S[T.sm_lam + s0];  // (the friction rows' bound needs it in any block)
+#pragma unroll
+  for (int m = 0; m < 3; ++m)
+    if (mask >> m & 1) {
+      if (m > 0) lam[m] = S[T.sm_lam + s0 + m];
+      me[m] = R[CF_ME + m];
+      IA[m] = R.v3(CF_I + 3 * m);
+    }
+  const float bias = R[CF_BI], mu = R[CF_MU];
+  auto row = [&](auto MI, auto AI, float lo, float hi, float b) {
     constexpr int m = decltype(MI)::value, ax = decltype(AI)::value;
     const float3 angA = cross_axis<ax>(ra);
     const float Jv = jv_lin<SEQ>(axis_of<ax>(va), angA, wa);
-    const float dl = row_solve<TAPE>(T, S, tp, it, s0 + m, Jv, R[CF_ME + m], bias, lo, hi, lam);
-    const float3 IA = R.v3(CF_I + 3 * m);
+    const float dl = row_solve<false>(T, Jv, me[m], b, lo, hi, lam[m], br[m]);
     lin_add<SEQ>(axis_of<ax>(va), dl, ima);
-    wa = axpy3(dl, IA, wa);
+    wa = axpy3(dl, IA[m], wa);
   };
   using I0 = std::integral_constant<int, 0>;
   using I1 = std::integral_constant<int, 1>;
   using I2 = std::integral_constant<int, 2>;
-  if (mask & 1) row(I0{}, I2{}, 0.f, __int_as_float(0x7f800000), R[CF_BI], ln);
-  const float mu = R[CF_MU];
-  if (mask & 2) {
-    float lam = S[T.sm_lam + s0 + 1];
-    const float hi = mu * ln;
-    row(I1{}, I0{}, -hi, hi, 0.f, lam);
-  }
-  if (mask & 4) {
-    float lam = S[T.sm_lam + s0 + 2];
-    const float hi = mu * ln;
-    row(I2{}, I1{}, -hi, hi, 0.f, lam);
-  }
+  if (mask & 1) row(I0{}, I2{}, 0.f, __int_as_float(0x7f800000), bias);
+  const float hi = mu * lam[0];
+  if (mask & 2) row(I1{}, I0{}, -hi, hi, 0.f);
+  if (mask & 4) row(I2{}, I1{}, -hi, hi, 0.f);
+#pragma unroll
+  for (int m = 0; m < 3; ++m)
+    if (mask >> m & 1) row_store<TAPE, false>(T, S, tp, it, s0 + m, lam[m], br[m]);
 }
 template <bool TAPE>
 __device__ __forceinline__ void pair_rows(const DevTopo& T, const SL& S, const TapeStep& tp, int it, const BlkOp& op,
@@ -574,7 +600,9 @@ __device__ __forceinline__ void pair_rows(const DevTopo& T, const SL& S, const T
     float Jv = 0.f;
     Jv += dotx(lin, va) + dotx(angA, wa);
     Jv += dotx(angB, wb) - dotx(lin, vb);
-    const float dl = row_solve<TAPE>(T, S, tp, it, s0 + m, Jv, R[PF_ME + m], m == 0 ? R[PF_BI] : 0.f, lo, hi, lam);
+    int br;
+    const float dl = row_solve<false>(T, Jv, R[PF_ME + m], m == 0 ? R[PF_BI] : 0.f, lo, hi, lam, br);
+    row_store<TAPE, false>(T, S, tp, it, s0 + m, lam, br);
     if (m == 0) ln = lam;
     va = va + (dl * ima) * lin;
     wa = wa + dl * R.v3(PF_IA + 3 * m);
@@ -590,46 +618,89 @@ template <bool TAPE, bool SEQ>
 __device__ __forceinline__ void blk_sweeps(const DevTopo& T, const SL& S, const SL& X, const TapeStep& tp, int warp) {
   const uint8_t* st0 = blk_bytes(T) + T.blk_stream + warp * T.blk_stream_len;
   const int nv = 6 * T.nb;
+  auto load = [&](int a, float3& v, float3& w, float& im) {
+    v = w = f3(0.f, 0.f, 0.f);
+    im = 0.f;
+    if (a < 0) return;
+    v = X.v3(18 * a + 12);
+    w = X.v3(18 * a + 15);
+    im = S[T.sm_invm + a];
+  };
+  auto store = [&](int a, float3 v, float3 w) {
+    if (a < 0) return;
+    X.s3(18 * a + 12, v);
+    X.s3(18 * a + 15, w);
+  };
+  auto rows = [&](const BlkOp& op, int it, float ima, float imb, float3& va, float3& wa, float3& vb, float3& wb) {
+    const int type = op.type(), idx = op.idx();
+    const SL R = type == BT_GROUND ? contact_rec(T, S, idx) : (type == BT_PAIR ? pair_rec(T, S, idx) : joint_rec(T, S, idx));
+    switch (type) {
+      case BT_JOINT:
+        if (op.mask() == 31) joint_rows<TAPE, SEQ, true>(T, S, tp, it, op, R, ima, imb, va, wa, vb, wb);
+        else joint_rows<TAPE, SEQ, false>(T, S, tp, it, op, R, ima, imb, va, wa, vb, wb);
+        break;
+      case BT_GROUND:
+        if (op.mask() == 7) contact_rows<TAPE, SEQ, true>(T, S, tp, it, op, R, ima, va, wa);
+        else contact_rows<TAPE, SEQ, false>(T, S, tp, it, op, R, ima, va, wa);
+        break;
+      case BT_PAIR: pair_rows<TAPE>(T, S, tp, it, op, R, ima, imb, va, wa, vb, wb); break;
+      default: hinge_row<TAPE>(T, S, tp, it, op, R, wa, wb); break;
+    }
+  };
+  if (T.blk_single) {
+    // one block: warp 0 keeps its bodies' velocities in registers over the sweeps
+    if (warp == 0) {
+      const bool on = st0[0] != 0;
+      const BlkOp op = blk_op(T, 0);
+      const int a = op.a(), b = op.b();
+      float3 va, wa, vb, wb;
+      float ima, imb;
+      load(a, va, wa, ima);
+      load(b, vb, wb, imb);
+      for (int it = 0; it < T.iters; ++it) {
+        if (on) rows(op, it, ima, imb, va, wa, vb, wb);
+        if (TAPE)
+          for (int c = 0; c < T.nb; ++c) {
+            float* vi = tp.viter + (it * nv + 6 * c) * 32;
+            const float3 v = c == a ? va : (c == b ? vb : X.v3(18 * c + 12));
+            const float3 w = c == a ? wa : (c == b ? wb : X.v3(18 * c + 15));
+            vi[0] = v.x; vi[32] = v.y; vi[64] = v.z;
+            vi[96] = w.x; vi[128] = w.y; vi[160] = w.z;
+          }
+      }
+      store(a, va, wa);
+      store(b, vb, wb);
+    }
+    cta_sync();
+    return;
+  }
   for (int it = 0; it < T.iters; ++it) {
     const uint8_t* st = st0;
     int e = *st++;
+    BlkOp nop = blk_op(T, e & 63);
     while (e) {
       const int nxt = *st++;  // (a stream ends with a zero; one more byte is allocated)
+      const BlkOp op = nop;
+      nop = blk_op(T, nxt & 63);  // the next entry's block while this one runs
       if (e & BS_OP) {
-        const BlkOp op = blk_op(T, e & 63);
         const int a = op.a(), b = op.b();
-        const int type = op.type(), idx = op.idx();
-        const SL R = type == BT_GROUND ? contact_rec(T, S, idx) : (type == BT_PAIR ? pair_rec(T, S, idx) : joint_rec(T, S, idx));
-        const SL Xa = X.at(18 * a + 12), Xb = X.at(18 * b + 12);
-        float3 va = f3(0.f, 0.f, 0.f), wa = va, vb = va, wb = va;
-        float ima = 0.f, imb = 0.f;
-        if (a >= 0) { va = Xa.v3(0); wa = Xa.v3(3); ima = S[T.sm_invm + a]; }
-        if (b >= 0) { vb = Xb.v3(0); wb = Xb.v3(3); imb = S[T.sm_invm + b]; }
-        switch (type) {
-          case BT_JOINT: joint_rows<TAPE, SEQ>(T, S, tp, it, op, R, ima, imb, va, wa, vb, wb); break;
-          case BT_GROUND: contact_rows<TAPE, SEQ>(T, S, tp, it, op, R, ima, va, wa); break;
-          case BT_PAIR: pair_rows<TAPE>(T, S, tp, it, op, R, ima, imb, va, wa, vb, wb); break;
-          default: hinge_row<TAPE>(T, S, tp, it, op, R, wa, wb); break;
-        }
-        if (a >= 0) { Xa.s3(0, va); Xa.s3(3, wa); }
-        if (b >= 0) { Xb.s3(0, vb); Xb.s3(3, wb); }
+        float3 va, wa, vb, wb;
+        float ima, imb;
+        load(a, va, wa, ima);
+        load(b, vb, wb, imb);
+        rows(op, it, ima, imb, va, wa, vb, wb);
+        store(a, va, wa);
+        store(b, vb, wb);
       }
       if (e & BS_BAR) cta_sync();
       e = nxt;
     }
     if (TAPE) {
       float* vi = tp.viter + it * nv * 32;
-      if (T.blk_single) {
-        if (warp == 0)
-          for (int b = 0; b < T.nb; ++b)
+      for (int b = warp; b < T.nb; b += 4)
 #pragma unroll
-            for (int k = 0; k < 6; ++k) vi[(6 * b + k) * 32] = X[18 * b + 12 + k];
-      } else {
-        for (int b = warp; b < T.nb; b += 4)
-#pragma unroll
-          for (int k = 0; k < 6; ++k) vi[(6 * b + k) * 32] = X[18 * b + 12 + k];
-        cta_sync();
-      }
+        for (int k = 0; k < 6; ++k) vi[(6 * b + k) * 32] = X[18 * b + 12 + k];
+      cta_sync();
     }
   }
   cta_sync();

@@ -33,7 +33,7 @@ struct RevBody {
   float3 v, w, vb, wb;
   float im, imb, ii[6], sb[6];
 };
-__device__ __forceinline__ void rev_load(const DevTopo& T, const SL& S, int b, RevBody& B) {
+__device__ __forceinline__ void rev_load(const DevTopo& T, const SL& S, const SL& VW, int b, RevBody& B) {
   B.imb = 0.f;
 #pragma unroll
   for (int q = 0; q < 6; ++q) B.sb[q] = 0.f;
@@ -44,24 +44,27 @@ __device__ __forceinline__ void rev_load(const DevTopo& T, const SL& S, int b, R
     for (int q = 0; q < 6; ++q) B.ii[q] = 0.f;
     return;
   }
-  B.v = S.v3(T.sm_vw + 6 * b);
-  B.w = S.v3(T.sm_vw + 6 * b + 3);
+  B.v = VW.v3(6 * b);
+  B.w = VW.v3(6 * b + 3);
   B.vb = S.v3(T.sm_vb + 6 * b);
   B.wb = S.v3(T.sm_vb + 6 * b + 3);
   B.im = S[T.sm_invm + b];
   load6(S, T.sm_iinv + 6 * b, B.ii);
 }
-__device__ __forceinline__ void rev_store(const DevTopo& T, const SL& S, int b, const RevBody& B, bool lin) {
+__device__ __forceinline__ void rev_store(const DevTopo& T, const SL& S, const SL& VW, int b, const RevBody& B, bool lin) {
   if (b < 0) return;
+  float ib[6];
+  load6(S, T.sm_iinvb + 6 * b, ib);
+  const float imb = S[T.sm_invmb + b];
   if (lin) {
-    S.s3(T.sm_vw + 6 * b, B.v);
+    VW.s3(6 * b, B.v);
     S.s3(T.sm_vb + 6 * b, B.vb);
-    S[T.sm_invmb + b] += B.imb;
+    S[T.sm_invmb + b] = imb + B.imb;
   }
-  S.s3(T.sm_vw + 6 * b + 3, B.w);
+  VW.s3(6 * b + 3, B.w);
   S.s3(T.sm_vb + 6 * b + 3, B.wb);
 #pragma unroll
-  for (int q = 0; q < 6; ++q) S[T.sm_iinvb + 6 * b + q] += B.sb[q];
+  for (int q = 0; q < 6; ++q) S[T.sm_iinvb + 6 * b + q] = ib[q] + B.sb[q];
 }
 
 // Products with r x e_K and with e_K x v (two non-zero components each).
@@ -113,16 +116,62 @@ __device__ __forceinline__ void sym_outer_axis(float (&q)[6], float3 g, float3 r
   }
 }
 
-// The impulse of slot s before sweep `it` updated it.
-__device__ __forceinline__ float lam_before(const DevTopo& T, const TapeStep& tp, int it, int s) {
-  return it > 0 ? tp.lam[((it - 1) * T.nslots + s) * 32] : (T.ws ? tp.lam0[s * 32] : 0.f);
+// One sweep's tape lines on chip: the impulses it left (la) and found (lb), its clamp branches, and
+// the velocities after it, which become the working copy.
+struct RevTape {
+  SL la, lb, vw;
+  const uint8_t* br;  // slot s at br[32 s]
+};
+__device__ __forceinline__ RevTape rev_tape(const DevTopo& T, const SL& S, int it) {
+  return RevTape{S.at(T.sm_rlam + it % 3 * T.nslots), S.at(T.sm_rlam + (it + 2) % 3 * T.nslots),
+                 S.at(T.sm_vw + (it & 1) * 6 * T.nb),
+                 reinterpret_cast<const uint8_t*>(g_smem + (T.sm_rbr + (it & 1) * ((T.nslots + 3) / 4)) * 32) + (threadIdx.x & 31)};
+}
+// n bytes of the tape record (a multiple of 16, like both addresses) into unit `unit`, asynchronously.
+__device__ __forceinline__ void rev_copy(int unit, const uint8_t* src, int n) {
+  const unsigned dst = (unsigned)__cvta_generic_to_shared(g_smem + unit * 32);
+  for (int o = threadIdx.x * 16; o < n; o += 128 * 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + o), "l"(src + o) : "memory");
+}
+// Impulses after sweep `it` (-1: before the first one) into the ring of three sweeps.
+__device__ __forceinline__ void rev_stage_lam(const DevTopo& T, const TapeStep& tp, int it) {
+  const int unit = T.sm_rlam + (it + 3) % 3 * T.nslots, n = T.nslots * 128;
+  if (it >= 0) rev_copy(unit, tp.rec + T.rec_lam + (size_t)it * n, n);
+  else if (T.ws) rev_copy(unit, tp.rec + T.rec_lam0, n);
+  else
+    for (int f = threadIdx.x; f < T.nslots * 32; f += 128) g_smem[unit * 32 + f] = 0.f;
+}
+// Velocities after sweep `it` and its clamp branches (two buffers each).
+__device__ __forceinline__ void rev_stage_sweep(const DevTopo& T, const TapeStep& tp, int it) {
+  const int nv = 6 * T.nb * 128, nb = T.nslots * 32;
+  rev_copy(T.sm_vw + (it & 1) * 6 * T.nb, tp.rec + T.rec_viter + (size_t)it * nv, nv);
+  rev_copy(T.sm_rbr + (it & 1) * ((T.nslots + 3) / 4), tp.rec + T.rec_br + (size_t)it * nb, nb);
+}
+// The last sweep's lines, asked for at the start of a step.
+__device__ __forceinline__ void rev_stage_first(const DevTopo& T, const TapeStep& tp) {
+  rev_stage_lam(T, tp, T.iters - 1);
+  rev_stage_lam(T, tp, T.iters - 2);
+  rev_stage_sweep(T, tp, T.iters - 1);
+}
+// Waits for sweep `it`'s lines and asks for those of the sweep before it (every warp calls). Read from
+// L2 where they are used, at the head of every block's chain, they cost more than the rows.
+__device__ __forceinline__ void rev_begin_sweep(const DevTopo& T, const TapeStep& tp, int it) {
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  cta_sync();
+  if (it > 0) {
+    rev_stage_lam(T, tp, it - 2);
+    rev_stage_sweep(T, tp, it - 1);
+  }
 }
 
-// A joint's linear and angular rows, last first.
+// Rows, last first. As in the rollout, a block loads everything it reads before its first row and
+// stores after its last one; adjoints of the record are summed in registers.
+// One linear row of a joint: lam is its impulse's adjoint, meb the sum of the effective mass' adjoint;
+// returns the adjoint of J v.
 template <int K>
-__device__ __forceinline__ void rev_lin(const DevTopo& T, const SL& S, const SL& R, int s, float la, float lb, float3 ra,
-                                        float3 rb, RevBody& A, RevBody& B, float3& rab, float3& rbb) {
-  const float dl = la - lb, me = R[JF_ME + K];
+__device__ __forceinline__ float rev_lin(const DevTopo& T, float la, float lb, float me, float bi, float3 ra, float3 rb,
+                                         RevBody& A, RevBody& B, float3& rab, float3& rbb, float& lam, float& meb) {
+  const float dl = la - lb;
   const float3 IA = symv_axis<K>(A.ii, ra), IBn = symv_axis<K>(B.ii, rb);  // the child's is -IBn
   // velocities before the row, then the adjoint of the row's change
   const float ca = dl * A.im, cb = dl * B.im;
@@ -131,8 +180,8 @@ __device__ __forceinline__ void rev_lin(const DevTopo& T, const SL& S, const SL&
   axis_of<K>(B.v) += cb;
   B.w = axpy3(dl, IBn, B.w);
   const float dbar = (A.im * axis_of<K>(A.vb) + dot3(IA, A.wb)) - (B.im * axis_of<K>(B.vb) + dot3(IBn, B.wb));
-  const float pbar = S[T.sm_lam + s] + dbar, jvb = -me * pbar;
-  S[T.sm_lam + s] = fmaf(pbar, fmaf(-me, T.gamma, 1.f), -dbar);
+  const float pbar = lam + dbar, jvb = -me * pbar;
+  lam = fmaf(pbar, fmaf(-me, T.gamma, 1.f), -dbar);
   // adjoints of M^-1 J^T (before the update of the velocity adjoints)
   const float3 ga = dl * A.wb, gb = dl * B.wb;
   add_e_cross<K>(rab, 1.f, axpy3(jvb, A.w, symv(A.ii, ga)));
@@ -142,120 +191,147 @@ __device__ __forceinline__ void rev_lin(const DevTopo& T, const SL& S, const SL&
   A.imb = fmaf(dl, axis_of<K>(A.vb), A.imb);
   B.imb = fmaf(-dl, axis_of<K>(B.vb), B.imb);
   const float Jv = (axis_of<K>(A.v) + dot_axis<K>(ra, A.w)) - (axis_of<K>(B.v) + dot_axis<K>(rb, B.w));
-  R[JR_N + JA_ME + K] += -pbar * (Jv + R[JF_BI + K] + T.gamma * lb);
-  R[JR_N + JA_BI + K] += jvb;
+  meb = -pbar * (Jv + bi + T.gamma * lb);
   axis_of<K>(A.vb) += jvb;
   add_axis<K>(A.wb, jvb, ra);
   axis_of<K>(B.vb) -= jvb;
   add_axis<K>(B.wb, -jvb, rb);
+  return jvb;
 }
 // A row without a linear part along the child's direction d (J_wb = d, J_wa = -d): angular, limit and
-// servo rows. Returns the adjoint of d. branch: 0 inside, 1 lower bound, 2 upper bound.
-__device__ __forceinline__ float3 rev_ang(const DevTopo& T, const SL& S, const SL& R, int m, int s, float la, float lb,
-                                          int br, float3 d, RevBody& A, RevBody& B, float& lbar) {
-  const float dl = la - lb, me = R[JF_ME + m];
+// servo rows. db: adjoint of d. branch: 0 inside, 1 lower bound, 2 upper bound; lbar: the clamped
+// impulse's adjoint.
+__device__ __forceinline__ float rev_ang(const DevTopo& T, float la, float lb, float me, float bi, int br, float3 d,
+                                         RevBody& A, RevBody& B, float3& db, float& lam, float& meb, float& lbar) {
+  const float dl = la - lb;
   const float3 IA = symv(A.ii, d), IB = symv(B.ii, d);  // the parent's is -IA
   A.w = axpy3(dl, IA, A.w);
   B.w = axpy3(-dl, IB, B.w);
   const float dbar = dot3(IB, B.wb) - dot3(IA, A.wb);
-  lbar = S[T.sm_lam + s] + dbar;
+  lbar = lam + dbar;
   const float pbar = br == 0 ? lbar : 0.f, jvb = -me * pbar;
-  S[T.sm_lam + s] = fmaf(pbar, fmaf(-me, T.gamma, 1.f), -dbar);
+  lam = fmaf(pbar, fmaf(-me, T.gamma, 1.f), -dbar);
   const float3 ga = dl * A.wb, gb = dl * B.wb;
-  const float3 db = (axpy3(jvb, B.w, symv(B.ii, gb))) - (axpy3(jvb, A.w, symv(A.ii, ga)));
+  db = (axpy3(jvb, B.w, symv(B.ii, gb))) - (axpy3(jvb, A.w, symv(A.ii, ga)));
   sym_outer(A.sb, -ga, d);
   sym_outer(B.sb, gb, d);
   const float Jv = dot3(d, B.w - A.w);
-  R[JR_N + JA_ME + m] += -pbar * (Jv + R[JF_BI + m] + T.gamma * lb);
-  R[JR_N + JA_BI + m] += jvb;
+  meb = -pbar * (Jv + bi + T.gamma * lb);
   A.wb = axpy3(-jvb, d, A.wb);
   B.wb = axpy3(jvb, d, B.wb);
-  return db;
+  return jvb;
 }
-__device__ __forceinline__ void acc3(const SL& R, int f, float3 v) { R.a3(f, v); }
 
-__device__ __forceinline__ void rev_joint(const DevTopo& T, const SL& S, const TapeStep& tp, int it, const BlkOp& op,
-                                          const SL& R, RevBody& A, RevBody& B) {
-  const int mask = op.mask(), s0 = op.slot();
-  float la[5], lb[5];
+template <bool FULL>
+__device__ __forceinline__ void rev_joint(const DevTopo& T, const SL& S, const RevTape& tp, const BlkOp& op, const SL& R,
+                                          RevBody& A, RevBody& B) {
+  const int mask = FULL ? 31 : op.mask(), s0 = op.slot();
+  const SL Q = R.at(JR_N);
+  const float3 ra = R.v3(JF_RA), rb = R.v3(JF_RB);
+  float la[5], lb[5], lam[5], me[5], bi[5], meb[5], bib[5];
+  float3 t[2], tb[2];
 #pragma unroll
   for (int k = 0; k < 5; ++k)
     if (mask >> k & 1) {
-      la[k] = tp.lam[(it * T.nslots + s0 + k) * 32];
-      lb[k] = lam_before(T, tp, it, s0 + k);
+      la[k] = tp.la[s0 + k];
+      lb[k] = tp.lb[s0 + k];
+      lam[k] = S[T.sm_lam + s0 + k];
+      me[k] = R[JF_ME + k];
+      bi[k] = R[JF_BI + k];
+      if (k >= 3) t[k - 3] = R.v3(JF_T + 3 * (k - 3));
     }
-  const float3 ra = R.v3(JF_RA), rb = R.v3(JF_RB);
   float unused;
 #pragma unroll
-  for (int k = 1; k >= 0; --k) {
-    if (!(mask >> (3 + k) & 1)) continue;
-    const float3 tb = rev_ang(T, S, R, 3 + k, s0 + 3 + k, la[3 + k], lb[3 + k], 0, -R.v3(JF_T + 3 * k), A, B, unused);
-    acc3(R, JR_N + JA_T + 3 * k, -tb);
-  }
-  if (mask & 7) {
-    float3 rab = f3(0.f, 0.f, 0.f), rbb = rab;
-    if (mask & 4) rev_lin<2>(T, S, R, s0 + 2, la[2], lb[2], ra, rb, A, B, rab, rbb);
-    if (mask & 2) rev_lin<1>(T, S, R, s0 + 1, la[1], lb[1], ra, rb, A, B, rab, rbb);
-    if (mask & 1) rev_lin<0>(T, S, R, s0, la[0], lb[0], ra, rb, A, B, rab, rbb);
-    acc3(R, JR_N + JA_RA, rab);
-    acc3(R, JR_N + JA_RB, rbb);
-  }
+  for (int k = 4; k >= 3; --k)
+    if (mask >> k & 1)
+      bib[k] = rev_ang(T, la[k], lb[k], me[k], bi[k], 0, -t[k - 3], A, B, tb[k - 3], lam[k], meb[k], unused);
+  float3 rab = f3(0.f, 0.f, 0.f), rbb = rab;
+  if (mask & 4) bib[2] = rev_lin<2>(T, la[2], lb[2], me[2], bi[2], ra, rb, A, B, rab, rbb, lam[2], meb[2]);
+  if (mask & 2) bib[1] = rev_lin<1>(T, la[1], lb[1], me[1], bi[1], ra, rb, A, B, rab, rbb, lam[1], meb[1]);
+  if (mask & 1) bib[0] = rev_lin<0>(T, la[0], lb[0], me[0], bi[0], ra, rb, A, B, rab, rbb, lam[0], meb[0]);
+#pragma unroll
+  for (int k = 0; k < 5; ++k)
+    if (mask >> k & 1) {
+      meb[k] += Q[JA_ME + k];
+      bib[k] += Q[JA_BI + k];
+      if (k >= 3) tb[k - 3] = Q.v3(JA_T + 3 * (k - 3)) - tb[k - 3];
+    }
+  rab = Q.v3(JA_RA) + rab;
+  rbb = Q.v3(JA_RB) + rbb;
+#pragma unroll
+  for (int k = 0; k < 5; ++k)
+    if (mask >> k & 1) {
+      S[T.sm_lam + s0 + k] = lam[k];
+      Q[JA_ME + k] = meb[k];
+      Q[JA_BI + k] = bib[k];
+      if (k >= 3) Q.s3(JA_T + 3 * (k - 3), tb[k - 3]);
+    }
+  Q.s3(JA_RA, rab);
+  Q.s3(JA_RB, rbb);
 }
-__device__ __forceinline__ void rev_hinge(const DevTopo& T, const SL& S, const TapeStep& tp, int it, const BlkOp& op,
-                                          const SL& R, int j, RevBody& A, RevBody& B) {
+__device__ __forceinline__ void rev_hinge(const DevTopo& T, const SL& S, const RevTape& tp, const BlkOp& op, const SL& R, int j,
+                                          RevBody& A, RevBody& B) {
   const bool lim = op.type() == BT_LIMIT;
-  const int s = op.slot(), o = (it * T.nslots + s) * 32;
+  const int s = op.slot(), m = lim ? 5 : 6;
+  const SL Q = R.at(JR_N);
   const float sg = lim ? R[JF_LS] : 1.f;
-  const int br = tp.br[o];
-  float lbar;
-  const float3 ub = rev_ang(T, S, R, lim ? 5 : 6, s, tp.lam[o], lam_before(T, tp, it, s), br, sg * S.v3(T.sm_ua + 3 * j), A,
-                            B, lbar);
-  acc3(R, JR_N + JA_U, sg * ub);
-  if (!lim) R[JR_N + JA_BND] += (br == 2 ? 1.f : (br == 1 ? -1.f : 0.f)) * lbar;
+  const int br = tp.br[s * 32];
+  const float me = R[JF_ME + m], bi = R[JF_BI + m], la = tp.la[s], lb = tp.lb[s];
+  const float meb0 = Q[JA_ME + m], bib0 = Q[JA_BI + m], bnd0 = Q[JA_BND];
+  const float3 u0 = Q.v3(JA_U), ua = S.v3(T.sm_ua + 3 * j);
+  float lam = S[T.sm_lam + s], meb, lbar;
+  float3 ub;
+  const float bib = rev_ang(T, la, lb, me, bi, br, sg * ua, A, B, ub, lam, meb, lbar);
+  S[T.sm_lam + s] = lam;
+  Q[JA_ME + m] = meb0 + meb;
+  Q[JA_BI + m] = bib0 + bib;
+  Q.s3(JA_U, u0 + sg * ub);
+  if (!lim) Q[JA_BND] = bnd0 + (br == 2 ? 1.f : (br == 1 ? -1.f : 0.f)) * lbar;
 }
-__device__ __forceinline__ void rev_contact(const DevTopo& T, const SL& S, const TapeStep& tp, int it, const BlkOp& op,
-                                            const SL& R, RevBody& A) {
+__device__ __forceinline__ void rev_contact(const DevTopo& T, const SL& S, const RevTape& tp, const BlkOp& op, const SL& R,
+                                            RevBody& A) {
   const int mask = op.mask(), s0 = op.slot();
-  float la[3], lb[3];
+  const SL Q = R.at(CR_N);
+  float la[3], lb[3], lam[3], me[3], meb[3];
   int br[3];
 #pragma unroll
   for (int m = 0; m < 3; ++m) {
-    const int o = (it * T.nslots + s0 + m) * 32;
-    la[m] = tp.lam[o];
-    lb[m] = lam_before(T, tp, it, s0 + m);
-    br[m] = tp.br[o];
+    la[m] = tp.la[s0 + m];
+    lb[m] = tp.lb[s0 + m];
+    br[m] = tp.br[(s0 + m) * 32];
+    lam[m] = S[T.sm_lam + s0 + m];
+    me[m] = R[CF_ME + m];
+    meb[m] = 0.f;
   }
   const float3 ra = R.v3(CF_RA);
-  const float mu = R[CF_MU];
+  const float mu = R[CF_MU], bias0 = R[CF_BI];
   float3 rab = f3(0.f, 0.f, 0.f);
   // the normal impulse a friction row saw: the sweep's own (the normal row comes first)
   const float lnrm = la[0];
-  float lbn = S[T.sm_lam + s0], mub = 0.f;
+  float mub = 0.f, bib = 0.f;
   auto row = [&](auto MI, auto AI, float bias) {
     constexpr int m = decltype(MI)::value, ax = decltype(AI)::value;
-    const float dl = la[m] - lb[m], me = R[CF_ME + m];
+    const float dl = la[m] - lb[m];
     const float3 IA = symv_axis<ax>(A.ii, ra);
     const float ca = dl * A.im;
     axis_of<ax>(A.v) -= ca;
     A.w = axpy3(-dl, IA, A.w);
     const float dbar = A.im * axis_of<ax>(A.vb) + dot3(IA, A.wb);
-    const float lbar = (m == 0 ? lbn : S[T.sm_lam + s0 + m]) + dbar;
-    const float pbar = br[m] == 0 ? lbar : 0.f, jvb = -me * pbar;
+    const float lbar = lam[m] + dbar;
+    const float pbar = br[m] == 0 ? lbar : 0.f, jvb = -me[m] * pbar;
     if (m > 0) {
       const float sg = br[m] == 2 ? 1.f : (br[m] == 1 ? -1.f : 0.f);
       mub += sg * lnrm * lbar;
-      lbn += sg * mu * lbar;
+      lam[0] += sg * mu * lbar;
     }
-    const float keep = fmaf(pbar, fmaf(-me, T.gamma, 1.f), -dbar);
-    if (m == 0) lbn = keep;
-    else S[T.sm_lam + s0 + m] = keep;
+    lam[m] = fmaf(pbar, fmaf(-me[m], T.gamma, 1.f), -dbar);
     const float3 ga = dl * A.wb;
     add_e_cross<ax>(rab, 1.f, axpy3(jvb, A.w, symv(A.ii, ga)));
     sym_outer_axis<ax>(A.sb, ga, ra);
     A.imb = fmaf(dl, axis_of<ax>(A.vb), A.imb);
     const float Jv = axis_of<ax>(A.v) + dot_axis<ax>(ra, A.w);
-    R[CR_N + CA_ME + m] += -pbar * (Jv + bias + T.gamma * lb[m]);
-    if (m == 0) R[CR_N + CA_BI] += jvb;
+    meb[m] = -pbar * (Jv + bias + T.gamma * lb[m]);
+    if (m == 0) bib = jvb;
     axis_of<ax>(A.vb) += jvb;
     add_axis<ax>(A.wb, jvb, ra);
   };
@@ -264,21 +340,31 @@ __device__ __forceinline__ void rev_contact(const DevTopo& T, const SL& S, const
   using I2 = std::integral_constant<int, 2>;
   if (mask & 4) row(I2{}, I1{}, 0.f);
   if (mask & 2) row(I1{}, I0{}, 0.f);
-  if (mask & 1) row(I0{}, I2{}, R[CF_BI]);
-  S[T.sm_lam + s0] = lbn;
-  R[CR_N + CA_MU] += mub;
-  acc3(R, CR_N + CA_RA, rab);
+  if (mask & 1) row(I0{}, I2{}, bias0);
+#pragma unroll
+  for (int m = 0; m < 3; ++m) meb[m] += Q[CA_ME + m];
+  bib += Q[CA_BI];
+  mub += Q[CA_MU];
+  rab = Q.v3(CA_RA) + rab;
+#pragma unroll
+  for (int m = 0; m < 3; ++m) {
+    S[T.sm_lam + s0 + m] = lam[m];  // (the normal's also from a block of friction rows alone)
+    Q[CA_ME + m] = meb[m];
+  }
+  Q[CA_BI] = bib;
+  Q[CA_MU] = mub;
+  Q.s3(CA_RA, rab);
 }
-__device__ __forceinline__ void rev_pair(const DevTopo& T, const SL& S, const TapeStep& tp, int it, const BlkOp& op,
-                                         const SL& R, RevBody& A, RevBody& B) {
+__device__ __forceinline__ void rev_pair(const DevTopo& T, const SL& S, const RevTape& tp, const BlkOp& op, const SL& R,
+                                         RevBody& A, RevBody& B) {
   const int mask = op.mask(), s0 = op.slot();
-  const float mu = R[PF_MU], lnrm = tp.lam[(it * T.nslots + s0) * 32];
+  const float mu = R[PF_MU], lnrm = tp.la[s0];
 #pragma unroll 1
   for (int m = 2; m >= 0; --m) {
     if (!(mask >> m & 1)) continue;
-    const int s = s0 + m, o = (it * T.nslots + s) * 32, br = tp.br[o];
+    const int s = s0 + m, br = tp.br[s * 32];
     const float3 lin = R.v3(PF_LIN + 3 * m), angA = R.v3(PF_ANGA + 3 * m), angB = R.v3(PF_ANGB + 3 * m);
-    const float lb = lam_before(T, tp, it, s), dl = tp.lam[o] - lb, me = R[PF_ME + m];
+    const float lb = tp.lb[s], dl = tp.la[s] - lb, me = R[PF_ME + m];
     const float3 IA = symv(A.ii, angA), IB = symv(B.ii, angB);
     A.v = axpy3(-dl * A.im, lin, A.v);
     A.w = axpy3(-dl, IA, A.w);
@@ -312,57 +398,44 @@ __device__ __forceinline__ void rev_pair(const DevTopo& T, const SL& S, const Ta
   }
 }
 
-// The velocities after sweep `it` into the working copy, and the tape lines of the sweep before it
-// into L1 (its impulses are read twice: as the sweep's own and as the next one's start).
-__device__ __forceinline__ void rev_begin_sweep(const DevTopo& T, const SL& S, const TapeStep& tp, int it, int warp) {
-  const float* vi = tp.viter + it * 6 * T.nb * 32;
-  for (int f = warp; f < 6 * T.nb; f += 4) S[T.sm_vw + f] = vi[f * 32];
-  if (it > 0) {
-    const int lane = threadIdx.x & 31;
-    const float* l0 = tp.lam - lane + (it - 1) * T.nslots * 32;
-    const float* v0 = vi - lane - 6 * T.nb * 32;
-    const uint8_t* b0 = tp.br - lane + (it - 1) * T.nslots * 32;
-    const float* p0 = it > 1 ? l0 - T.nslots * 32 : (T.ws ? tp.lam0 - lane : l0);
-    for (int f = threadIdx.x; f < T.nslots; f += 128) prefetch_l1(p0 + f * 32);
-    for (int f = threadIdx.x; f < 6 * T.nb; f += 128) prefetch_l1(v0 + f * 32);
-    for (int f = threadIdx.x; f < (T.nslots + 3) / 4; f += 128) prefetch_l1(b0 + f * 128);
-  }
-}
-
 // The sweeps backwards (every warp calls; ends after a CTA barrier). On entry VB holds the adjoint
 // of the solver's output velocities, on exit that of its input velocities.
 __device__ __forceinline__ void blk_sweeps_rev(const DevTopo& T, const SL& S, const TapeStep& tp, int warp) {
   const uint8_t* st0 = blk_bytes(T) + T.blk_stream + warp * T.blk_stream_len;
+  auto rows = [&](const BlkOp& op, const RevTape& rt, RevBody& A, RevBody& B) {
+    const int type = op.type(), idx = op.idx();
+    if (type == BT_GROUND) rev_contact(T, S, rt, op, contact_rec(T, S, idx), A);
+    else if (type == BT_JOINT) {
+      if (op.mask() == 31) rev_joint<true>(T, S, rt, op, joint_rec(T, S, idx), A, B);
+      else rev_joint<false>(T, S, rt, op, joint_rec(T, S, idx), A, B);
+    } else if (type == BT_PAIR) rev_pair(T, S, rt, op, pair_rec(T, S, idx), A, B);
+    else rev_hinge(T, S, rt, op, joint_rec(T, S, idx), idx, A, B);
+  };
   for (int it = T.iters - 1; it >= 0; --it) {
-    rev_begin_sweep(T, S, tp, it, warp);
-    cta_sync();
+    rev_begin_sweep(T, tp, it);
+    const RevTape rt = rev_tape(T, S, it);
     const uint8_t* st = st0;
     int e = *st++;
+    BlkOp nop = blk_op(T, e & 63);
     while (e) {
       const int nxt = *st++;
+      const BlkOp op = nop;
+      nop = blk_op(T, nxt & 63);  // the next entry's block while this one runs
       if (e & BS_OP) {
-        const BlkOp op = blk_op(T, e & 63);
-        const int a = op.a(), b = op.b(), type = op.type(), idx = op.idx();
+        const int a = op.a(), b = op.b(), type = op.type();
+        const bool lin = type <= BT_JOINT || type >= BT_GROUND;
         RevBody A, B;
-        rev_load(T, S, a, A);
-        if (type == BT_GROUND) {
-          rev_contact(T, S, tp, it, op, contact_rec(T, S, idx), A);
-          rev_store(T, S, a, A, true);
-        } else {
-          rev_load(T, S, b, B);
-          if (type == BT_JOINT) rev_joint(T, S, tp, it, op, joint_rec(T, S, idx), A, B);
-          else if (type == BT_PAIR) rev_pair(T, S, tp, it, op, pair_rec(T, S, idx), A, B);
-          else rev_hinge(T, S, tp, it, op, joint_rec(T, S, idx), idx, A, B);
-          const bool lin = type == BT_JOINT || type == BT_PAIR;
-          rev_store(T, S, a, A, lin);
-          rev_store(T, S, b, B, lin);
-        }
+        rev_load(T, S, rt.vw, a, A);
+        rev_load(T, S, rt.vw, b, B);
+        rows(op, rt, A, B);
+        rev_store(T, S, rt.vw, a, A, lin);
+        rev_store(T, S, rt.vw, b, B, lin);
       }
       if (e & BS_BAR) cta_sync();
       e = nxt;
     }
-    cta_sync();
   }
+  cta_sync();
 }
 
 // ------------------------------------------------------------------------------ items
@@ -1081,6 +1154,7 @@ __device__ __forceinline__ void blk_reverse_step(const DevTopo& T, const DevPtrs
   const TapeStep tp = tape_step(T, D, ts);
   const LaneT<SL> L{S, C.P, S, i};
   const BLaneT<SL> Bl{L, C.X, C.G, GC{tp.vminus, 32}};
+  rev_stage_first(T, tp);
   if (load_x1)
     for (int f = warp; f < nf; f += 4) C.X[f] = x_t1[(size_t)f * Bp + i];
   if (T.grad_decay != 1.f) {  // section 3.2: the adjoint from later steps shrinks by alpha per step
@@ -1101,15 +1175,6 @@ __device__ __forceinline__ void blk_reverse_step(const DevTopo& T, const DevPtrs
     for (int q = 0; q < 6; ++q) S[T.sm_iinvb + 6 * b + q] = 0.f;
   }
   for (int s = warp; s < T.nslots; s += 4) S[T.sm_lam + s] = 0.f;  // impulse adjoints
-  {  // the last sweep's tape lines into L1 (rev_begin_sweep asks for the following ones)
-    const int it = T.iters - 1;
-    for (int s = threadIdx.x; s < T.nslots; s += 128) {
-      prefetch_l1(tp.lam - lane + (it * T.nslots + s) * 32);
-      prefetch_l1(it > 0 ? tp.lam - lane + ((it - 1) * T.nslots + s) * 32 : (T.ws ? tp.lam0 - lane + s * 32 : tp.lam - lane));
-      if (s * 4 < T.nslots) prefetch_l1(tp.br - lane + it * T.nslots * 32 + s * 128);
-    }
-    for (int f = threadIdx.x; f < 6 * T.nb; f += 128) prefetch_l1(tp.viter - lane + (it * 6 * T.nb + f) * 32);
-  }
   inverse_inertia(T, L, C.X, mine);
   cta_sync();
   // the step's records, re-formed bit for bit
@@ -1278,7 +1343,7 @@ __global__ void __launch_bounds__(128, 1) k_backward_seg_blk(const __grid_consta
       blk_step<true, Q>(Tf, D, L, X, act, t, t - ta, nullptr, T.n_layers > 0 ? D.dump + (size_t)t * Bp + i : nullptr, warp);
     }
     for (int f = warp; f < nf; f += 4) D.seg[(size_t)(tb - ta) * sb + (size_t)f * Bp + i] = X[f];
-    __threadfence_block();
+    __threadfence();  // the reverse reads the tape through L2
     cta_sync();
     blk_load(T, D);
     cta_sync();

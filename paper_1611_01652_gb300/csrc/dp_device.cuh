@@ -94,6 +94,7 @@ struct DevTopo {
   int blk_fwd, blk_bwd;  // 1: rollouts and steps / reverse passes of this world run on the four-warp step
   int rec_rows;          // 1: the tape records hold the constraint rows (read by the one-warp reverse)
   int rec_j, rec_c, rec_p;  // strides of the joints', contacts' and pairs' records
+  int sm_rlam, sm_rbr;   // four-warp reverse: staged tape lines (impulses, clamp branches)
   int sm_hbuf;           // controller buffers over the records (bfloat16 activations or delta planes, or ping-pong)
   int cslot;
   int16_t jslot[DPK_MAXJ], jlim[DPK_MAXJ], jmot[DPK_MAXJ];
