@@ -247,7 +247,7 @@ void plan_smem_blk_fwd(DevTopo& T, int keep = 0) {
   T.sm_wbr = take(T.nj);
   T.sm_lam = take(T.nslots);
   T.sm_h = take(T.n_rec);
-  T.sm_ws = take(76 + T.n_wsg);  // learned start: features and outputs per warp, harvest row ids
+  T.sm_ws = take(19 * T.blk_nw + T.n_wsg);  // learned start: features and outputs per warp, harvest row ids
   T.sm_prog = take((T.blk_bytes_total + 127) / 128);
   // controller activations and the records share one region: the records are assembled after the
   // servo targets have consumed the controller output

@@ -22,8 +22,11 @@
 
 extern __shared__ float g_smem[];
 
-// CTA barrier 1 over the four warps (each warp arrives from its own code path).
-__device__ __forceinline__ void cta_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+// CTA barrier 1 over all warps (each warp arrives from its own code path).
+__device__ __forceinline__ void cta_sync() { asm volatile("bar.sync 1;" ::: "memory"); }
+// Warps of the CTA (DevTopo.blk_nw), and the joints and bodies k of warp w (k % warps == w) as a mask.
+__device__ __forceinline__ int blk_nw() { return blockDim.x >> 5; }
+__device__ __forceinline__ uint32_t blk_mine(int warp) { return (blk_nw() == 8 ? 0x01010101u : 0x11111111u) << warp; }
 
 // Compact records in shared memory ([field][32 lanes], DevTopo.sm_rows; stride rec_j, rec_c, rec_p),
 // one per joint, contact sphere and sphere pair. The rollout keeps I^-1 J_w behind the first JR_N
@@ -139,7 +142,7 @@ __device__ __forceinline__ void blk_stream(const DevTopo& T, int warp, bool reve
   bool any = false;
   if (lane < nl) {
     const int level = reverse ? nl - 1 - lane : lane;
-    for (int w = 0; w < 4; ++w) {
+    for (int w = 0; w < blk_nw(); ++w) {
       const uint8_t* f = base + T.blk_lev + w * (nl + 1) + level;
       const unsigned long long m = ((1ull << f[1]) - 1ull) & ~((1ull << f[0]) - 1ull) & alive;
       any |= m != 0ull;
@@ -368,9 +371,9 @@ __device__ __forceinline__ void pair_assemble(const DevTopo& T, const SL& S, con
 template <bool INV, class G, class VV>
 __device__ __forceinline__ void blk_assemble(const DevTopo& T, const SL& S, const G& P, const SL& X, const VV& V, uint8_t* ao,
                                              int warp) {
-  for (int j = warp; j < T.nj; j += 4) joint_assemble<INV>(T, S, P, X, j, ao);
-  for (int q = warp; q < T.ns; q += 4) contact_assemble<INV>(T, S, P, X, V, q, ao);
-  for (int p = warp; p < T.np; p += 4) pair_assemble<INV>(T, S, P, X, V, p, ao);
+  for (int j = warp; j < T.nj; j += blk_nw()) joint_assemble<INV>(T, S, P, X, j, ao);
+  for (int q = warp; q < T.ns; q += blk_nw()) contact_assemble<INV>(T, S, P, X, V, q, ao);
+  for (int p = warp; p < T.np; p += blk_nw()) pair_assemble<INV>(T, S, P, X, V, p, ao);
 }
 
 // One row in full (the stages that walk slots: the learned warm start, the residual).
@@ -697,7 +700,7 @@ __device__ __forceinline__ void blk_sweeps(const DevTopo& T, const SL& S, const 
     }
     if (TAPE) {
       float* vi = tp.viter + it * nv * 32;
-      for (int b = warp; b < T.nb; b += 4)
+      for (int b = warp; b < T.nb; b += blk_nw())
 #pragma unroll
         for (int k = 0; k < 6; ++k) vi[(6 * b + k) * 32] = X[18 * b + 12 + k];
       cta_sync();

@@ -130,7 +130,7 @@ __device__ __forceinline__ RevTape rev_tape(const DevTopo& T, const SL& S, int i
 // n bytes of the tape record (a multiple of 16, like both addresses) into unit `unit`, asynchronously.
 __device__ __forceinline__ void rev_copy(int unit, const uint8_t* src, int n) {
   const unsigned dst = (unsigned)__cvta_generic_to_shared(g_smem + unit * 32);
-  for (int o = threadIdx.x * 16; o < n; o += 128 * 16)
+  for (int o = threadIdx.x * 16; o < n; o += blockDim.x * 16)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + o), "l"(src + o) : "memory");
 }
 // Impulses after sweep `it` (-1: before the first one) into the ring of three sweeps.
@@ -139,7 +139,7 @@ __device__ __forceinline__ void rev_stage_lam(const DevTopo& T, const TapeStep& 
   if (it >= 0) rev_copy(unit, tp.rec + T.rec_lam + (size_t)it * n, n);
   else if (T.ws) rev_copy(unit, tp.rec + T.rec_lam0, n);
   else
-    for (int f = threadIdx.x; f < T.nslots * 32; f += 128) g_smem[unit * 32 + f] = 0.f;
+    for (int f = threadIdx.x; f < T.nslots * 32; f += blockDim.x) g_smem[unit * 32 + f] = 0.f;
 }
 // Velocities after sweep `it` and its clamp branches (two buffers each).
 __device__ __forceinline__ void rev_stage_sweep(const DevTopo& T, const TapeStep& tp, int it) {
@@ -926,12 +926,12 @@ __device__ __forceinline__ void features_reverse_joints(const DevTopo& T, const 
   int k = 0;
   if (T.features & 1) {
     for (int m = 0; m < T.n_motors; ++m)
-      if ((T.motor_joint[m] & 3) == warp) S[T.sm_thb + T.motor_joint[m]] += sbar[k + m];
+      if ((T.motor_joint[m] & (blk_nw() - 1)) == warp) S[T.sm_thb + T.motor_joint[m]] += sbar[k + m];
     k += T.n_motors;
   }
   if (T.features & 2)
     for (int m = 0; m < T.n_motors; ++m)
-      if ((T.motor_joint[m] & 3) == warp) S[T.sm_thdb + T.motor_joint[m]] += sbar[k + m];
+      if ((T.motor_joint[m] & (blk_nw() - 1)) == warp) S[T.sm_thdb + T.motor_joint[m]] += sbar[k + m];
 }
 template <class AV>
 __device__ __forceinline__ void features_reverse_rest(const DevTopo& T, const RevCtx& C, const AV& sbar) {
@@ -1003,14 +1003,14 @@ __device__ __forceinline__ void mask_delta(float (&d)[NT][4], int mt, int n1, co
 // The tensor-core controller reversed on the four warps: ub the output adjoint, sbar receives the
 // input adjoint, col the step's dump column of lane 0. The planes (four of [32][H + 8] bfloat16) lie
 // over the records, whose packages have been added up by then. Ends before a barrier.
-template <int H>
-__device__ __forceinline__ void ctrl_backward_4w(const DevTopo& T, const DevPtrs& D, const SL& ub, const SL& sbar, float* col,
+template <int H, int NW>
+__device__ __forceinline__ void ctrl_backward_nw(const DevTopo& T, const DevPtrs& D, const SL& ub, const SL& sbar, float* col,
                                                  int warp) {
-  constexpr int NT = H / 32, KT = H / 16;
+  constexpr int NT = H / (8 * NW), KT = H / 16;
   constexpr CtrlTCLayout Lw = ctrl_tc_layout(H, H);
   const __nv_bfloat16* Wc = D.Wtc;
   const size_t N = (size_t)T.horizon * T.Bp;
-  const int n1 = warp * (H / 4), no = T.widths[3], lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+  const int n1 = warp * (H / NW), no = T.widths[3], lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
   __nv_bfloat16* p0 = reinterpret_cast<__nv_bfloat16*>(g_smem + T.sm_hbuf * 32);
   __nv_bfloat16 *h2 = p0, *l2 = p0 + 32 * (H + 8), *h1 = p0 + 64 * (H + 8), *l1 = p0 + 96 * (H + 8);
 #pragma unroll
@@ -1063,7 +1063,7 @@ __device__ __forceinline__ void ctrl_backward_4w(const DevTopo& T, const DevPtrs
     }
   }
   cta_sync();
-  {
+  if (warp < CTRL_TC_KP0 / 8) {  // eight inputs a warp
     float s[2][1][4];
     zero_acc<1>(s[0]);
     zero_acc<1>(s[1]);
@@ -1085,26 +1085,26 @@ __device__ __forceinline__ void ctrl_backward_4w(const DevTopo& T, const DevPtrs
       store_c<1>(s[mt], mt, warp * 8, T.widths[0], [&](int f, int r, float v) { sbar.lane_at(f, r) = v; });
   }
 }
-template <int H>
-__device__ __noinline__ void ctrl_backward_4w_call(const DevTopo& T, const DevPtrs& D, SL ub, SL sbar, float* col, int warp) {
-  ctrl_backward_4w<H>(T, D, ub, sbar, col, warp);
+template <int H, int NW>
+__device__ __noinline__ void ctrl_backward_nw_call(const DevTopo& T, const DevPtrs& D, SL ub, SL sbar, float* col, int warp) {
+  ctrl_backward_nw<H, NW>(T, D, ub, sbar, col, warp);
 }
 template <class Q>
 __device__ __forceinline__ void ctrl_backward_blk(const DevTopo& T, const DevPtrs& D, const SL& ub, const SL& sbar, float* col,
                                                   int warp) {
   if constexpr (Q::CTRL_H == 128) {
-    ctrl_backward_4w<128>(T, D, ub, sbar, col, warp);
+    ctrl_backward_nw<128, Q::NW>(T, D, ub, sbar, col, warp);
   } else if constexpr (Q::CTRL_H == 256) {
-    ctrl_backward_4w_call<256>(T, D, ub, sbar, col, warp);
+    ctrl_backward_nw_call<256, Q::NW>(T, D, ub, sbar, col, warp);
   } else {
-    if (T.widths[1] == 64) ctrl_backward_4w_call<64>(T, D, ub, sbar, col, warp);
-    else if (T.widths[1] == 128) ctrl_backward_4w_call<128>(T, D, ub, sbar, col, warp);
-    else ctrl_backward_4w_call<256>(T, D, ub, sbar, col, warp);
+    if (T.widths[1] == 64) ctrl_backward_nw_call<64, Q::NW>(T, D, ub, sbar, col, warp);
+    else if (T.widths[1] == 128) ctrl_backward_nw_call<128, Q::NW>(T, D, ub, sbar, col, warp);
+    else ctrl_backward_nw_call<256, Q::NW>(T, D, ub, sbar, col, warp);
   }
 }
 // The fp32-arithmetic controller reversed (see controller_reverse), 8 inputs of a layer per warp and
 // pass; ping-pong buffers z0, z1 over the records.
-__device__ __forceinline__ void controller_reverse_4w(const DevTopo& T, const DevPtrs& D, const GW* act, const GW* del,
+__device__ __forceinline__ void controller_reverse_nw(const DevTopo& T, const DevPtrs& D, const GW* act, const GW* del,
                                                       const SL& z0, const SL& z1, const SL& sbar, int warp) {
   const int L = T.n_layers;
   SL cur = z0, nxt = z1;
@@ -1112,18 +1112,18 @@ __device__ __forceinline__ void controller_reverse_4w(const DevTopo& T, const De
     const int ni = T.widths[l], no = T.widths[l + 1];
     const float* Wn = D.Wn + T.w_off[l];
     if (l > 0) {
-      dense_bwd(Wn, ni, no, cur, act[l], nxt, true, false, 8 * warp, 32);
+      dense_bwd(Wn, ni, no, cur, act[l], nxt, true, false, 8 * warp, 8 * blk_nw());
       cta_sync();
-      for (int k = warp; k < ni; k += 4) del[l - 1][k] = nxt[k];
+      for (int k = warp; k < ni; k += blk_nw()) del[l - 1][k] = nxt[k];
       const SL tmp = cur;
       cur = nxt;
       nxt = tmp;
     } else {
-      dense_bwd(Wn, ni, no, cur, act[0], sbar, false, false, 8 * warp, 32);
+      dense_bwd(Wn, ni, no, cur, act[0], sbar, false, false, 8 * warp, 8 * blk_nw());
     }
   }
   if (T.skip)
-    dense_bwd(D.Wn + T.w_off[L], T.widths[0], T.widths[L], del[L - 1], act[0], sbar, false, true, 8 * warp, 32);
+    dense_bwd(D.Wn + T.w_off[L], T.widths[0], T.widths[L], del[L - 1], act[0], sbar, false, true, 8 * warp, 8 * blk_nw());
 }
 
 // ------------------------------------------------------------------------------ one step
@@ -1132,13 +1132,13 @@ __device__ __forceinline__ void controller_reverse_4w(const DevTopo& T, const De
 __device__ __forceinline__ void rev_prefetch_step(const DevTopo& T, const DevPtrs& D, int t, int ts, const float* x) {
   const int Bp = T.Bp, nf = 18 * T.nb, base = blockIdx.x * 32;
   if (threadIdx.x < 32) prefetch_record_l2(T, tape_step(T, D, ts).rec);
-  for (int f = threadIdx.x; f < nf; f += 128) prefetch_l2(x + (size_t)f * Bp + base);
+  for (int f = threadIdx.x; f < nf; f += blockDim.x) prefetch_l2(x + (size_t)f * Bp + base);
   // the controller's activation rows (its delta rows are written, not read, by the reverse)
   if (T.n_layers == 0 || T.ext_ctrl) return;
   const size_t N = (size_t)T.horizon * Bp;
   const float* d = D.dump + (size_t)t * Bp + base;
   for (int l = 0; l <= T.n_layers; ++l)
-    for (int r = threadIdx.x; r < T.widths[l]; r += 128) prefetch_l2(d + (size_t)(T.dump_act[l] + r) * N);
+    for (int r = threadIdx.x; r < T.widths[l]; r += blockDim.x) prefetch_l2(d + (size_t)(T.dump_act[l] + r) * N);
 }
 
 // Reverse of step t from its tape slot ts (every warp calls; ends after a CTA barrier). C.XB holds the
@@ -1149,32 +1149,32 @@ __device__ __forceinline__ void blk_reverse_step(const DevTopo& T, const DevPtrs
                                                  const float* x_t, const float* x_t1, bool load_x1, int warp) {
   const int i = C.i, Bp = T.Bp, nf = 18 * T.nb, lane = threadIdx.x & 31;
   const size_t N = (size_t)T.horizon * Bp, n = (size_t)t * Bp + i;
-  const uint32_t mine = 0x11111111u << warp;
+  const uint32_t mine = blk_mine(warp);
   const SL& S = C.S;
   const TapeStep tp = tape_step(T, D, ts);
   const LaneT<SL> L{S, C.P, S, i};
   const BLaneT<SL> Bl{L, C.X, C.G, GC{tp.vminus, 32}};
   rev_stage_first(T, tp);
   if (load_x1)
-    for (int f = warp; f < nf; f += 4) C.X[f] = x_t1[(size_t)f * Bp + i];
+    for (int f = warp; f < nf; f += blk_nw()) C.X[f] = x_t1[(size_t)f * Bp + i];
   if (T.grad_decay != 1.f) {  // section 3.2: the adjoint from later steps shrinks by alpha per step
-    for (int f = warp; f < nf; f += 4) C.XB[f] *= T.grad_decay;
+    for (int f = warp; f < nf; f += blk_nw()) C.XB[f] *= T.grad_decay;
     if (warp == 0)
       for (int k = 0; k < T.n_rec; ++k) S[T.sm_hb + k] *= T.grad_decay;  // and so does h's
   }
   cta_sync();
   // loss term (by the loss body's warp) and integrator, x_{t+1} on chip
-  if ((T.loss_body & 3) == warp) loss_reverse(T, Bl, C.X, C.XB, loss_weight(T, t + 1, D.hz[i]) * C.dl);
+  if ((T.loss_body & (blk_nw() - 1)) == warp) loss_reverse(T, Bl, C.X, C.XB, loss_weight(T, t + 1, D.hz[i]) * C.dl);
   integrate_reverse(T, GL{const_cast<float*>(x_t) + i, Bp}, C.X, C.XB, C.VB, mine);
   // x_t on chip, body by body (no other warp reads a body's x_{t+1}); accumulators zeroed
-  for (int b = warp; b < T.nb; b += 4) {
+  for (int b = warp; b < T.nb; b += blk_nw()) {
 #pragma unroll
     for (int f = 0; f < 18; ++f) C.X[18 * b + f] = x_t[(size_t)(18 * b + f) * Bp + i];
     S[T.sm_invmb + b] = 0.f;
 #pragma unroll
     for (int q = 0; q < 6; ++q) S[T.sm_iinvb + 6 * b + q] = 0.f;
   }
-  for (int s = warp; s < T.nslots; s += 4) S[T.sm_lam + s] = 0.f;  // impulse adjoints
+  for (int s = warp; s < T.nslots; s += blk_nw()) S[T.sm_lam + s] = 0.f;  // impulse adjoints
   inverse_inertia(T, L, C.X, mine);
   cta_sync();
   // the step's records, re-formed bit for bit
@@ -1183,25 +1183,25 @@ __device__ __forceinline__ void blk_reverse_step(const DevTopo& T, const DevPtrs
   const GW au = T.ext_ctrl ? GW{D.u_ext + n * T.ext_nop, 1} : GW{D.dump + (size_t)T.dump_act[u] * N + n, N};
   servo_targets(T, L, au, mine);
   blk_assemble<false>(T, S, C.P, C.X, VelTape{GS{tp.vminus}}, nullptr, warp);
-  for (int j = warp; j < T.nj; j += 4)
+  for (int j = warp; j < T.nj; j += blk_nw())
     for (int q = 0; q < JA_N; ++q) joint_rec(T, S, j)[JR_N + q] = 0.f;
-  for (int c = warp; c < T.ns; c += 4)
+  for (int c = warp; c < T.ns; c += blk_nw())
     for (int q = 0; q < CA_N; ++q) contact_rec(T, S, c)[CR_N + q] = 0.f;
-  for (int c = warp; c < T.np; c += 4)
+  for (int c = warp; c < T.np; c += blk_nw())
     for (int q = 0; q < PA_N; ++q) pair_rec(T, S, c)[PR_N + q] = 0.f;
   cta_sync();
   blk_stream(T, warp, true);
   blk_sweeps_rev(T, S, tp, warp);
   const bool ws = T.ws != 0;
-  for (int j = warp; j < T.nj; j += 4) joint_reverse(T, C, tp, ws, j);
-  for (int q = warp; q < T.ns; q += 4) contact_reverse(T, C, tp, ws, q);
-  for (int p = warp; p < T.np; p += 4) pair_reverse(T, C, tp, ws, p);
+  for (int j = warp; j < T.nj; j += blk_nw()) joint_reverse(T, C, tp, ws, j);
+  for (int q = warp; q < T.ns; q += blk_nw()) contact_reverse(T, C, tp, ws, q);
+  for (int p = warp; p < T.np; p += blk_nw()) pair_reverse(T, C, tp, ws, p);
   // servo targets: the joint's warp has its adjoint
   const SL zb = S.at(T.sm_zb);
   const int nout = T.n_layers > 0 ? T.widths[T.n_layers] : 0;
   for (int m = 0; m < T.n_motors; ++m) {
     const int j = T.motor_joint[m];
-    if ((j & 3) != warp) continue;
+    if ((j & (blk_nw() - 1)) != warp) continue;
     const float g = S[T.sm_wstb + j], br = S[T.sm_wbr + j];
     float ub = 0.f;
     if (br == 0.f) {
@@ -1224,12 +1224,12 @@ __device__ __forceinline__ void blk_reverse_step(const DevTopo& T, const DevPtrs
     }
   }
   cta_sync();
-  for (int b = warp; b < T.nb; b += 4) body_reverse(T, C, b);
+  for (int b = warp; b < T.nb; b += blk_nw()) body_reverse(T, C, b);
   if (T.ext_ctrl) {
     // wide controller: the output adjoint goes to the batched products; the features' adjoint comes
     // back into the next launch
     float* ubx = D.ub_ext + (size_t)i * 16;
-    for (int o = warp; o < 16; o += 4) {
+    for (int o = warp; o < 16; o += blk_nw()) {
       ubx[o] = o < nout ? zb[o] : 0.f;
       if (o < nout) D.dump[(size_t)(T.dump_del[T.n_layers - 1] + o) * N + n] = zb[o];  // output layer's delta
     }
@@ -1240,7 +1240,7 @@ __device__ __forceinline__ void blk_reverse_step(const DevTopo& T, const DevPtrs
       act[l] = GW{D.dump + (size_t)T.dump_act[l] * N + n, N};
       del[l] = GW{D.dump + (size_t)T.dump_del[l] * N + n, N};
     }
-    for (int o = warp; o < nout; o += 4) del[T.n_layers - 1][o] = zb[o];
+    for (int o = warp; o < nout; o += blk_nw()) del[T.n_layers - 1][o] = zb[o];
     cta_sync();  // the packages have been read: the controller's buffers may overwrite them
     const SL sbar = S.at(T.sm_sbar);
     if (T.mlp_tc) {
@@ -1249,9 +1249,9 @@ __device__ __forceinline__ void blk_reverse_step(const DevTopo& T, const DevPtrs
       int maxw = 1;
       for (int l = 0; l <= T.n_layers; ++l) maxw = max(maxw, T.widths[l]);
       const SL z1 = S.at(T.sm_hbuf), z2 = S.at(T.sm_hbuf + maxw);
-      for (int o = warp; o < nout; o += 4) z1[o] = zb[o];
+      for (int o = warp; o < nout; o += blk_nw()) z1[o] = zb[o];
       cta_sync();
-      controller_reverse_4w(T, D, act, del, z1, z2, sbar, warp);
+      controller_reverse_nw(T, D, act, del, z1, z2, sbar, warp);
     }
     cta_sync();
     features_reverse_joints(T, S, sbar, warp);
@@ -1263,9 +1263,9 @@ __device__ __forceinline__ void blk_reverse_step(const DevTopo& T, const DevPtrs
   } else {
     cta_sync();
   }
-  for (int j = warp; j < T.nj; j += 4) hinge_reverse_item(T, C, j);
+  for (int j = warp; j < T.nj; j += blk_nw()) hinge_reverse_item(T, C, j);
   cta_sync();
-  for (int b = warp; b < T.nb; b += 4) hinge_reverse_body(T, C, b);
+  for (int b = warp; b < T.nb; b += blk_nw()) hinge_reverse_body(T, C, b);
   cta_sync();
 }
 
@@ -1287,12 +1287,12 @@ __device__ __forceinline__ RevCtx rev_ctx(const DevTopo& T, const DevPtrs& D, fl
 
 // Reverse mode through the last rollout, whole tape: every step from it, last first.
 template <class Q>
-__global__ void __launch_bounds__(128, 1) k_backward_blk(const __grid_constant__ DevTopo T, const __grid_constant__ DevPtrs D) {
+__global__ void __launch_bounds__(32 * Q::NW, 1) k_backward_blk(const __grid_constant__ DevTopo T, const __grid_constant__ DevPtrs D) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int i = blockIdx.x * 32 + lane, Bp = T.Bp, nf = 18 * T.nb;
   const RevCtx C = rev_ctx(T, D, g_smem + lane, i);
   blk_load(T, D);
-  for (int f = warp; f < nf; f += 4) C.XB[f] = 0.f;
+  for (int f = warp; f < nf; f += blk_nw()) C.XB[f] = 0.f;
   if (warp == 0)
     for (int k = 0; k < T.n_rec; ++k) C.S[T.sm_hb + k] = 0.f;  // no adjoint reaches h^T
   const size_t sb = (size_t)nf * Bp;
@@ -1306,13 +1306,13 @@ __global__ void __launch_bounds__(128, 1) k_backward_blk(const __grid_constant__
     if (warp == 0) blk_loss_initial_reverse(T, D, C);
     cta_sync();
   }
-  for (int f = warp; f < nf; f += 4) D.grad_state0[(size_t)f * Bp + i] = C.XB[f];
+  for (int f = warp; f < nf; f += blk_nw()) D.grad_state0[(size_t)f * Bp + i] = C.XB[f];
 }
 
 // Reverse mode from checkpoints: each segment (last first) is stepped again with its tape (layout Tf),
 // then reversed (layout T). The state adjoint and that of h lie in front of both layouts.
 template <class Q>
-__global__ void __launch_bounds__(128, 1) k_backward_seg_blk(const __grid_constant__ DevTopo T, const __grid_constant__ DevTopo Tf,
+__global__ void __launch_bounds__(32 * Q::NW, 1) k_backward_seg_blk(const __grid_constant__ DevTopo T, const __grid_constant__ DevTopo Tf,
                                                              const __grid_constant__ DevPtrs D) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int i = blockIdx.x * 32 + lane, Bp = T.Bp, nf = 18 * T.nb;
@@ -1322,7 +1322,7 @@ __global__ void __launch_bounds__(128, 1) k_backward_seg_blk(const __grid_consta
   const SL X{sm + Tf.sm_x * 32};
   SL act[DPK_MAXL + 1];
   for (int l = 0; l <= DPK_MAXL; ++l) act[l] = SL{sm + Tf.sm_act[l] * 32};
-  for (int f = warp; f < nf; f += 4) C.XB[f] = 0.f;
+  for (int f = warp; f < nf; f += blk_nw()) C.XB[f] = 0.f;
   if (warp == 0)
     for (int k = 0; k < T.n_rec; ++k) C.S[T.sm_hb + k] = 0.f;  // no adjoint reaches h^T
   const size_t sb = (size_t)nf * Bp;
@@ -1331,18 +1331,18 @@ __global__ void __launch_bounds__(128, 1) k_backward_seg_blk(const __grid_consta
     const int ta = c * K, tb = min(Tw, ta + K);
     cta_sync();  // the layouts share their memory
     blk_load(Tf, D);
-    for (int f = warp; f < nf; f += 4) X[f] = D.ckpt[(size_t)c * sb + (size_t)f * Bp + i];
+    for (int f = warp; f < nf; f += blk_nw()) X[f] = D.ckpt[(size_t)c * sb + (size_t)f * Bp + i];
     if (T.ws)  // the previous impulses the segment's first step started from
-      for (int s = warp; s < T.nslots; s += 4) L.S[Tf.sm_lam + s] = D.ckpt_lam[((size_t)c * T.nslots + s) * Bp + i];
+      for (int s = warp; s < T.nslots; s += blk_nw()) L.S[Tf.sm_lam + s] = D.ckpt_lam[((size_t)c * T.nslots + s) * Bp + i];
     if (warp == 0)
       for (int k = 0; k < T.n_rec; ++k)  // the controller's recurrent state at the segment's start
         L.S[Tf.sm_h + k] = D.ckpt_h[((size_t)c * T.n_rec + k) * Bp + i];
     cta_sync();
     for (int t = ta; t < tb; ++t) {
-      for (int f = warp; f < nf; f += 4) D.seg[(size_t)(t - ta) * sb + (size_t)f * Bp + i] = X[f];
+      for (int f = warp; f < nf; f += blk_nw()) D.seg[(size_t)(t - ta) * sb + (size_t)f * Bp + i] = X[f];
       blk_step<true, Q>(Tf, D, L, X, act, t, t - ta, nullptr, T.n_layers > 0 ? D.dump + (size_t)t * Bp + i : nullptr, warp);
     }
-    for (int f = warp; f < nf; f += 4) D.seg[(size_t)(tb - ta) * sb + (size_t)f * Bp + i] = X[f];
+    for (int f = warp; f < nf; f += blk_nw()) D.seg[(size_t)(tb - ta) * sb + (size_t)f * Bp + i] = X[f];
     __threadfence();  // the reverse reads the tape through L2
     cta_sync();
     blk_load(T, D);
@@ -1355,13 +1355,13 @@ __global__ void __launch_bounds__(128, 1) k_backward_seg_blk(const __grid_consta
     if (warp == 0) blk_loss_initial_reverse(T, D, C);
     cta_sync();
   }
-  for (int f = warp; f < nf; f += 4) D.grad_state0[(size_t)f * Bp + i] = C.XB[f];
+  for (int f = warp; f < nf; f += blk_nw()) D.grad_state0[(size_t)f * Bp + i] = C.XB[f];
 }
 
 // The wide controller's per-step reverse launches (see k_backward_ext in dp_steps.cuh): the feature
 // adjoint of x_{t+1}, then the reverse of step t.
 template <class Q>
-__global__ void __launch_bounds__(128, 1) k_backward_ext_blk(const __grid_constant__ DevTopo T, const __grid_constant__ DevPtrs D,
+__global__ void __launch_bounds__(32 * Q::NW, 1) k_backward_ext_blk(const __grid_constant__ DevTopo T, const __grid_constant__ DevPtrs D,
                                                              int t) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int i = blockIdx.x * 32 + lane, Bp = T.Bp, nf = 18 * T.nb;
@@ -1370,26 +1370,26 @@ __global__ void __launch_bounds__(128, 1) k_backward_ext_blk(const __grid_consta
   if (t >= Tw) return;                // this group's rollout ended before step t
   blk_load(T, D);
   const size_t sb = (size_t)nf * Bp;
-  const uint32_t mine = 0x11111111u << warp;
-  for (int f = warp; f < nf; f += 4) C.XB[f] = D.grad_state0[(size_t)f * Bp + i];
+  const uint32_t mine = blk_mine(warp);
+  for (int f = warp; f < nf; f += blk_nw()) C.XB[f] = D.grad_state0[(size_t)f * Bp + i];
   const int tn = t + 1;
   if (t > 0) rev_prefetch_step(T, D, t, t, D.ckpt + (size_t)t * sb);
   if (tn < Tw) {  // adjoint of the features of x_{t+1}
     const float* xs = D.ckpt + (size_t)tn * sb;
-    for (int f = warp; f < nf; f += 4) C.X[f] = xs[(size_t)f * Bp + i];
+    for (int f = warp; f < nf; f += blk_nw()) C.X[f] = xs[(size_t)f * Bp + i];
     cta_sync();
     const LaneT<SL> L{C.S, C.P, C.S, i};
     hinge_kinematics(T, L, C.X, mine);
-    for (int j = warp; j < T.nj; j += 4) {
+    for (int j = warp; j < T.nj; j += blk_nw()) {
       C.S[T.sm_thb + j] = C.S[T.sm_thdb + j] = 0.f;
       C.S.s3(T.sm_uab + 3 * j, f3(0.f, 0.f, 0.f));
     }
     const GC sbar{D.sbar_ext + (size_t)i * T.ext_k0p, 1};
     features_reverse_joints(T, C.S, sbar, warp);
     if (warp == 3) features_reverse_rest(T, C, sbar);
-    for (int j = warp; j < T.nj; j += 4) hinge_reverse_item(T, C, j);
+    for (int j = warp; j < T.nj; j += blk_nw()) hinge_reverse_item(T, C, j);
     cta_sync();
-    for (int b = warp; b < T.nb; b += 4) hinge_reverse_body(T, C, b);
+    for (int b = warp; b < T.nb; b += blk_nw()) hinge_reverse_body(T, C, b);
     cta_sync();
   }
   if (t >= 0) {
@@ -1398,7 +1398,7 @@ __global__ void __launch_bounds__(128, 1) k_backward_ext_blk(const __grid_consta
     if (warp == 0 && T.loss_kind == 3) blk_loss_initial_reverse(T, D, C);
     cta_sync();
   }
-  for (int f = warp; f < nf; f += 4) D.grad_state0[(size_t)f * Bp + i] = C.XB[f];
+  for (int f = warp; f < nf; f += blk_nw()) D.grad_state0[(size_t)f * Bp + i] = C.XB[f];
 }
 
 template <class Q>
@@ -1408,12 +1408,12 @@ static cudaError_t launch_backward_blk_t(const DevTopo& T, const DevTopo& Ts, co
     const size_t smem = (size_t)T.sm_total * 128;
     e = cudaFuncSetAttribute(k_backward_blk<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_backward_blk<Q><<<T.Bp / 32, 128, smem, s>>>(T, D);
+    k_backward_blk<Q><<<T.Bp / 32, 32 * T.blk_nw, smem, s>>>(T, D);
   } else {
     const size_t smem = (size_t)(T.sm_total > Ts.sm_total ? T.sm_total : Ts.sm_total) * 128;
     e = cudaFuncSetAttribute(k_backward_seg_blk<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_backward_seg_blk<Q><<<T.Bp / 32, 128, smem, s>>>(T, Ts, D);
+    k_backward_seg_blk<Q><<<T.Bp / 32, 32 * T.blk_nw, smem, s>>>(T, Ts, D);
   }
   return cudaGetLastError();
 }

@@ -7,17 +7,17 @@
 // SEQ the parent's share of J v is one chain of multiply-adds from the linear velocity on and the
 // linear update is fused (the quadruped's and the arms' worlds); without it the angular product is
 // summed by itself and the linear impulse is rounded first (every other robot). Each keeps the
-// rounding its worlds have always had.
+// rounding its worlds have always had. NW: the warps of a CTA (blk_warps in dp_plan.cu).
 struct BlkQuad {
-  static constexpr int CTRL_H = 128;
+  static constexpr int CTRL_H = 128, NW = 8;
   static constexpr bool SEQ = true;
 };
 struct BlkArm {
-  static constexpr int CTRL_H = 256;
+  static constexpr int CTRL_H = 256, NW = 8;
   static constexpr bool SEQ = true;
 };
 struct BlkDyn {
-  static constexpr int CTRL_H = 0;
+  static constexpr int CTRL_H = 0, NW = 4;
   static constexpr bool SEQ = false;
 };
 
@@ -66,14 +66,14 @@ __device__ __forceinline__ void store_hidden(const float (&acc)[NT][4], int mt, 
 // order. in: the features, out: the outputs, dump: the step's dump column of lane 0 (or NULL).
 // Called by every warp with the features complete; the outputs are complete after the caller's
 // next barrier.
-template <int H>
-__device__ __forceinline__ void ctrl_forward_4w(const DevTopo& T, const DevPtrs& D, const SL& in, const SL& out,
+template <int H, int NW>
+__device__ __forceinline__ void ctrl_forward_nw(const DevTopo& T, const DevPtrs& D, const SL& in, const SL& out,
                                                 float* dump, int warp) {
-  constexpr int NT = H / 32, KT = H / 16, KT0 = CTRL_TC_KP0 / 16;
+  constexpr int NT = H / (8 * NW), KT = H / 16, KT0 = CTRL_TC_KP0 / 16;
   constexpr CtrlTCLayout Lw = ctrl_tc_layout(H, H);
   const __nv_bfloat16* Wc = D.Wtc;
   const size_t N = (size_t)T.horizon * T.Bp;
-  const int n1 = warp * (H / 4), K0 = T.widths[0], no = T.widths[3];
+  const int n1 = warp * (H / NW), K0 = T.widths[0], no = T.widths[3];
   __nv_bfloat16 *h1 = ctrl_hidden<H>(T, 1), *h2 = ctrl_hidden<H>(T, 2);
   {
     float acc[2][NT][4];
@@ -137,35 +137,35 @@ __device__ __forceinline__ void ctrl_forward_4w(const DevTopo& T, const DevPtrs&
     store_c<2>(acc, warp, 0, no, [&](int f, int r, float v) { out.lane_at(f, r) = v; });
   }
 }
-template <int H>
-__device__ __noinline__ void ctrl_forward_4w_call(const DevTopo& T, const DevPtrs& D, SL in, SL out, float* dump, int warp) {
-  ctrl_forward_4w<H>(T, D, in, out, dump, warp);
+template <int H, int NW>
+__device__ __noinline__ void ctrl_forward_nw_call(const DevTopo& T, const DevPtrs& D, SL in, SL out, float* dump, int warp) {
+  ctrl_forward_nw<H, NW>(T, D, in, out, dump, warp);
 }
 template <class Q>
 __device__ __forceinline__ void ctrl_forward_blk(const DevTopo& T, const DevPtrs& D, const SL& in, const SL& out,
                                                  float* dump, int warp) {
   if constexpr (Q::CTRL_H == 128) {
-    ctrl_forward_4w<128>(T, D, in, out, dump, warp);
+    ctrl_forward_nw<128, Q::NW>(T, D, in, out, dump, warp);
   } else if constexpr (Q::CTRL_H == 256) {
-    ctrl_forward_4w_call<256>(T, D, in, out, dump, warp);
+    ctrl_forward_nw_call<256, Q::NW>(T, D, in, out, dump, warp);
   } else {
-    if (T.widths[1] == 64) ctrl_forward_4w_call<64>(T, D, in, out, dump, warp);
-    else if (T.widths[1] == 128) ctrl_forward_4w_call<128>(T, D, in, out, dump, warp);
-    else ctrl_forward_4w_call<256>(T, D, in, out, dump, warp);
+    if (T.widths[1] == 64) ctrl_forward_nw_call<64, Q::NW>(T, D, in, out, dump, warp);
+    else if (T.widths[1] == 128) ctrl_forward_nw_call<128, Q::NW>(T, D, in, out, dump, warp);
+    else ctrl_forward_nw_call<256, Q::NW>(T, D, in, out, dump, warp);
   }
 }
 
 // The fp32-arithmetic controller on the four warps: 8 outputs of a layer per warp and pass.
-__device__ __forceinline__ void controller_forward_4w(const DevTopo& T, const DevPtrs& D, const SL* act, int warp) {
+__device__ __forceinline__ void controller_forward_nw(const DevTopo& T, const DevPtrs& D, const SL* act, int warp) {
   for (int l = 0; l < T.n_layers; ++l) {
     dense_fwd(D.Wt + T.w_off[l], D.bias + T.w_off[l], T.widths[l], T.widths[l + 1], act[l], act[l + 1],
-              l + 1 < T.n_layers, false, T.ctrl_round != 0, 8 * warp, 32);
+              l + 1 < T.n_layers, false, T.ctrl_round != 0, 8 * warp, 8 * blk_nw());
     if (l + 1 < T.n_layers) cta_sync();
   }
   if (T.skip) {  // a warp adds to the outputs it wrote
     const int l = T.n_layers;
     dense_fwd(D.Wt + T.w_off[l], D.bias + T.w_off[l], T.widths[0], T.widths[l], act[0], act[l], false, true, false,
-              8 * warp, 32);
+              8 * warp, 8 * blk_nw());
   }
 }
 
@@ -178,14 +178,14 @@ __device__ __forceinline__ void blk_features(const DevTopo& T, const DevPtrs& D,
   if (T.features & 1) {
     for (int m = 0; m < T.n_motors; ++m) {
       const int j = T.motor_joint[m];
-      if ((j & 3) == warp) act0[k + m] = qz(T, S[T.sm_th + j]);
+      if ((j & (blk_nw() - 1)) == warp) act0[k + m] = qz(T, S[T.sm_th + j]);
     }
     k += T.n_motors;
   }
   if (T.features & 2) {
     for (int m = 0; m < T.n_motors; ++m) {
       const int j = T.motor_joint[m];
-      if ((j & 3) == warp) act0[k + m] = qz(T, S[T.sm_thd + j]);
+      if ((j & (blk_nw() - 1)) == warp) act0[k + m] = qz(T, S[T.sm_thd + j]);
     }
     k += T.n_motors;
   }
@@ -225,7 +225,7 @@ __device__ __forceinline__ void blk_features(const DevTopo& T, const DevPtrs& D,
 // the previous step with, projected on the rows' bounds; limits start cold.
 __device__ __forceinline__ void blk_damped_start(const DevTopo& T, const SL& S, int warp) {
   const SL lam = S.at(T.sm_lam);
-  for (int j = warp; j < T.nj; j += 4) {
+  for (int j = warp; j < T.nj; j += blk_nw()) {
     const SL R = joint_rec(T, S, j);
     const int s0 = T.jslot[j], n = T.jtype[j] == 1 ? 5 : 3;
     for (int k = 0; k < n; ++k) lam[s0 + k] = R[JF_ME + k] != 0.f ? T.ws_alpha * lam[s0 + k] : 0.f;
@@ -236,7 +236,7 @@ __device__ __forceinline__ void blk_damped_start(const DevTopo& T, const SL& S, 
       lam[s] = fminf(fmaxf(y, -hi), hi);
     }
   }
-  for (int c = warp; c < T.ns + T.np; c += 4) {
+  for (int c = warp; c < T.ns + T.np; c += blk_nw()) {
     const bool pair = c >= T.ns;
     const SL R = pair ? pair_rec(T, S, c - T.ns) : contact_rec(T, S, c);
     const int s0 = T.cslot + 3 * c;
@@ -256,7 +256,7 @@ __device__ __forceinline__ void blk_apply_start(const DevTopo& T, const SL& S, c
   const SL lam = S.at(T.sm_lam);
   const uint8_t* first = blk_bytes(T) + T.blk_inc0;
   const uint8_t* inc = blk_bytes(T) + T.blk_inc;
-  for (int b = warp; b < T.nb; b += 4) {
+  for (int b = warp; b < T.nb; b += blk_nw()) {
     float3 v = X.v3(18 * b + 12), w = X.v3(18 * b + 15);
     const float im = S[T.sm_invm + b];
     const int k0 = first[b], k1 = first[b + 1];
@@ -337,9 +337,9 @@ static __device__ __noinline__ void blk_network_start(const DevTopo& T, const De
     if ((c < T.ns ? contact_rec(T, S, c)[CF_ME] : pair_rec(T, S, c - T.ns)[PF_ME]) != 0.f) ++nact;
   const float gn = sqrtf(T.gravity[0] * T.gravity[0] + T.gravity[1] * T.gravity[1] + T.gravity[2] * T.gravity[2]);
   const float share = mtot * gn * T.dt / (float)max(1, nact);
-  const SL F = S.at(T.sm_ws + 19 * warp), Y = S.at(T.sm_ws + 19 * warp + 16), H = S.at(T.sm_ws + 76);
+  const SL F = S.at(T.sm_ws + 19 * warp), Y = S.at(T.sm_ws + 19 * warp + 16), H = S.at(T.sm_ws + 19 * blk_nw());
   const int lane = threadIdx.x & 31;
-  for (int g = warp; g < T.n_wsg; g += 4) {
+  for (int g = warp; g < T.n_wsg; g += blk_nw()) {
     const int type = T.wsg_type[g];
     const int s0 = T.wsg_slot[g][0], s1 = T.wsg_slot[g][1], s2 = T.wsg_slot[g][2];
     const bool contact = type == WSG_GROUND || type == WSG_PAIR;
@@ -427,14 +427,14 @@ static __device__ __noinline__ void blk_network_start(const DevTopo& T, const De
     }
   }
   if (T.ws)
-    for (int j = warp; j < T.nj; j += 4)
+    for (int j = warp; j < T.nj; j += blk_nw())
       if (T.jlim[j] >= 0) lam[T.jlim[j]] = 0.f;  // limits start cold
 }
 
 // Harvest: per reserved group, the network's ideal output (see harvest_finish in dp_forward.cuh).
 static __device__ __noinline__ void blk_harvest_finish(const DevTopo& T, const DevPtrs& D, const SL S, int warp) {
-  const SL H = S.at(T.sm_ws + 76);
-  for (int g = warp; g < T.n_wsg; g += 4) {
+  const SL H = S.at(T.sm_ws + 19 * blk_nw());
+  for (int g = warp; g < T.n_wsg; g += blk_nw()) {
     const int id = __float_as_int(H[g]);
     if (id < 0) continue;
     float* row = D.harvest + (long long)id * 19;
@@ -480,13 +480,13 @@ __device__ __forceinline__ void blk_step(const DevTopo& T, const DevPtrs& D, con
                                          int t, int ts, uint8_t* ao, float* dump_col, int warp) {
   const SL& S = L.S;
   const int Bp = T.Bp, lane = threadIdx.x & 31;
-  const uint32_t mine = 0x11111111u << warp;  // items and bodies k % 4 == warp
+  const uint32_t mine = blk_mine(warp);
   hinge_kinematics(T, L, X, mine);
   const int u = T.n_layers > 0 ? T.n_layers : 0;
   if (T.ext_ctrl) {
     // wide controller: its output for this step was computed between launches
     const float* ue = D.u_ext + ((size_t)t * Bp + L.i) * T.ext_nop;
-    for (int m = warp; m < T.widths[u]; m += 4) act[u][m] = ue[m];
+    for (int m = warp; m < T.widths[u]; m += blk_nw()) act[u][m] = ue[m];
     cta_sync();
   } else if (T.n_layers > 0) {
     blk_features(T, D, L, X, t, act[0], warp);
@@ -494,7 +494,7 @@ __device__ __forceinline__ void blk_step(const DevTopo& T, const DevPtrs& D, con
     if (T.mlp_tc)
       ctrl_forward_blk<Q>(T, D, act[0], act[u], dump_col ? dump_col - lane : nullptr, warp);
     else
-      controller_forward_4w(T, D, act, warp);
+      controller_forward_nw(T, D, act, warp);
     cta_sync();
     if (T.n_rec && warp == 0) {  // h^{t+1} = tanh of the last outputs
       const int base = T.widths[u] - T.n_rec;
@@ -510,7 +510,7 @@ __device__ __forceinline__ void blk_step(const DevTopo& T, const DevPtrs& D, con
       const size_t N = (size_t)T.horizon * Bp;
       for (int l = 0; l <= T.n_layers; ++l) {
         if (T.mlp_tc && l > 0 && l < T.n_layers) continue;  // hidden layers went straight to the dump
-        for (int k = warp; k < T.widths[l]; k += 4) dump_col[(size_t)(T.dump_act[l] + k) * N] = act[l][k];
+        for (int k = warp; k < T.widths[l]; k += blk_nw()) dump_col[(size_t)(T.dump_act[l] + k) * N] = act[l][k];
       }
     }
   } else {
@@ -521,7 +521,7 @@ __device__ __forceinline__ void blk_step(const DevTopo& T, const DevPtrs& D, con
   TapeStep tp{};
   if (TAPE) {
     tp = tape_step(T, D, ts);
-    for (int b = warp; b < T.nb; b += 4)
+    for (int b = warp; b < T.nb; b += blk_nw())
 #pragma unroll
       for (int k = 0; k < 6; ++k) tp.vminus[(6 * b + k) * 32] = X[18 * b + 12 + k];
   }
@@ -530,7 +530,7 @@ __device__ __forceinline__ void blk_step(const DevTopo& T, const DevPtrs& D, con
   const bool net = D.harvest || (T.ws && T.ws_net);
   if (!T.ws) {
     if (!net)  // (the harvest reads the previous impulses first)
-      for (int s = warp; s < T.nslots; s += 4) S[T.sm_lam + s] = 0.f;
+      for (int s = warp; s < T.nslots; s += blk_nw()) S[T.sm_lam + s] = 0.f;
   } else if (!net) {
     blk_damped_start(T, S, warp);
   }
@@ -539,17 +539,17 @@ __device__ __forceinline__ void blk_step(const DevTopo& T, const DevPtrs& D, con
     blk_network_start(T, D, L, X, warp);
     cta_sync();
     if (!T.ws) {
-      for (int s = warp; s < T.nslots; s += 4) S[T.sm_lam + s] = 0.f;
+      for (int s = warp; s < T.nslots; s += blk_nw()) S[T.sm_lam + s] = 0.f;
       cta_sync();
     }
   }
   if (T.ws) {
     blk_apply_start(T, S, X, warp);
     if (TAPE)
-      for (int s = warp; s < T.nslots; s += 4) tp.lam0[s * 32] = S[T.sm_lam + s];
+      for (int s = warp; s < T.nslots; s += blk_nw()) tp.lam0[s * 32] = S[T.sm_lam + s];
   }
   if (TAPE && T.rec_rows)
-    for (int s = warp; s < T.nslots; s += 4) {
+    for (int s = warp; s < T.nslots; s += blk_nw()) {
       const RowRec r = blk_row(T, S, s);
       const GS R = GS{tp.rows + s * RF_N * 32};
       R.s3(RF_LIN, r.lin); R.s3(RF_ANGA, r.angA); R.s3(RF_ANGB, r.angB); R.s3(RF_IA, r.IA); R.s3(RF_IB, r.IB);
@@ -570,7 +570,7 @@ __device__ __forceinline__ void blk_step(const DevTopo& T, const DevPtrs& D, con
 // Rollouts and steps (see k_forward in dp_steps.cuh for rollout's values) on four warps per group of
 // 32 instances, one CTA per group.
 template <bool REC, class Q>
-__global__ void __launch_bounds__(128, 1) k_forward_blk(const __grid_constant__ DevTopo T, const __grid_constant__ DevPtrs D,
+__global__ void __launch_bounds__(32 * Q::NW, 1) k_forward_blk(const __grid_constant__ DevTopo T, const __grid_constant__ DevPtrs D,
                                                         const float* __restrict__ x0, int t0, int nsteps, int rollout) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int i = blockIdx.x * 32 + lane;
@@ -583,8 +583,8 @@ __global__ void __launch_bounds__(128, 1) k_forward_blk(const __grid_constant__ 
   const bool fresh = rollout == 1 || (rollout == 2 && t0 == 0);
   const float* xs = fresh ? x0 : D.state;
   blk_load(T, D);
-  for (int f = warp; f < nf; f += 4) X[f] = xs[(size_t)f * Bp + i];
-  for (int s = warp; s < T.nslots; s += 4) L.S[T.sm_lam + s] = fresh ? 0.f : D.lam_prev[(size_t)s * Bp + i];
+  for (int f = warp; f < nf; f += blk_nw()) X[f] = xs[(size_t)f * Bp + i];
+  for (int s = warp; s < T.nslots; s += blk_nw()) L.S[T.sm_lam + s] = fresh ? 0.f : D.lam_prev[(size_t)s * Bp + i];
   if (warp == 0)
     for (int k = 0; k < T.n_rec; ++k) L.S[T.sm_h + k] = fresh ? 0.f : D.hrec[(size_t)k * Bp + i];
   cta_sync();
@@ -599,14 +599,14 @@ __global__ void __launch_bounds__(128, 1) k_forward_blk(const __grid_constant__ 
     if (rollout) {
       if (t % D.ckpt_every == 0) {
         const size_t c = (size_t)(t / D.ckpt_every);
-        for (int f = warp; f < nf; f += 4) D.ckpt[(c * nf + f) * Bp + i] = X[f];
+        for (int f = warp; f < nf; f += blk_nw()) D.ckpt[(c * nf + f) * Bp + i] = X[f];
         if (D.ckpt_lam)
-          for (int s = warp; s < T.nslots; s += 4) D.ckpt_lam[(c * T.nslots + s) * Bp + i] = L.S[T.sm_lam + s];
+          for (int s = warp; s < T.nslots; s += blk_nw()) D.ckpt_lam[(c * T.nslots + s) * Bp + i] = L.S[T.sm_lam + s];
         if (D.ckpt_h && warp == 0)
           for (int q = 0; q < T.n_rec; ++q) D.ckpt_h[(c * T.n_rec + q) * Bp + i] = L.S[T.sm_h + q];
       }
       if (D.traj && i < B)
-        for (int f = warp; f < nf; f += 4) D.traj[((size_t)t * B + i) * nf + f] = X[f];
+        for (int f = warp; f < nf; f += blk_nw()) D.traj[((size_t)t * B + i) * nf + f] = X[f];
     }
     // the activity log is per rollout step (rollout parts) or per call step (dp_step)
     uint8_t* ao = (D.active && i < B) ? D.active + ((size_t)(rollout == 2 ? t : k) * B + i) * T.nslots : nullptr;
@@ -622,26 +622,26 @@ __global__ void __launch_bounds__(128, 1) k_forward_blk(const __grid_constant__ 
     }
   }
   if (rollout && D.traj && i < B)
-    for (int f = warp; f < nf; f += 4) D.traj[((size_t)(t0 + nrun) * B + i) * nf + f] = X[f];
+    for (int f = warp; f < nf; f += blk_nw()) D.traj[((size_t)(t0 + nrun) * B + i) * nf + f] = X[f];
   if (T.ext_ctrl && t0 + nrun < T.horizon) {
     // wide controller: input features of the next step, bf16 for the products, and the
     // activation dump column for the weight gradient
     const int tn = t0 + nrun;
-    hinge_kinematics(T, L, X, 0x11111111u << warp);
+    hinge_kinematics(T, L, X, blk_mine(warp));
     blk_features(T, D, L, X, tn, act[0], warp);
     cta_sync();
     __nv_bfloat16* sx = D.s_ext + (size_t)i * T.ext_k0p;
-    for (int q = warp; q < T.ext_k0p; q += 4) {
+    for (int q = warp; q < T.ext_k0p; q += blk_nw()) {
       const float v = q < T.widths[0] ? act[0][q] : 0.f;
       sx[q] = __float2bfloat16_rn(v);
       if (REC && q < T.widths[0]) D.dump[(size_t)(T.dump_act[0] + q) * N + (size_t)tn * Bp + i] = v;
     }
   }
-  for (int s = warp; s < T.nslots; s += 4) D.lam_prev[(size_t)s * Bp + i] = L.S[T.sm_lam + s];
+  for (int s = warp; s < T.nslots; s += blk_nw()) D.lam_prev[(size_t)s * Bp + i] = L.S[T.sm_lam + s];
   if (warp == 0)
     for (int q = 0; q < T.n_rec; ++q) D.hrec[(size_t)q * Bp + i] = L.S[T.sm_h + q];
   bool bad = false;
-  for (int f = warp; f < nf; f += 4) {
+  for (int f = warp; f < nf; f += blk_nw()) {
     D.state[(size_t)f * Bp + i] = X[f];
     bad |= !isfinite(X[f]);
   }
@@ -658,6 +658,6 @@ static cudaError_t launch_forward_blk_t(const DevTopo& T, const DevPtrs& D, cons
   const size_t smem = (size_t)T.sm_total * 32 * sizeof(float);
   cudaError_t e = cudaFuncSetAttribute(k_forward_blk<REC, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_forward_blk<REC, Q><<<T.Bp / 32, 128, smem, s>>>(T, D, x0, t0, nsteps, rollout);
+  k_forward_blk<REC, Q><<<T.Bp / 32, 32 * T.blk_nw, smem, s>>>(T, D, x0, t0, nsteps, rollout);
   return cudaGetLastError();
 }

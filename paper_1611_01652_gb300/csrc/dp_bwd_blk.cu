@@ -16,6 +16,6 @@ cudaError_t launch_backward_ext_blk(const DevTopo& T, const DevPtrs& D, int t, c
   const size_t smem = (size_t)T.sm_total * 128;
   cudaError_t e = cudaFuncSetAttribute(k_backward_ext_blk<BlkQuad>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_backward_ext_blk<BlkQuad><<<T.Bp / 32, 128, smem, s>>>(T, D, t);
+  k_backward_ext_blk<BlkQuad><<<T.Bp / 32, 32 * T.blk_nw, smem, s>>>(T, D, t);
   return cudaGetLastError();
 }

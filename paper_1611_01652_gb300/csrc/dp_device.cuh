@@ -89,6 +89,7 @@ struct DevTopo {
   // are scheduled and its records fit on chip; byte offsets in the program's region of shared
   // memory (sm_prog): level table, bodies' item lists (first index per body, entries), live flags,
   // streams; slots of each joint's first linear row, limit row and servo row, and of the contacts
+  int blk_nw;  // warps of a CTA
   int blk, blk_nops, blk_nlev, blk_single, blk_words, blk_bytes_total;
   int blk_lev, blk_inc0, blk_inc, blk_live, blk_stream, blk_stream_len, sm_prog;
   int blk_fwd, blk_bwd;  // 1: rollouts and steps / reverse passes of this world run on the four-warp step

@@ -30,6 +30,9 @@ bool plan_blocks(DevTopo& T, std::vector<int32_t>& blob) {
     if (T.skind[s] == RK_MOTOR) T.jmot[T.sidx[s]] = (int16_t)s;
     if (T.skind[s] >= RK_GN) T.cslot = s;
   }
+  // Warps: eight for the compiled topologies (the quadruped has 8 joints, 9 bodies, 8 contacts; two
+  // warps a scheduler also hide each other's latencies), four for the other robots.
+  const int nw = T.blk_nw = T.topo_id != 0 ? 8 : 4;
   // Blocks: a row joins the block of its item when that block is the last one on every body the
   // row touches (so the block's rows are adjacent for both bodies), else it starts a new block.
   std::vector<Op> ops;
@@ -82,7 +85,7 @@ bool plan_blocks(DevTopo& T, std::vector<int32_t>& blob) {
   // Levels: the ready blocks with the longest remaining chains first, each on the least loaded
   // warp; a block that would make the level longer than its most urgent block waits.
   int done = 0, nlev = 0;
-  std::vector<std::vector<int>> runs[4];
+  std::vector<std::vector<int>> runs[8];
   while (done < n) {
     std::vector<int> ready;
     for (int k = 0; k < n; ++k) {
@@ -92,12 +95,12 @@ bool plan_blocks(DevTopo& T, std::vector<int32_t>& blob) {
       if (ok) ready.push_back(k);
     }
     std::stable_sort(ready.begin(), ready.end(), [&](int x, int y) { return ops[x].path > ops[y].path; });
-    int load[4] = {0, 0, 0, 0}, cnt[4] = {0, 0, 0, 0};
+    int load[8] = {0}, cnt[8] = {0};
     const int cap = std::max(1, ops[ready[0]].weight);
-    for (auto& r : runs) r.emplace_back();
+    for (int g = 0; g < nw; ++g) runs[g].emplace_back();
     for (int k : ready) {
       int w = 0;
-      for (int g = 1; g < 4; ++g)
+      for (int g = 1; g < nw; ++g)
         if (load[g] < load[w] || (load[g] == load[w] && cnt[g] < cnt[w])) w = g;
       if (cnt[w] > 0 && load[w] + ops[k].weight > cap) continue;
       ops[k].level = nlev;
@@ -112,10 +115,10 @@ bool plan_blocks(DevTopo& T, std::vector<int32_t>& blob) {
   // blob: descriptors grouped by warp and level, then the level table (bytes), the bodies' item
   // lists, the live flags and the streams
   std::vector<uint8_t> b;
-  std::vector<uint8_t> lev(4 * (nlev + 1));
+  std::vector<uint8_t> lev(nw * (nlev + 1));
   std::vector<int32_t> desc;
   int pos = 0;
-  for (int w = 0; w < 4; ++w) {
+  for (int w = 0; w < nw; ++w) {
     for (int l = 0; l < nlev; ++l) {
       lev[w * (nlev + 1) + l] = (uint8_t)pos;
       for (int k : runs[w][l]) {
@@ -159,7 +162,7 @@ bool plan_blocks(DevTopo& T, std::vector<int32_t>& blob) {
   T.blk_live = (int)b.size();
   T.blk_stream_len = n + nlev + 2;
   T.blk_stream = T.blk_live + T.nj + T.ns + T.np;
-  T.blk_bytes_total = T.blk_stream + 4 * T.blk_stream_len;
+  T.blk_bytes_total = T.blk_stream + nw * T.blk_stream_len;
   T.blk_nops = n;
   T.blk_nlev = nlev;
   T.blk_single = n == 1;
