@@ -40,6 +40,73 @@ struct GemmEpi {
 
 __device__ __forceinline__ float bf16_round(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
+// The epilogues form every value of a thread's fragments first (fragment_values: the loads of the bias
+// or of the activations' mask, all in flight together) and store them after. Mixed with the stores,
+// each of the 64 mask loads waited for the one before it (the compiler has to assume that a store may
+// change the next load's value), which was most of a reverse product's time.
+// Element k of fragment (mt, nt): row m0 + 16 mt + g (+ 8), column n0 + 8 nt + 2 q (+ 1).
+template <int MT, int NT>
+__device__ __forceinline__ void fragment_values(const GemmEpi& e, int m0, int n0, int M, float (&acc)[MT][NT][4]) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt) {
+    const int n = n0 + nt * 8 + 2 * q;
+    if (e.kind == EPI_BWD_HIDDEN) {
+      float a[MT][4];
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int m = m0 + mt * 16 + g + (k >= 2 ? 8 : 0);
+          a[mt][k] = m < M ? e.mask[(size_t)(e.mask_row + n + (k & 1)) * e.ncol + e.col0 + m] : 0.f;
+        }
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (!(a[mt][k] > 0.f)) acc[mt][nt][k] = 0.f;
+    } else if (e.kind != EPI_BWD_IN) {
+      const float b[2] = {n < e.nvalid ? e.bias[n] : 0.f, n + 1 < e.nvalid ? e.bias[n + 1] : 0.f};
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float v = acc[mt][nt][k] + b[k & 1];
+          acc[mt][nt][k] = e.kind == EPI_FWD_HIDDEN ? bf16_round(fmaxf(v, 0.f)) : (n + (k & 1) < e.nvalid ? v : 0.f);
+        }
+    }
+  }
+}
+template <int MT, int NT>
+__device__ __forceinline__ void fragment_store(const GemmEpi& e, int m0, int n0, int M, const float (&acc)[MT][NT][4]) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+#pragma unroll
+  for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int m = m0 + mt * 16 + g + 8 * h, n = n0 + nt * 8 + 2 * q;
+        if (m >= M) continue;
+        const float v0 = acc[mt][nt][2 * h], v1 = acc[mt][nt][2 * h + 1];
+        const size_t o = (size_t)m * e.ldo + n;  // even, like ldo
+        if (e.kind == EPI_FWD_HIDDEN) {
+          *reinterpret_cast<uint32_t*>(static_cast<__nv_bfloat16*>(e.out) + o) = pack_bf16(v0, v1);
+        } else if (e.kind == EPI_BWD_HIDDEN) {
+          const float h0 = bf16_round(v0), h1 = bf16_round(v1);
+          *reinterpret_cast<uint32_t*>(static_cast<__nv_bfloat16*>(e.out) + o) = pack_bf16(h0, h1);
+          *reinterpret_cast<uint32_t*>(e.out_lo + o) = pack_bf16(v0 - h0, v1 - h1);
+        } else {
+          *reinterpret_cast<float2*>(static_cast<float*>(e.out) + o) = make_float2(v0, v1);
+        }
+        if (e.dump) {
+          float* d = e.dump + (size_t)(e.dump_row + n) * e.ncol + e.col0 + m;
+          if (n < e.nvalid) d[0] = v0;
+          if (n + 1 < e.nvalid) d[e.ncol] = v1;
+        }
+      }
+}
+
 template <int NT, bool AF32>
 __global__ void __launch_bounds__(128) k_ctrl_gemm(const void* __restrict__ Av, int lda,
                                                    const __nv_bfloat16* __restrict__ B, int M, int N, int K,
@@ -56,7 +123,8 @@ __global__ void __launch_bounds__(128) k_ctrl_gemm(const void* __restrict__ Av, 
     for (int b = 0; b < NT; ++b)
 #pragma unroll
       for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.f;
-  for (int kt = 0; kt < K / 16; ++kt) {
+#pragma unroll 8
+  for (int kt = 0; kt < K / 16; ++kt) {  // (unrolled: the loads of eight chunks in flight)
     const int c = kt * 16 + 2 * q;
     uint32_t ah[2][4], al[2][4];
 #pragma unroll
@@ -93,41 +161,18 @@ __global__ void __launch_bounds__(128) k_ctrl_gemm(const void* __restrict__ Av, 
       }
     }
   }
-  // epilogue: element (m, n) of fragment position k: rows g / g+8, columns 2q / 2q+1
-#pragma unroll
-  for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int m = m0 + mt * 16 + g + (k >= 2 ? 8 : 0);
-        const int n = n0 + nt * 8 + 2 * q + (k & 1);
-        float v = acc[mt][nt][k];
-        if (e.kind == EPI_FWD_HIDDEN) {
-          v = bf16_round(fmaxf(v + e.bias[n], 0.f));
-          static_cast<__nv_bfloat16*>(e.out)[(size_t)m * e.ldo + n] = __float2bfloat16_rn(v);
-        } else if (e.kind == EPI_FWD_OUT) {
-          v = n < e.nvalid ? v + e.bias[n] : 0.f;
-          static_cast<float*>(e.out)[(size_t)m * e.ldo + n] = v;
-        } else if (e.kind == EPI_BWD_HIDDEN) {
-          if (!(e.mask[(size_t)(e.mask_row + n) * e.ncol + e.col0 + m] > 0.f)) v = 0.f;
-          const float hi = bf16_round(v);
-          static_cast<__nv_bfloat16*>(e.out)[(size_t)m * e.ldo + n] = __float2bfloat16_rn(hi);
-          e.out_lo[(size_t)m * e.ldo + n] = __float2bfloat16_rn(v - hi);
-        } else {
-          static_cast<float*>(e.out)[(size_t)m * e.ldo + n] = v;
-        }
-        if (e.dump && n < e.nvalid) e.dump[(size_t)(e.dump_row + n) * e.ncol + e.col0 + m] = v;
-      }
+  fragment_values(e, m0, n0, M, acc);
+  fragment_store(e, m0, n0, M, acc);
 }
 
 // ---------------------------------------------------------------------------------------------
 // Tiled products: a CTA of 8 warps computes a 128 x BN tile of C = A B^T; A (bf16, optionally a
 // second bf16 plane holding the low part of a split fp32 operand) and B are staged through
-// shared memory in 32-column k-chunks by cp.async (double buffered, rows past M zero-filled),
+// shared memory in 32-column k-chunks by cp.async (TST buffers, so that a chunk has the time of the
+// two before it to arrive; rows past M zero-filled; one barrier a chunk),
 // fragments are read with ldmatrix from rows padded to 40 halves (80 bytes: the 8 row addresses
 // of an 8x8 matrix fall in 8 different 16-byte bank groups).
-constexpr int TBM = 128, TBK = 32, TLDS = 40;
+constexpr int TBM = 128, TBK = 32, TLDS = 40, TST = 4;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -149,8 +194,8 @@ __global__ void __launch_bounds__(256) k_tc_gemm(const __nv_bfloat16* __restrict
   constexpr int WN = BN / 32, WM = 8 / WN, WTM = TBM / WM, MT = WTM / 16;
   constexpr int APL = TBM * TLDS, BPL = BN * TLDS;  // halves per plane and stage
   extern __shared__ __align__(16) unsigned char tc_smem[];
-  __nv_bfloat16* sA = reinterpret_cast<__nv_bfloat16*>(tc_smem);       // [2][SPLIT+1][APL]
-  __nv_bfloat16* sB = sA + 2 * (SPLIT ? 2 : 1) * APL;                    // [2][BPL]
+  __nv_bfloat16* sA = reinterpret_cast<__nv_bfloat16*>(tc_smem);       // [TST][SPLIT+1][APL]
+  __nv_bfloat16* sB = sA + TST * (SPLIT ? 2 : 1) * APL;                  // [TST][BPL]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, q = lane & 3;
   const int m0 = blockIdx.y * TBM, n0 = blockIdx.x * BN;
@@ -178,16 +223,17 @@ __global__ void __launch_bounds__(256) k_tc_gemm(const __nv_bfloat16* __restrict
 #pragma unroll
       for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.f;
   const int nk = K / TBK;
-  load(0, 0);
+#pragma unroll
+  for (int c = 0; c < TST - 1; ++c) {
+    if (c < nk) load(c, c);
+    else asm volatile("cp.async.commit_group;" ::: "memory");
+  }
   for (int kc = 0; kc < nk; ++kc) {
-    const int buf = kc & 1;
-    if (kc + 1 < nk) {
-      load(kc + 1, buf ^ 1);
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-    } else {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-    }
-    __syncthreads();
+    const int buf = kc % TST;
+    asm volatile("cp.async.wait_group %0;" ::"n"(TST - 2) : "memory");
+    __syncthreads();  // chunk kc has arrived for every thread, and chunk kc - 1 is used up
+    if (kc + TST - 1 < nk) load(kc + TST - 1, (kc + TST - 1) % TST);
+    else asm volatile("cp.async.commit_group;" ::: "memory");
     const __nv_bfloat16* a_hi = sA + (size_t)(buf * (SPLIT ? 2 : 1)) * APL;
     const __nv_bfloat16* b_s = sB + (size_t)buf * BPL;
 #pragma unroll
@@ -212,37 +258,15 @@ __global__ void __launch_bounds__(256) k_tc_gemm(const __nv_bfloat16* __restrict
         }
       }
     }
-    __syncthreads();
   }
-#pragma unroll
-  for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int m = m0 + wr + mt * 16 + g + (k >= 2 ? 8 : 0);
-        const int n = n0 + wc + nt * 8 + 2 * q + (k & 1);
-        if (m >= M) continue;
-        float v = acc[mt][nt][k];
-        if (e.kind == EPI_FWD_HIDDEN) {
-          v = bf16_round(fmaxf(v + e.bias[n], 0.f));
-          static_cast<__nv_bfloat16*>(e.out)[(size_t)m * e.ldo + n] = __float2bfloat16_rn(v);
-        } else if (e.kind == EPI_BWD_HIDDEN) {
-          if (!(e.mask[(size_t)(e.mask_row + n) * e.ncol + e.col0 + m] > 0.f)) v = 0.f;
-          const float hi = bf16_round(v);
-          static_cast<__nv_bfloat16*>(e.out)[(size_t)m * e.ldo + n] = __float2bfloat16_rn(hi);
-          e.out_lo[(size_t)m * e.ldo + n] = __float2bfloat16_rn(v - hi);
-        } else {
-          static_cast<float*>(e.out)[(size_t)m * e.ldo + n] = v;
-        }
-        if (e.dump) e.dump[(size_t)(e.dump_row + n) * e.ncol + e.col0 + m] = v;
-      }
+  fragment_values(e, m0 + wr, n0 + wc, M, acc);
+  fragment_store(e, m0 + wr, n0 + wc, M, acc);
 }
 
 template <int BN, bool SPLIT>
 cudaError_t tc_gemm(const __nv_bfloat16* Ahi, const __nv_bfloat16* Alo, const __nv_bfloat16* B, int M, int N, int K,
                     const GemmEpi& e, cudaStream_t s) {
-  const int smem = (2 * (SPLIT ? 2 : 1) * TBM * TLDS + 2 * BN * TLDS) * (int)sizeof(__nv_bfloat16);
+  const int smem = TST * ((SPLIT ? 2 : 1) * TBM * TLDS + BN * TLDS) * (int)sizeof(__nv_bfloat16);
   cudaError_t r = cudaFuncSetAttribute(k_tc_gemm<BN, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (r != cudaSuccess) return r;
   dim3 grid(N / BN, (M + TBM - 1) / TBM);
