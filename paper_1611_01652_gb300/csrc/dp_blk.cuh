@@ -487,10 +487,12 @@ __device__ __forceinline__ void lin_sub(float& v, float dl, float im) {
 // world). Everything a block reads from the record is loaded before its first row and every result
 // is stored after its last one: a store between the rows would keep the loads of the next row behind
 // it, and each row would wait for shared memory (some 30 cycles) besides its own chain of products.
-template <bool TAPE, bool SEQ, bool FULL>
+// ready() meets the barrier of the level before and loads the velocities: all that only this block
+// changes (its record, its impulses) is loaded ahead of it, while the warp would wait there.
+template <bool TAPE, bool SEQ, bool FULL, class RD>
 __device__ __forceinline__ void joint_rows(const DevTopo& T, const SL& S, const TapeStep& tp, int it, const BlkOp& op,
                                            const SL& R, float ima, float imb, float3& va, float3& wa, float3& vb,
-                                           float3& wb) {
+                                           float3& wb, const RD& ready) {
   const int mask = FULL ? 31 : op.mask(), s0 = op.slot();
   const float3 ra = R.v3(JF_RA), rb = R.v3(JF_RB);
   float lam[5], me[5], bi[5];
@@ -505,6 +507,7 @@ __device__ __forceinline__ void joint_rows(const DevTopo& T, const SL& S, const 
       IB[k] = R.v3(k < 3 ? JF_IBL + 3 * k : JF_IBT + 3 * (k - 3));
       if (k >= 3) t[k - 3] = R.v3(JF_T + 3 * (k - 3));
     }
+  ready();
   int br;
   auto lin = [&](auto KI) {
     constexpr int k = decltype(KI)::value;
@@ -532,9 +535,9 @@ __device__ __forceinline__ void joint_rows(const DevTopo& T, const SL& S, const 
   for (int k = 0; k < 5; ++k)
     if (mask >> k & 1) row_store<TAPE, true>(T, S, tp, it, s0 + k, lam[k], 0);
 }
-template <bool TAPE>
+template <bool TAPE, class RD>
 __device__ __forceinline__ void hinge_row(const DevTopo& T, const SL& S, const TapeStep& tp, int it, const BlkOp& op,
-                                          const SL& R, float3& wa, float3& wb) {
+                                          const SL& R, float3& wa, float3& wb, const RD& ready) {
   const bool lim = op.type() == BT_LIMIT;
   const int m = lim ? 5 : 6, s = op.slot();
   const float sg = lim ? R[JF_LS] : 1.f;
@@ -544,6 +547,7 @@ __device__ __forceinline__ void hinge_row(const DevTopo& T, const SL& S, const T
   const float me = R[JF_ME + m], bi = R[JF_BI + m];
   const float hi = lim ? __int_as_float(0x7f800000) : R[JF_BND], lo = lim ? 0.f : -hi;
   const float3 IA = -(sg * R.v3(JF_IAU)), IB = sg * R.v3(JF_IBU);
+  ready();
   const float Jv = dotx(angA, wa) + dotx(angB, wb);
   int br;
   const float dl = row_solve<false>(T, Jv, me, bi, lo, hi, lam, br);
@@ -551,23 +555,24 @@ __device__ __forceinline__ void hinge_row(const DevTopo& T, const SL& S, const T
   wb = axpy3(dl, IB, wb);
   row_store<TAPE, false>(T, S, tp, it, s, lam, br);
 }
-template <bool TAPE, bool SEQ, bool FULL>
+template <bool TAPE, bool SEQ, bool FULL, class RD>
 __device__ __forceinline__ void contact_rows(const DevTopo& T, const SL& S, const TapeStep& tp, int it, const BlkOp& op,
-                                             const SL& R, float ima, float3& va, float3& wa) {
+                                             const SL& R, float ima, float3& va, float3& wa, const RD& ready) {
   const int mask = FULL ? 7 : op.mask(), s0 = op.slot();
   const float3 ra = R.v3(CF_RA);
   float lam[3], me[3];
   float3 IA[3];
   int br[3];
-  lam[0] = S[T.sm_lam + s0];  // (the friction rows' bound needs it in any block)
 #pragma unroll
   for (int m = 0; m < 3; ++m)
     if (mask >> m & 1) {
-      if (m > 0) lam[m] = S[T.sm_lam + s0 + m];
+      lam[m] = S[T.sm_lam + s0 + m];
       me[m] = R[CF_ME + m];
       IA[m] = R.v3(CF_I + 3 * m);
     }
   const float bias = R[CF_BI], mu = R[CF_MU];
+  ready();
+  if (!(mask & 1)) lam[0] = S[T.sm_lam + s0];  // the friction rows' bound: another block's impulse
   auto row = [&](auto MI, auto AI, float lo, float hi, float b) {
     constexpr int m = decltype(MI)::value, ax = decltype(AI)::value;
     const float3 angA = cross_axis<ax>(ra);
@@ -587,11 +592,12 @@ __device__ __forceinline__ void contact_rows(const DevTopo& T, const SL& S, cons
   for (int m = 0; m < 3; ++m)
     if (mask >> m & 1) row_store<TAPE, false>(T, S, tp, it, s0 + m, lam[m], br[m]);
 }
-template <bool TAPE>
+template <bool TAPE, class RD>
 __device__ __forceinline__ void pair_rows(const DevTopo& T, const SL& S, const TapeStep& tp, int it, const BlkOp& op,
                                           const SL& R, float ima, float imb, float3& va, float3& wa, float3& vb,
-                                          float3& wb) {
+                                          float3& wb, const RD& ready) {
   const int mask = op.mask(), s0 = op.slot();
+  ready();
   float ln = S[T.sm_lam + s0];
 #pragma unroll 1
   for (int m = 0; m < 3; ++m) {
@@ -634,24 +640,25 @@ __device__ __forceinline__ void blk_sweeps(const DevTopo& T, const SL& S, const 
     X.s3(18 * a + 12, v);
     X.s3(18 * a + 15, w);
   };
-  auto rows = [&](const BlkOp& op, int it, float ima, float imb, float3& va, float3& wa, float3& vb, float3& wb) {
+  auto rows = [&](const BlkOp& op, int it, float ima, float imb, float3& va, float3& wa, float3& vb, float3& wb,
+                  const auto& ready) {
     const int type = op.type(), idx = op.idx();
     const SL R = type == BT_GROUND ? contact_rec(T, S, idx) : (type == BT_PAIR ? pair_rec(T, S, idx) : joint_rec(T, S, idx));
     switch (type) {
       case BT_JOINT:
-        if (op.mask() == 31) joint_rows<TAPE, SEQ, true>(T, S, tp, it, op, R, ima, imb, va, wa, vb, wb);
-        else joint_rows<TAPE, SEQ, false>(T, S, tp, it, op, R, ima, imb, va, wa, vb, wb);
+        if (op.mask() == 31) joint_rows<TAPE, SEQ, true>(T, S, tp, it, op, R, ima, imb, va, wa, vb, wb, ready);
+        else joint_rows<TAPE, SEQ, false>(T, S, tp, it, op, R, ima, imb, va, wa, vb, wb, ready);
         break;
       case BT_GROUND:
-        if (op.mask() == 7) contact_rows<TAPE, SEQ, true>(T, S, tp, it, op, R, ima, va, wa);
-        else contact_rows<TAPE, SEQ, false>(T, S, tp, it, op, R, ima, va, wa);
+        if (op.mask() == 7) contact_rows<TAPE, SEQ, true>(T, S, tp, it, op, R, ima, va, wa, ready);
+        else contact_rows<TAPE, SEQ, false>(T, S, tp, it, op, R, ima, va, wa, ready);
         break;
-      case BT_PAIR: pair_rows<TAPE>(T, S, tp, it, op, R, ima, imb, va, wa, vb, wb); break;
-      default: hinge_row<TAPE>(T, S, tp, it, op, R, wa, wb); break;
+      case BT_PAIR: pair_rows<TAPE>(T, S, tp, it, op, R, ima, imb, va, wa, vb, wb, ready); break;
+      default: hinge_row<TAPE>(T, S, tp, it, op, R, wa, wb, ready); break;
     }
   };
-  if (T.blk_single) {
-    // one block: warp 0 keeps its bodies' velocities in registers over the sweeps
+  if (!SEQ && T.blk_single) {
+    // one block (never a compiled topology): warp 0 keeps its bodies' velocities in registers over the sweeps
     if (warp == 0) {
       const bool on = st0[0] != 0;
       const BlkOp op = blk_op(T, 0);
@@ -661,7 +668,7 @@ __device__ __forceinline__ void blk_sweeps(const DevTopo& T, const SL& S, const 
       load(a, va, wa, ima);
       load(b, vb, wb, imb);
       for (int it = 0; it < T.iters; ++it) {
-        if (on) rows(op, it, ima, imb, va, wa, vb, wb);
+        if (on) rows(op, it, ima, imb, va, wa, vb, wb, [] {});
         if (TAPE)
           for (int c = 0; c < T.nb; ++c) {
             float* vi = tp.viter + (it * nv + 6 * c) * 32;
@@ -677,6 +684,7 @@ __device__ __forceinline__ void blk_sweeps(const DevTopo& T, const SL& S, const 
     cta_sync();
     return;
   }
+  bool pend = false;  // a barrier to meet before the next velocities are read
   for (int it = 0; it < T.iters; ++it) {
     const uint8_t* st = st0;
     int e = *st++;
@@ -687,23 +695,28 @@ __device__ __forceinline__ void blk_sweeps(const DevTopo& T, const SL& S, const 
       nop = blk_op(T, nxt & 63);  // the next entry's block while this one runs
       if (e & BS_OP) {
         const int a = op.a(), b = op.b();
-        float3 va, wa, vb, wb;
-        float ima, imb;
-        load(a, va, wa, ima);
-        load(b, vb, wb, imb);
-        rows(op, it, ima, imb, va, wa, vb, wb);
+        float3 va = f3(0.f, 0.f, 0.f), wa = va, vb = va, wb = va;
+        const float ima = a >= 0 ? S[T.sm_invm + a] : 0.f, imb = b >= 0 ? S[T.sm_invm + b] : 0.f;
+        rows(op, it, ima, imb, va, wa, vb, wb, [&] {
+          if (pend) cta_sync();
+          if (a >= 0) { va = X.v3(18 * a + 12); wa = X.v3(18 * a + 15); }
+          if (b >= 0) { vb = X.v3(18 * b + 12); wb = X.v3(18 * b + 15); }
+        });
         store(a, va, wa);
         store(b, vb, wb);
+      } else if (pend) {
+        cta_sync();
       }
-      if (e & BS_BAR) cta_sync();
+      pend = e & BS_BAR;
       e = nxt;
     }
     if (TAPE) {
+      if (pend) cta_sync();
       float* vi = tp.viter + it * nv * 32;
       for (int b = warp; b < T.nb; b += blk_nw())
 #pragma unroll
         for (int k = 0; k < 6; ++k) vi[(6 * b + k) * 32] = X[18 * b + 12 + k];
-      cta_sync();
+      pend = true;
     }
   }
   cta_sync();

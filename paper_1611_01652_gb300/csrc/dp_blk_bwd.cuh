@@ -33,23 +33,22 @@ struct RevBody {
   float3 v, w, vb, wb;
   float im, imb, ii[6], sb[6];
 };
-__device__ __forceinline__ void rev_load(const DevTopo& T, const SL& S, const SL& VW, int b, RevBody& B) {
+__device__ __forceinline__ void rev_init(const DevTopo& T, const SL& S, int b, RevBody& B) {
   B.imb = 0.f;
 #pragma unroll
-  for (int q = 0; q < 6; ++q) B.sb[q] = 0.f;
-  if (b < 0) {
-    B.v = B.w = B.vb = B.wb = f3(0.f, 0.f, 0.f);
-    B.im = 0.f;
-#pragma unroll
-    for (int q = 0; q < 6; ++q) B.ii[q] = 0.f;
-    return;
-  }
+  for (int q = 0; q < 6; ++q) B.sb[q] = B.ii[q] = 0.f;
+  B.v = B.w = B.vb = B.wb = f3(0.f, 0.f, 0.f);
+  B.im = 0.f;
+  if (b < 0) return;
+  B.im = S[T.sm_invm + b];
+  load6(S, T.sm_iinv + 6 * b, B.ii);
+}
+__device__ __forceinline__ void rev_load(const DevTopo& T, const SL& S, const SL& VW, int b, RevBody& B) {
+  if (b < 0) return;
   B.v = VW.v3(6 * b);
   B.w = VW.v3(6 * b + 3);
   B.vb = S.v3(T.sm_vb + 6 * b);
   B.wb = S.v3(T.sm_vb + 6 * b + 3);
-  B.im = S[T.sm_invm + b];
-  load6(S, T.sm_iinv + 6 * b, B.ii);
 }
 __device__ __forceinline__ void rev_store(const DevTopo& T, const SL& S, const SL& VW, int b, const RevBody& B, bool lin) {
   if (b < 0) return;
@@ -164,8 +163,9 @@ __device__ __forceinline__ void rev_begin_sweep(const DevTopo& T, const TapeStep
   }
 }
 
-// Rows, last first. As in the rollout, a block loads everything it reads before its first row and
-// stores after its last one; adjoints of the record are summed in registers.
+// Rows, last first. As in the rollout, a block loads everything it reads before its first row (what
+// only it changes ahead of ready()) and stores after its last one; adjoints of the record are summed in
+// registers.
 // One linear row of a joint: lam is its impulse's adjoint, meb the sum of the effective mass' adjoint;
 // returns the adjoint of J v.
 template <int K>
@@ -222,9 +222,9 @@ __device__ __forceinline__ float rev_ang(const DevTopo& T, float la, float lb, f
   return jvb;
 }
 
-template <bool FULL>
+template <bool FULL, class RD>
 __device__ __forceinline__ void rev_joint(const DevTopo& T, const SL& S, const RevTape& tp, const BlkOp& op, const SL& R,
-                                          RevBody& A, RevBody& B) {
+                                          RevBody& A, RevBody& B, const RD& ready) {
   const int mask = FULL ? 31 : op.mask(), s0 = op.slot();
   const SL Q = R.at(JR_N);
   const float3 ra = R.v3(JF_RA), rb = R.v3(JF_RB);
@@ -240,6 +240,7 @@ __device__ __forceinline__ void rev_joint(const DevTopo& T, const SL& S, const R
       bi[k] = R[JF_BI + k];
       if (k >= 3) t[k - 3] = R.v3(JF_T + 3 * (k - 3));
     }
+  ready();
   float unused;
 #pragma unroll
   for (int k = 4; k >= 3; --k)
@@ -269,8 +270,9 @@ __device__ __forceinline__ void rev_joint(const DevTopo& T, const SL& S, const R
   Q.s3(JA_RA, rab);
   Q.s3(JA_RB, rbb);
 }
+template <class RD>
 __device__ __forceinline__ void rev_hinge(const DevTopo& T, const SL& S, const RevTape& tp, const BlkOp& op, const SL& R, int j,
-                                          RevBody& A, RevBody& B) {
+                                          RevBody& A, RevBody& B, const RD& ready) {
   const bool lim = op.type() == BT_LIMIT;
   const int s = op.slot(), m = lim ? 5 : 6;
   const SL Q = R.at(JR_N);
@@ -278,8 +280,10 @@ __device__ __forceinline__ void rev_hinge(const DevTopo& T, const SL& S, const R
   const int br = tp.br[s * 32];
   const float me = R[JF_ME + m], bi = R[JF_BI + m], la = tp.la[s], lb = tp.lb[s];
   const float meb0 = Q[JA_ME + m], bib0 = Q[JA_BI + m], bnd0 = Q[JA_BND];
-  const float3 u0 = Q.v3(JA_U), ua = S.v3(T.sm_ua + 3 * j);
+  const float3 ua = S.v3(T.sm_ua + 3 * j);
   float lam = S[T.sm_lam + s], meb, lbar;
+  ready();
+  const float3 u0 = Q.v3(JA_U);  // (the joint's limit and servo row share it)
   float3 ub;
   const float bib = rev_ang(T, la, lb, me, bi, br, sg * ua, A, B, ub, lam, meb, lbar);
   S[T.sm_lam + s] = lam;
@@ -288,8 +292,9 @@ __device__ __forceinline__ void rev_hinge(const DevTopo& T, const SL& S, const R
   Q.s3(JA_U, u0 + sg * ub);
   if (!lim) Q[JA_BND] = bnd0 + (br == 2 ? 1.f : (br == 1 ? -1.f : 0.f)) * lbar;
 }
+template <class RD>
 __device__ __forceinline__ void rev_contact(const DevTopo& T, const SL& S, const RevTape& tp, const BlkOp& op, const SL& R,
-                                            RevBody& A) {
+                                            RevBody& A, const RD& ready) {
   const int mask = op.mask(), s0 = op.slot();
   const SL Q = R.at(CR_N);
   float la[3], lb[3], lam[3], me[3], meb[3];
@@ -306,6 +311,9 @@ __device__ __forceinline__ void rev_contact(const DevTopo& T, const SL& S, const
   const float3 ra = R.v3(CF_RA);
   const float mu = R[CF_MU], bias0 = R[CF_BI];
   float3 rab = f3(0.f, 0.f, 0.f);
+  ready();
+  if (mask != 7)  // another block of this contact changes their adjoints too
+    for (int m = 0; m < 3; ++m) lam[m] = S[T.sm_lam + s0 + m];
   // the normal impulse a friction row saw: the sweep's own (the normal row comes first)
   const float lnrm = la[0];
   float mub = 0.f, bib = 0.f;
@@ -355,8 +363,10 @@ __device__ __forceinline__ void rev_contact(const DevTopo& T, const SL& S, const
   Q[CA_MU] = mub;
   Q.s3(CA_RA, rab);
 }
+template <class RD>
 __device__ __forceinline__ void rev_pair(const DevTopo& T, const SL& S, const RevTape& tp, const BlkOp& op, const SL& R,
-                                         RevBody& A, RevBody& B) {
+                                         RevBody& A, RevBody& B, const RD& ready) {
+  ready();
   const int mask = op.mask(), s0 = op.slot();
   const float mu = R[PF_MU], lnrm = tp.la[s0];
 #pragma unroll 1
@@ -399,23 +409,49 @@ __device__ __forceinline__ void rev_pair(const DevTopo& T, const SL& S, const Re
 }
 
 // The sweeps backwards (every warp calls; ends after a CTA barrier). On entry VB holds the adjoint
-// of the solver's output velocities, on exit that of its input velocities.
+// of the solver's output velocities, on exit that of its input velocities. ONE: the robot may be of one
+// block, whose warp keeps the bodies' adjoints in registers over the sweeps.
+template <bool ONE>
 __device__ __forceinline__ void blk_sweeps_rev(const DevTopo& T, const SL& S, const TapeStep& tp, int warp) {
   const uint8_t* st0 = blk_bytes(T) + T.blk_stream + warp * T.blk_stream_len;
-  auto rows = [&](const BlkOp& op, const RevTape& rt, RevBody& A, RevBody& B) {
+  auto rows = [&](const BlkOp& op, const RevTape& rt, RevBody& A, RevBody& B, const auto& ready) {
     const int type = op.type(), idx = op.idx();
-    if (type == BT_GROUND) rev_contact(T, S, rt, op, contact_rec(T, S, idx), A);
+    if (type == BT_GROUND) rev_contact(T, S, rt, op, contact_rec(T, S, idx), A, ready);
     else if (type == BT_JOINT) {
-      if (op.mask() == 31) rev_joint<true>(T, S, rt, op, joint_rec(T, S, idx), A, B);
-      else rev_joint<false>(T, S, rt, op, joint_rec(T, S, idx), A, B);
-    } else if (type == BT_PAIR) rev_pair(T, S, rt, op, pair_rec(T, S, idx), A, B);
-    else rev_hinge(T, S, rt, op, joint_rec(T, S, idx), idx, A, B);
+      if (op.mask() == 31) rev_joint<true>(T, S, rt, op, joint_rec(T, S, idx), A, B, ready);
+      else rev_joint<false>(T, S, rt, op, joint_rec(T, S, idx), A, B, ready);
+    } else if (type == BT_PAIR) rev_pair(T, S, rt, op, pair_rec(T, S, idx), A, B, ready);
+    else rev_hinge(T, S, rt, op, joint_rec(T, S, idx), idx, A, B, ready);
   };
+  if (ONE && T.blk_single) {
+    const bool on = warp == 0 && st0[0] != 0;
+    const BlkOp op = blk_op(T, 0);
+    const int a = op.a(), b = op.b();
+    RevBody A, B;
+    SL vw = S.at(T.sm_vw);
+    rev_init(T, S, a, A);
+    rev_init(T, S, b, B);
+    rev_load(T, S, vw, a, A);
+    rev_load(T, S, vw, b, B);
+    for (int it = T.iters - 1; it >= 0; --it) {
+      rev_begin_sweep(T, tp, it);
+      const RevTape rt = rev_tape(T, S, it);
+      if (!on) continue;
+      vw = rt.vw;
+      if (a >= 0) { A.v = vw.v3(6 * a); A.w = vw.v3(6 * a + 3); }
+      if (b >= 0) { B.v = vw.v3(6 * b); B.w = vw.v3(6 * b + 3); }
+      rows(op, rt, A, B, [] {});
+    }
+    if (on) { rev_store(T, S, vw, a, A, true); rev_store(T, S, vw, b, B, true); }
+    cta_sync();
+    return;
+  }
   for (int it = T.iters - 1; it >= 0; --it) {
     rev_begin_sweep(T, tp, it);
     const RevTape rt = rev_tape(T, S, it);
     const uint8_t* st = st0;
     int e = *st++;
+    bool pend = false;  // a level's barrier to meet before the next velocities are read
     BlkOp nop = blk_op(T, e & 63);
     while (e) {
       const int nxt = *st++;
@@ -425,13 +461,19 @@ __device__ __forceinline__ void blk_sweeps_rev(const DevTopo& T, const SL& S, co
         const int a = op.a(), b = op.b(), type = op.type();
         const bool lin = type <= BT_JOINT || type >= BT_GROUND;
         RevBody A, B;
-        rev_load(T, S, rt.vw, a, A);
-        rev_load(T, S, rt.vw, b, B);
-        rows(op, rt, A, B);
+        rev_init(T, S, a, A);
+        rev_init(T, S, b, B);
+        rows(op, rt, A, B, [&] {
+          if (pend) cta_sync();
+          rev_load(T, S, rt.vw, a, A);
+          rev_load(T, S, rt.vw, b, B);
+        });
         rev_store(T, S, rt.vw, a, A, lin);
         rev_store(T, S, rt.vw, b, B, lin);
+      } else if (pend) {
+        cta_sync();
       }
-      if (e & BS_BAR) cta_sync();
+      pend = e & BS_BAR;  // (the last one is met with the next sweep's)
       e = nxt;
     }
   }
@@ -1191,7 +1233,7 @@ __device__ __forceinline__ void blk_reverse_step(const DevTopo& T, const DevPtrs
     for (int q = 0; q < PA_N; ++q) pair_rec(T, S, c)[PR_N + q] = 0.f;
   cta_sync();
   blk_stream(T, warp, true);
-  blk_sweeps_rev(T, S, tp, warp);
+  blk_sweeps_rev<!Q::SEQ>(T, S, tp, warp);
   const bool ws = T.ws != 0;
   for (int j = warp; j < T.nj; j += blk_nw()) joint_reverse(T, C, tp, ws, j);
   for (int q = warp; q < T.ns; q += blk_nw()) contact_reverse(T, C, tp, ws, q);

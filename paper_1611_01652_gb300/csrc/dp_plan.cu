@@ -99,9 +99,14 @@ bool plan_blocks(DevTopo& T, std::vector<int32_t>& blob) {
     const int cap = std::max(1, ops[ready[0]].weight);
     for (int g = 0; g < nw; ++g) runs[g].emplace_back();
     for (int k : ready) {
-      int w = 0;
-      for (int g = 1; g < nw; ++g)
+      // the first warp of the level rotates: the warps of a level's most urgent blocks were idle in the
+      // one before, and load their next record while they wait for its barrier
+      const int first = nlev * 3 % nw;
+      int w = first;
+      for (int q = 1; q < nw; ++q) {
+        const int g = (first + q) % nw;
         if (load[g] < load[w] || (load[g] == load[w] && cnt[g] < cnt[w])) w = g;
+      }
       if (cnt[w] > 0 && load[w] + ops[k].weight > cap) continue;
       ops[k].level = nlev;
       ops[k].warp = w;
