@@ -127,59 +127,52 @@ __global__ void __launch_bounds__(32 * WS_WARPS) k_ws_fwdbwd(const __nv_bfloat16
 
 // Split-K weight and bias gradient, all three layers in one launch (blockIdx.y: the layer, blockIdx.x:
 // the split's columns): partial[split] holds a whole gradient in the master weights' layout. A CTA of
-// 256 threads forms the layer's M x C products (M, C <= 64; 4 x 4 per thread, fp32) 32 columns at a
+// 256 threads forms the layer's M x C products (M, C <= 64; up to 4 x 4 per thread, fp32) 32 columns at a
 // time, the next columns on their way in registers meanwhile; thread t < M also sums delta row t, the
 // bias gradient.
-// Bound: FFMA (32768 rows: 0.7 GFLOP over the three padded tiles), if the chip is full. A split per
+// Bound: FFMA (32768 rows: 0.35 GFLOP), if the chip is full. A split per
 // 16384 columns left two CTAs on 152 SMs: 5634 us at 32768 rows. With one per 256 columns (at most
-// 256) the three layers are 384 CTAs there.
+// 256) the three layers are 384 CTAs there: the whole training step 5673 -> 82 us, and 70 us with each
+// layer's own tile (a 64 x 64 tile for all three kept 1.5 of 3 tiles' products for padding).
 constexpr int DW_K = 32, DW_LD = DW_K + 4;
-__global__ void __launch_bounds__(256) k_ws_dw(const float* __restrict__ act, const float* __restrict__ del, long long np,
-                                               long long chunk, float* __restrict__ partial) {
-  __shared__ __align__(16) float As[64][DW_LD], Bs[64][DW_LD];
-  const int layer = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int M = layer == 2 ? WsTC::NO : (layer == 1 ? WsTC::H2 : WsTC::H1);
-  const int C = layer == 2 ? WsTC::H2 : (layer == 1 ? WsTC::H1 : WsTC::K0);
-  const float* dl = del + (size_t)(layer == 2 ? WsTC::H1 + WsTC::H2 : (layer == 1 ? WsTC::H1 : 0)) * np;
-  const float* al = act + (size_t)(layer == 2 ? WsTC::K0 + WsTC::H1 : (layer == 1 ? WsTC::K0 : 0)) * np;
-  const int fw = layer == 2 ? WsTC::F_W3 : (layer == 1 ? WsTC::F_W2 : WsTC::F_W1);
-  const int fb = layer == 2 ? WsTC::F_B3 : (layer == 1 ? WsTC::F_B2 : WsTC::F_B1);
+template <int M, int C>
+__device__ __forceinline__ void ws_dw_layer(float (&As)[64][DW_LD], float (&Bs)[64][DW_LD], const float* __restrict__ dl,
+                                            const float* __restrict__ al, long long np, long long chunk, float* __restrict__ W,
+                                            float* __restrict__ b) {
+  constexpr int U = (M + 15) / 16, V = (C + 15) / 16;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const long long n0 = (long long)blockIdx.x * chunk, n1 = min(np, n0 + chunk);  // multiples of DW_K
   const int tx = tid & 15, ty = tid >> 4;
-  float ra[8], rb[8];
-  auto fetch = [&](long long n) {  // a warp takes eight rows of each operand, a lane one column
+  float ra[2 * U], rb[2 * V];
+  auto fetch = [&](long long n) {  // a warp takes every eighth row of each operand, a lane one column
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int r = warp + 8 * q;
-      ra[q] = r < M ? __ldg(dl + (size_t)r * np + n + lane) : 0.f;
-      rb[q] = r < C ? __ldg(al + (size_t)r * np + n + lane) : 0.f;
-    }
+    for (int q = 0; q < 2 * U; ++q) ra[q] = warp + 8 * q < M ? __ldg(dl + (size_t)(warp + 8 * q) * np + n + lane) : 0.f;
+#pragma unroll
+    for (int q = 0; q < 2 * V; ++q) rb[q] = warp + 8 * q < C ? __ldg(al + (size_t)(warp + 8 * q) * np + n + lane) : 0.f;
   };
-  float acc[4][4] = {}, bsum = 0.f;
+  float acc[U][V] = {}, bsum = 0.f;
   const bool work = ty < M && tx < C;  // rows ty + 16 u, columns tx + 16 v
   if (n0 < n1) fetch(n0);
   for (long long n = n0; n < n1; n += DW_K) {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      As[warp + 8 * q][lane] = ra[q];
-      Bs[warp + 8 * q][lane] = rb[q];
-    }
+    for (int q = 0; q < 2 * U; ++q) As[warp + 8 * q][lane] = ra[q];
+#pragma unroll
+    for (int q = 0; q < 2 * V; ++q) Bs[warp + 8 * q][lane] = rb[q];
     __syncthreads();
     if (n + DW_K < n1) fetch(n + DW_K);
     if (work) {
 #pragma unroll
       for (int k = 0; k < DW_K; k += 4) {
-        float4 a[4], b[4];
+        float4 x[U], y[V];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          a[u] = *reinterpret_cast<const float4*>(&As[ty + 16 * u][k]);
-          b[u] = *reinterpret_cast<const float4*>(&Bs[tx + 16 * u][k]);
-        }
+        for (int u = 0; u < U; ++u) x[u] = *reinterpret_cast<const float4*>(&As[ty + 16 * u][k]);
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
+        for (int v = 0; v < V; ++v) y[v] = *reinterpret_cast<const float4*>(&Bs[tx + 16 * v][k]);
 #pragma unroll
-          for (int v = 0; v < 4; ++v)
-            acc[u][v] = fmaf(a[u].w, b[v].w, fmaf(a[u].z, b[v].z, fmaf(a[u].y, b[v].y, fmaf(a[u].x, b[v].x, acc[u][v]))));
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int v = 0; v < V; ++v)
+            acc[u][v] = fmaf(x[u].w, y[v].w, fmaf(x[u].z, y[v].z, fmaf(x[u].y, y[v].y, fmaf(x[u].x, y[v].x, acc[u][v]))));
       }
     }
     if (tid < M)
@@ -187,15 +180,27 @@ __global__ void __launch_bounds__(256) k_ws_dw(const float* __restrict__ act, co
       for (int k = 0; k < DW_K; ++k) bsum += As[tid][k];
     __syncthreads();
   }
-  float* P = partial + (size_t)blockIdx.x * WsTC::PARAMS;
 #pragma unroll
-  for (int u = 0; u < 4; ++u)
+  for (int u = 0; u < U; ++u)
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
+    for (int v = 0; v < V; ++v) {
       const int o = ty + 16 * u, c = tx + 16 * v;
-      if (o < M && c < C) P[fw + o * C + c] = acc[u][v];
+      if (o < M && c < C) W[o * C + c] = acc[u][v];
     }
-  if (tid < M) P[fb + tid] = bsum;
+  if (tid < M) b[tid] = bsum;
+}
+__global__ void __launch_bounds__(256) k_ws_dw(const float* __restrict__ act, const float* __restrict__ del, long long np,
+                                               long long chunk, float* __restrict__ partial) {
+  __shared__ __align__(16) float As[64][DW_LD], Bs[64][DW_LD];
+  float* P = partial + (size_t)blockIdx.x * WsTC::PARAMS;
+  if (blockIdx.y == 0)
+    ws_dw_layer<WsTC::H1, WsTC::K0>(As, Bs, del, act, np, chunk, P + WsTC::F_W1, P + WsTC::F_B1);
+  else if (blockIdx.y == 1)
+    ws_dw_layer<WsTC::H2, WsTC::H1>(As, Bs, del + (size_t)WsTC::H1 * np, act + (size_t)WsTC::K0 * np, np, chunk,
+                                    P + WsTC::F_W2, P + WsTC::F_B2);
+  else
+    ws_dw_layer<WsTC::NO, WsTC::H2>(As, Bs, del + (size_t)(WsTC::H1 + WsTC::H2) * np,
+                                    act + (size_t)(WsTC::K0 + WsTC::H1) * np, np, chunk, P + WsTC::F_W3, P + WsTC::F_B3);
 }
 
 // The splits' partials added up in a fixed order, 32 parameters a block, eight threads each; the last
