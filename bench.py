@@ -40,11 +40,11 @@ SM_COUNT, FP32_LANES, MAX_SM_MHZ = 152, 128, 2070.0
 RESID_TOL = 0.02
 # sweep counts of the warm-start gate
 WS_ITERS = (5, 7, 10, 14)
-# DRAM bytes (read + written) per instance-step of k_backward_mw, damped start at 10 sweeps:
+# DRAM bytes (read + written) per instance-step of k_backward_blk, damped start at 10 sweeps:
 # dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture of one launch at B = 1024,
-# T = 20 (295.9 MB + 18.6 MB, the kernel as built now) / (B T). The tape is read once per
+# T = 20 (176.9 MB + 15.8 MB, the kernel as built now) / (B T). The tape is read once per
 # launch, so the traffic of the full launch scales with B T.
-BWD_TRAFFIC_PER_INST_STEP = {10: (295889920 + 18576896) / (1024 * 20)}
+BWD_TRAFFIC_PER_INST_STEP = {10: (176907264 + 15763456) / (1024 * 20)}
 
 
 def parse():
@@ -745,7 +745,7 @@ def main():
     derived = SM_COUNT * FP32_LANES * 2 * MAX_SM_MHZ * 1e6 / 1e12  # TFLOP/s, FP32 FMA at max SM clock
     peak = fp32_peak if fp32_peak > 0 else derived
     achieved = fl["reverse"] * B * T / (head["bwd_ms"] / 1e3) / 1e12
-    roofline = {"bound": "alu", "kernel": "k_backward_mw<QuadrupedTopo> (dp_backward)", "achieved": achieved,
+    roofline = {"bound": "alu", "kernel": "k_backward_blk<BlkQuad> (dp_backward)", "achieved": achieved,
                 "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": (BWD_TRAFFIC_PER_INST_STEP[it] * B * T
                                                       if it in BWD_TRAFFIC_PER_INST_STEP else None),
