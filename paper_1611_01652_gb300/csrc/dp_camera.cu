@@ -404,6 +404,8 @@ __device__ __forceinline__ void red_texels(float* D, size_t i, size_t n, bool ve
 // 240 us. A texture is usually stretched over several pixels, so the neighbouring pixels of a warp that
 // sample the same four texels are summed first (shuffles over each run of lanes), and the run's first
 // lane adds a texture row's two texels with 16-byte reductions: frames and gradients 3329 -> 890 us.
+// TEX: with the textures' gradient (its sums cost registers that the pose gradient alone does not need).
+template <bool TEX>
 __global__ void __launch_bounds__(kThreads) k_render_bwd(const __grid_constant__ CamArgs A, const float* __restrict__ state,
                                                          const float* __restrict__ tex, const float* __restrict__ dimage,
                                                          float* __restrict__ dstate, float* __restrict__ dtex,
@@ -446,7 +448,7 @@ __global__ void __launch_bounds__(kThreads) k_render_bwd(const __grid_constant__
         const float t00 = __ldg(T + i00), t01 = __ldg(T + i01), t10 = __ldg(T + i10), t11 = __ldg(T + i11);
         dfx += gi * ((1.f - S.fy) * (t01 - t00) + S.fy * (t11 - t10));
         dfy += gi * (((1.f - S.fx) * t10 + S.fx * t11) - ((1.f - S.fx) * t00 + S.fx * t01));
-        if (gi != 0.f) {
+        if (TEX && gi != 0.f) {
           tg[ch] = gi * (1.f - S.fx) * (1.f - S.fy);
           tg[3 + ch] = gi * S.fx * (1.f - S.fy);
           tg[6 + ch] = gi * (1.f - S.fx) * S.fy;
@@ -534,7 +536,7 @@ __global__ void __launch_bounds__(kThreads) k_render_bwd(const __grid_constant__
     }
   }
   const unsigned full = 0xffffffffu;
-  if (dtex && __any_sync(full, kt >= 0)) {
+  if (TEX && __any_sync(full, kt >= 0)) {
     const int lane = threadIdx.x & 31;
     const int kxy = kx0 * 2 + kdx, kyy = ky0 * 2 + kdy;
     // (every lane takes part in the three shuffles)
@@ -667,8 +669,12 @@ dp_status dp_render_backward(const dp_camera* cam, const dp_scene* scene, int32_
     e = cudaMemsetAsync(dtextures, 0, sizeof(float) * (size_t)scene->n_tex * A.th * A.tw * 3, s);
   const size_t n = (size_t)A.W * A.H * A.B;
   if (e == cudaSuccess && n > 0) {
-    k_render_bwd<<<(unsigned)((n + kChunk - 1) / kChunk), kThreads, 0, s>>>(A, state, textures, dimage, dstate, dtextures,
-                                                                                 (size_t)scene->n_tex * A.th * A.tw * 3);
+    const unsigned grid = (unsigned)((n + kChunk - 1) / kChunk);
+    if (dtextures)
+      k_render_bwd<true><<<grid, kThreads, 0, s>>>(A, state, textures, dimage, dstate, dtextures,
+                                                    (size_t)scene->n_tex * A.th * A.tw * 3);
+    else
+      k_render_bwd<false><<<grid, kThreads, 0, s>>>(A, state, textures, dimage, dstate, nullptr, 0);
     e = cudaGetLastError();
   }
   if (e != cudaSuccess) { g_cam_err = cudaGetErrorString(e); return DP_ECUDA; }
