@@ -166,7 +166,8 @@ __device__ __forceinline__ void rev_begin_sweep(const DevTopo& T, const TapeStep
 // Rows, last first. As in the rollout, a block loads everything it reads before its first row (what
 // only it changes ahead of ready()) and stores after its last one; adjoints of the record are summed in
 // registers.
-// One linear row of a joint: lam is its impulse's adjoint, meb the sum of the effective mass' adjoint;
+// One linear row of a joint: lam is its impulse's adjoint, meb the sum of the effective mass' adjoint
+// (over the step: each row's share is added by one fused multiply-add);
 // returns the adjoint of J v.
 template <int K>
 __device__ __forceinline__ float rev_lin(const DevTopo& T, float la, float lb, float me, float bi, float3 ra, float3 rb,
@@ -191,7 +192,7 @@ __device__ __forceinline__ float rev_lin(const DevTopo& T, float la, float lb, f
   A.imb = fmaf(dl, axis_of<K>(A.vb), A.imb);
   B.imb = fmaf(-dl, axis_of<K>(B.vb), B.imb);
   const float Jv = (axis_of<K>(A.v) + dot_axis<K>(ra, A.w)) - (axis_of<K>(B.v) + dot_axis<K>(rb, B.w));
-  meb = -pbar * (Jv + bi + T.gamma * lb);
+  meb += -pbar * (Jv + bi + T.gamma * lb);
   axis_of<K>(A.vb) += jvb;
   add_axis<K>(A.wb, jvb, ra);
   axis_of<K>(B.vb) -= jvb;
@@ -216,7 +217,7 @@ __device__ __forceinline__ float rev_ang(const DevTopo& T, float la, float lb, f
   sym_outer(A.sb, -ga, d);
   sym_outer(B.sb, gb, d);
   const float Jv = dot3(d, B.w - A.w);
-  meb = -pbar * (Jv + bi + T.gamma * lb);
+  meb += -pbar * (Jv + bi + T.gamma * lb);
   A.wb = axpy3(-jvb, d, A.wb);
   B.wb = axpy3(jvb, d, B.wb);
   return jvb;
@@ -238,6 +239,7 @@ __device__ __forceinline__ void rev_joint(const DevTopo& T, const SL& S, const R
       lam[k] = S[T.sm_lam + s0 + k];
       me[k] = R[JF_ME + k];
       bi[k] = R[JF_BI + k];
+      meb[k] = Q[JA_ME + k];
       if (k >= 3) t[k - 3] = R.v3(JF_T + 3 * (k - 3));
     }
   ready();
@@ -253,7 +255,6 @@ __device__ __forceinline__ void rev_joint(const DevTopo& T, const SL& S, const R
 #pragma unroll
   for (int k = 0; k < 5; ++k)
     if (mask >> k & 1) {
-      meb[k] += Q[JA_ME + k];
       bib[k] += Q[JA_BI + k];
       if (k >= 3) tb[k - 3] = Q.v3(JA_T + 3 * (k - 3)) - tb[k - 3];
     }
@@ -279,15 +280,15 @@ __device__ __forceinline__ void rev_hinge(const DevTopo& T, const SL& S, const R
   const float sg = lim ? R[JF_LS] : 1.f;
   const int br = tp.br[s * 32];
   const float me = R[JF_ME + m], bi = R[JF_BI + m], la = tp.la[s], lb = tp.lb[s];
-  const float meb0 = Q[JA_ME + m], bib0 = Q[JA_BI + m], bnd0 = Q[JA_BND];
+  const float bib0 = Q[JA_BI + m], bnd0 = Q[JA_BND];
   const float3 ua = S.v3(T.sm_ua + 3 * j);
-  float lam = S[T.sm_lam + s], meb, lbar;
+  float lam = S[T.sm_lam + s], meb = Q[JA_ME + m], lbar;
   ready();
   const float3 u0 = Q.v3(JA_U);  // (the joint's limit and servo row share it)
   float3 ub;
   const float bib = rev_ang(T, la, lb, me, bi, br, sg * ua, A, B, ub, lam, meb, lbar);
   S[T.sm_lam + s] = lam;
-  Q[JA_ME + m] = meb0 + meb;
+  Q[JA_ME + m] = meb;
   Q[JA_BI + m] = bib0 + bib;
   Q.s3(JA_U, u0 + sg * ub);
   if (!lim) Q[JA_BND] = bnd0 + (br == 2 ? 1.f : (br == 1 ? -1.f : 0.f)) * lbar;
@@ -306,14 +307,17 @@ __device__ __forceinline__ void rev_contact(const DevTopo& T, const SL& S, const
     br[m] = tp.br[(s0 + m) * 32];
     lam[m] = S[T.sm_lam + s0 + m];
     me[m] = R[CF_ME + m];
-    meb[m] = 0.f;
+    meb[m] = Q[CA_ME + m];
   }
   const float3 ra = R.v3(CF_RA);
   const float mu = R[CF_MU], bias0 = R[CF_BI];
   float3 rab = f3(0.f, 0.f, 0.f);
   ready();
-  if (mask != 7)  // another block of this contact changes their adjoints too
-    for (int m = 0; m < 3; ++m) lam[m] = S[T.sm_lam + s0 + m];
+  if (mask != 7)  // another block of this contact changes their adjoints and sums too
+    for (int m = 0; m < 3; ++m) {
+      lam[m] = S[T.sm_lam + s0 + m];
+      meb[m] = Q[CA_ME + m];
+    }
   // the normal impulse a friction row saw: the sweep's own (the normal row comes first)
   const float lnrm = la[0];
   float mub = 0.f, bib = 0.f;
@@ -338,7 +342,7 @@ __device__ __forceinline__ void rev_contact(const DevTopo& T, const SL& S, const
     sym_outer_axis<ax>(A.sb, ga, ra);
     A.imb = fmaf(dl, axis_of<ax>(A.vb), A.imb);
     const float Jv = axis_of<ax>(A.v) + dot_axis<ax>(ra, A.w);
-    meb[m] = -pbar * (Jv + bias + T.gamma * lb[m]);
+    meb[m] += -pbar * (Jv + bias + T.gamma * lb[m]);
     if (m == 0) bib = jvb;
     axis_of<ax>(A.vb) += jvb;
     add_axis<ax>(A.wb, jvb, ra);
@@ -349,8 +353,6 @@ __device__ __forceinline__ void rev_contact(const DevTopo& T, const SL& S, const
   if (mask & 4) row(I2{}, I1{}, 0.f);
   if (mask & 2) row(I1{}, I0{}, 0.f);
   if (mask & 1) row(I0{}, I2{}, bias0);
-#pragma unroll
-  for (int m = 0; m < 3; ++m) meb[m] += Q[CA_ME + m];
   bib += Q[CA_BI];
   mub += Q[CA_MU];
   rab = Q.v3(CA_RA) + rab;
