@@ -182,7 +182,7 @@ __device__ __forceinline__ float rev_lin(const DevTopo& T, float la, float lb, f
   B.w = axpy3(dl, IBn, B.w);
   const float dbar = (A.im * axis_of<K>(A.vb) + dot3(IA, A.wb)) - (B.im * axis_of<K>(B.vb) + dot3(IBn, B.wb));
   const float pbar = lam + dbar, jvb = -me * pbar;
-  lam = fmaf(pbar, fmaf(-me, T.gamma, 1.f), -dbar);
+  lam = fmaf(-me * T.gamma, pbar, lam);  // pbar (1 - me gamma) - dbar, without the cancellation
   // adjoints of M^-1 J^T (before the update of the velocity adjoints)
   const float3 ga = dl * A.wb, gb = dl * B.wb;
   add_e_cross<K>(rab, 1.f, axpy3(jvb, A.w, symv(A.ii, ga)));
@@ -211,7 +211,7 @@ __device__ __forceinline__ float rev_ang(const DevTopo& T, float la, float lb, f
   const float dbar = dot3(IB, B.wb) - dot3(IA, A.wb);
   lbar = lam + dbar;
   const float pbar = br == 0 ? lbar : 0.f, jvb = -me * pbar;
-  lam = fmaf(pbar, fmaf(-me, T.gamma, 1.f), -dbar);
+  lam = br == 0 ? fmaf(-me * T.gamma, pbar, lam) : -dbar;
   const float3 ga = dl * A.wb, gb = dl * B.wb;
   db = (axpy3(jvb, B.w, symv(B.ii, gb))) - (axpy3(jvb, A.w, symv(A.ii, ga)));
   sym_outer(A.sb, -ga, d);
@@ -336,7 +336,7 @@ __device__ __forceinline__ void rev_contact(const DevTopo& T, const SL& S, const
       mub += sg * lnrm * lbar;
       lam[0] += sg * mu * lbar;
     }
-    lam[m] = fmaf(pbar, fmaf(-me[m], T.gamma, 1.f), -dbar);
+    lam[m] = br[m] == 0 ? fmaf(-me[m] * T.gamma, pbar, lam[m]) : -dbar;
     const float3 ga = dl * A.wb;
     add_e_cross<ax>(rab, 1.f, axpy3(jvb, A.w, symv(A.ii, ga)));
     sym_outer_axis<ax>(A.sb, ga, ra);
