@@ -276,31 +276,43 @@ int plan_smem_blk_bwd(DevTopo& T) {
   T.sm_xb = take(18 * T.nb);
   T.sm_hb = take(T.n_rec);
   const int keep = o;
-  T.sm_x = take(18 * T.nb);
+  const bool rows = T.topo_id != 0;  // compiled topologies: the adjoints row by row
+  const int nbr = (T.nslots + 3) / 4;  // clamp branches (bytes)
+  const int sbar = T.n_layers > 0 && !T.ext_ctrl ? T.widths[0] : 1, zb = T.n_layers > 0 ? std::max(T.widths[T.n_layers], 16) : 1;
+  // staged tape lines: impulses after three sweeps, velocities and branches of two
+  const int over = T.nslots + 6 * T.nb + nbr;
+  T.sm_x = take(rows ? std::max(18 * T.nb, over) : 18 * T.nb);
   T.sm_vb = take(6 * T.nb);
-  T.sm_vw = take(2 * 6 * T.nb);                  // two sweeps
-  T.sm_rlam = take(3 * T.nslots);                // impulses after three sweeps
-  T.sm_rbr = take(2 * ((T.nslots + 3) / 4));     // clamp branches (bytes) of two
+  T.sm_vw = take((rows ? 1 : 2) * 6 * T.nb);
+  T.sm_rlam = take(rows ? std::max(2 * T.nslots, sbar + zb + 6 * T.nj) : 3 * T.nslots);
+  T.sm_rbr = take((rows ? 1 : 2) * nbr);
+  // what the first sweep does not need lies over x_t, which is read again after the sweeps
+  T.sm_rlam2 = T.sm_x;
+  T.sm_vw2 = T.sm_x + T.nslots;
+  T.sm_rbr2 = T.sm_x + T.nslots + 6 * T.nb;
   T.sm_iinv = take(6 * T.nb);
   T.sm_invm = take(T.nb);
-  T.sm_iinvb = take(6 * T.nb);
+  T.sm_iinvb = take((rows ? 9 : 6) * T.nb);
   T.sm_invmb = take(T.nb);
   T.sm_th = take(T.nj);
   T.sm_thd = take(T.nj);
   T.sm_ua = take(3 * T.nj);
   T.sm_wst = take(T.nj);
   T.sm_wbr = take(T.nj);
-  T.sm_thb = take(T.nj);
-  T.sm_thdb = take(T.nj);
-  T.sm_uab = take(3 * T.nj);
-  T.sm_wstb = take(T.nj);
   T.sm_lam = take(T.nslots);
-  T.sm_sbar = take(T.n_layers > 0 && !T.ext_ctrl ? T.widths[0] : 1);
-  T.sm_zb = take(T.n_layers > 0 ? std::max(T.widths[T.n_layers], 16) : 1);
+  // what lives between the sweeps and the next step's staging may share the staged impulses' memory
+  int after = T.sm_rlam;
+  auto late = [&](int n) { if (!rows) return take(n); const int r = after; after += n; return r; };
+  T.sm_thb = late(T.nj);
+  T.sm_thdb = late(T.nj);
+  T.sm_uab = late(3 * T.nj);
+  T.sm_wstb = late(T.nj);
+  T.sm_sbar = late(sbar);
+  T.sm_zb = late(zb);
   T.sm_prog = take((T.blk_bytes_total + 127) / 128);
   T.sm_rows = T.sm_hbuf = o;
-  T.rec_j = 58;
-  T.rec_c = 21;
+  T.rec_j = rows ? RX_REC_J : 58;
+  T.rec_c = rows ? RX_REC_C : 21;
   T.rec_p = 64;
   int buf = 1;  // the controller's buffers lie over the records
   if (T.mlp_tc) buf = 2 * (T.widths[1] + 8);  // four planes of [32][H + 8] bfloat16

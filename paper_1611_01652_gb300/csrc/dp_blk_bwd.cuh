@@ -13,8 +13,10 @@
 //     four warps) and the hinge kinematics (items, packages again).
 // A body belongs to one block at a time (levels), one warp outside the sweeps, so every sum has one
 // writer and a fixed order.
+// The compiled topologies (kernels with SEQ) form the same adjoints row by row: their blocks, items and
+// packages are in dp_blk_rows.cuh, those here are every other robot's.
 #pragma once
-#include "dp_blk_fwd.cuh"
+#include "dp_blk_rows.cuh"
 
 // Accumulators behind a record's first fields (joints: JA_* from JR_N on, contacts from CR_N, pairs
 // from PR_N), and the packages that overwrite the records.
@@ -121,10 +123,29 @@ struct RevTape {
   SL la, lb, vw;
   const uint8_t* br;  // slot s at br[32 s]
 };
+// Where sweep `it`'s impulses (a ring of three sweeps), velocities and branches (two) lie. ROWS (compiled
+// topologies): the buffers that the first sweep does not need lie over x_t (sm_rlam2, sm_vw2, sm_rbr2):
+// nothing is written to them before the records are formed.
+template <bool ROWS>
+__device__ __forceinline__ int rev_lam_at(const DevTopo& T, int it) {
+  if (!ROWS) return T.sm_rlam + (it + 3) % 3 * T.nslots;
+  const int k = (T.iters - 1 - it) % 3;
+  return k == 2 ? T.sm_rlam2 : T.sm_rlam + k * T.nslots;
+}
+template <bool ROWS>
+__device__ __forceinline__ int rev_vw_at(const DevTopo& T, int it) {
+  if (!ROWS) return T.sm_vw + (it & 1) * 6 * T.nb;
+  return (T.iters - 1 - it) & 1 ? T.sm_vw2 : T.sm_vw;
+}
+template <bool ROWS>
+__device__ __forceinline__ int rev_br_at(const DevTopo& T, int it) {
+  if (!ROWS) return T.sm_rbr + (it & 1) * ((T.nslots + 3) / 4);
+  return (T.iters - 1 - it) & 1 ? T.sm_rbr2 : T.sm_rbr;
+}
+template <bool ROWS>
 __device__ __forceinline__ RevTape rev_tape(const DevTopo& T, const SL& S, int it) {
-  return RevTape{S.at(T.sm_rlam + it % 3 * T.nslots), S.at(T.sm_rlam + (it + 2) % 3 * T.nslots),
-                 S.at(T.sm_vw + (it & 1) * 6 * T.nb),
-                 reinterpret_cast<const uint8_t*>(g_smem + (T.sm_rbr + (it & 1) * ((T.nslots + 3) / 4)) * 32) + (threadIdx.x & 31)};
+  return RevTape{S.at(rev_lam_at<ROWS>(T, it)), S.at(rev_lam_at<ROWS>(T, it - 1)), S.at(rev_vw_at<ROWS>(T, it)),
+                 reinterpret_cast<const uint8_t*>(g_smem + rev_br_at<ROWS>(T, it) * 32) + (threadIdx.x & 31)};
 }
 // n bytes of the tape record (a multiple of 16, like both addresses) into unit `unit`, asynchronously.
 __device__ __forceinline__ void rev_copy(int unit, const uint8_t* src, int n) {
@@ -133,33 +154,37 @@ __device__ __forceinline__ void rev_copy(int unit, const uint8_t* src, int n) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + o), "l"(src + o) : "memory");
 }
 // Impulses after sweep `it` (-1: before the first one) into the ring of three sweeps.
+template <bool ROWS>
 __device__ __forceinline__ void rev_stage_lam(const DevTopo& T, const TapeStep& tp, int it) {
-  const int unit = T.sm_rlam + (it + 3) % 3 * T.nslots, n = T.nslots * 128;
+  const int unit = rev_lam_at<ROWS>(T, it), n = T.nslots * 128;
   if (it >= 0) rev_copy(unit, tp.rec + T.rec_lam + (size_t)it * n, n);
   else if (T.ws) rev_copy(unit, tp.rec + T.rec_lam0, n);
   else
     for (int f = threadIdx.x; f < T.nslots * 32; f += blockDim.x) g_smem[unit * 32 + f] = 0.f;
 }
 // Velocities after sweep `it` and its clamp branches (two buffers each).
+template <bool ROWS>
 __device__ __forceinline__ void rev_stage_sweep(const DevTopo& T, const TapeStep& tp, int it) {
   const int nv = 6 * T.nb * 128, nb = T.nslots * 32;
-  rev_copy(T.sm_vw + (it & 1) * 6 * T.nb, tp.rec + T.rec_viter + (size_t)it * nv, nv);
-  rev_copy(T.sm_rbr + (it & 1) * ((T.nslots + 3) / 4), tp.rec + T.rec_br + (size_t)it * nb, nb);
+  rev_copy(rev_vw_at<ROWS>(T, it), tp.rec + T.rec_viter + (size_t)it * nv, nv);
+  rev_copy(rev_br_at<ROWS>(T, it), tp.rec + T.rec_br + (size_t)it * nb, nb);
 }
 // The last sweep's lines, asked for at the start of a step.
+template <bool ROWS>
 __device__ __forceinline__ void rev_stage_first(const DevTopo& T, const TapeStep& tp) {
-  rev_stage_lam(T, tp, T.iters - 1);
-  rev_stage_lam(T, tp, T.iters - 2);
-  rev_stage_sweep(T, tp, T.iters - 1);
+  rev_stage_lam<ROWS>(T, tp, T.iters - 1);
+  rev_stage_lam<ROWS>(T, tp, T.iters - 2);
+  rev_stage_sweep<ROWS>(T, tp, T.iters - 1);
 }
 // Waits for sweep `it`'s lines and asks for those of the sweep before it (every warp calls). Read from
 // L2 where they are used, at the head of every block's chain, they cost more than the rows.
+template <bool ROWS>
 __device__ __forceinline__ void rev_begin_sweep(const DevTopo& T, const TapeStep& tp, int it) {
   asm volatile("cp.async.wait_all;" ::: "memory");
   cta_sync();
   if (it > 0) {
-    rev_stage_lam(T, tp, it - 2);
-    rev_stage_sweep(T, tp, it - 1);
+    rev_stage_lam<ROWS>(T, tp, it - 2);
+    rev_stage_sweep<ROWS>(T, tp, it - 1);
   }
 }
 
@@ -411,21 +436,29 @@ __device__ __forceinline__ void rev_pair(const DevTopo& T, const SL& S, const Re
 }
 
 // The sweeps backwards (every warp calls; ends after a CTA barrier). On entry VB holds the adjoint
-// of the solver's output velocities, on exit that of its input velocities. ONE: the robot may be of one
-// block, whose warp keeps the bodies' adjoints in registers over the sweeps.
-template <bool ONE>
+// of the solver's output velocities, on exit that of its input velocities. ROWS: the sums row by row
+// (compiled topologies, dp_blk_rows.cuh); else the robot may be of one block, whose warp keeps the bodies'
+// adjoints in registers over the sweeps.
+template <bool ROWS>
 __device__ __forceinline__ void blk_sweeps_rev(const DevTopo& T, const SL& S, const TapeStep& tp, int warp) {
   const uint8_t* st0 = blk_bytes(T) + T.blk_stream + warp * T.blk_stream_len;
-  auto rows = [&](const BlkOp& op, const RevTape& rt, RevBody& A, RevBody& B, const auto& ready) {
+  using Body = std::conditional_t<ROWS, RowBody, RevBody>;
+  auto rows = [&](const BlkOp& op, const RevTape& rt, Body& A, Body& B, const auto& ready) {
     const int type = op.type(), idx = op.idx();
-    if (type == BT_GROUND) rev_contact(T, S, rt, op, contact_rec(T, S, idx), A, ready);
+    if constexpr (ROWS) {  // (a compiled topology has no sphere pairs)
+      if (type == BT_GROUND) rx_contact(T, S, rt, op, contact_rec(T, S, idx), A, ready);
+      else if (type == BT_JOINT) {
+        if (op.mask() == 31) rx_joint<true>(T, S, rt, op, joint_rec(T, S, idx), A, B, ready);
+        else rx_joint<false>(T, S, rt, op, joint_rec(T, S, idx), A, B, ready);
+      } else rx_hinge(T, S, rt, op, joint_rec(T, S, idx), A, B, ready);
+    } else if (type == BT_GROUND) rev_contact(T, S, rt, op, contact_rec(T, S, idx), A, ready);
     else if (type == BT_JOINT) {
       if (op.mask() == 31) rev_joint<true>(T, S, rt, op, joint_rec(T, S, idx), A, B, ready);
       else rev_joint<false>(T, S, rt, op, joint_rec(T, S, idx), A, B, ready);
     } else if (type == BT_PAIR) rev_pair(T, S, rt, op, pair_rec(T, S, idx), A, B, ready);
     else rev_hinge(T, S, rt, op, joint_rec(T, S, idx), idx, A, B, ready);
   };
-  if (ONE && T.blk_single) {
+  if constexpr (!ROWS) if (T.blk_single) {
     const bool on = warp == 0 && st0[0] != 0;
     const BlkOp op = blk_op(T, 0);
     const int a = op.a(), b = op.b();
@@ -436,8 +469,8 @@ __device__ __forceinline__ void blk_sweeps_rev(const DevTopo& T, const SL& S, co
     rev_load(T, S, vw, a, A);
     rev_load(T, S, vw, b, B);
     for (int it = T.iters - 1; it >= 0; --it) {
-      rev_begin_sweep(T, tp, it);
-      const RevTape rt = rev_tape(T, S, it);
+      rev_begin_sweep<ROWS>(T, tp, it);
+      const RevTape rt = rev_tape<ROWS>(T, S, it);
       if (!on) continue;
       vw = rt.vw;
       if (a >= 0) { A.v = vw.v3(6 * a); A.w = vw.v3(6 * a + 3); }
@@ -449,8 +482,8 @@ __device__ __forceinline__ void blk_sweeps_rev(const DevTopo& T, const SL& S, co
     return;
   }
   for (int it = T.iters - 1; it >= 0; --it) {
-    rev_begin_sweep(T, tp, it);
-    const RevTape rt = rev_tape(T, S, it);
+    rev_begin_sweep<ROWS>(T, tp, it);
+    const RevTape rt = rev_tape<ROWS>(T, S, it);
     const uint8_t* st = st0;
     int e = *st++;
     bool pend = false;  // a level's barrier to meet before the next velocities are read
@@ -462,16 +495,28 @@ __device__ __forceinline__ void blk_sweeps_rev(const DevTopo& T, const SL& S, co
       if (e & BS_OP) {
         const int a = op.a(), b = op.b(), type = op.type();
         const bool lin = type <= BT_JOINT || type >= BT_GROUND;
-        RevBody A, B;
-        rev_init(T, S, a, A);
-        rev_init(T, S, b, B);
-        rows(op, rt, A, B, [&] {
-          if (pend) cta_sync();
-          rev_load(T, S, rt.vw, a, A);
-          rev_load(T, S, rt.vw, b, B);
-        });
-        rev_store(T, S, rt.vw, a, A, lin);
-        rev_store(T, S, rt.vw, b, B, lin);
+        Body A, B;
+        if constexpr (ROWS) {
+          rx_init(T, S, a, A);
+          rx_init(T, S, b, B);
+          rows(op, rt, A, B, [&] {
+            if (pend) cta_sync();
+            rx_load(T, S, rt.vw, a, A);
+            rx_load(T, S, rt.vw, b, B);
+          });
+          rx_store(T, S, rt.vw, a, A, lin);
+          rx_store(T, S, rt.vw, b, B, lin);
+        } else {
+          rev_init(T, S, a, A);
+          rev_init(T, S, b, B);
+          rows(op, rt, A, B, [&] {
+            if (pend) cta_sync();
+            rev_load(T, S, rt.vw, a, A);
+            rev_load(T, S, rt.vw, b, B);
+          });
+          rev_store(T, S, rt.vw, a, A, lin);
+          rev_store(T, S, rt.vw, b, B, lin);
+        }
       } else if (pend) {
         cta_sync();
       }
@@ -963,6 +1008,21 @@ __device__ __forceinline__ void hinge_reverse_body(const DevTopo& T, const RevCt
   for (int q = 0; q < 9; ++q) C.XB[18 * b + 3 + q] = gR[q];
 }
 
+// Every joint's hinge kinematics reversed (every warp calls; ends after a CTA barrier).
+template <class Q>
+__device__ __forceinline__ void blk_hinge_reverse(const DevTopo& T, const RevCtx& C, int warp) {
+  if constexpr (Q::SEQ) {
+    for (int j = warp; j < T.nj; j += blk_nw()) rx_hinge_item(T, C, j);
+    cta_sync();
+    for (int b = warp; b < T.nb; b += blk_nw()) rx_hinge_body(T, C, b);
+  } else {
+    for (int j = warp; j < T.nj; j += blk_nw()) hinge_reverse_item(T, C, j);
+    cta_sync();
+    for (int b = warp; b < T.nb; b += blk_nw()) hinge_reverse_body(T, C, b);
+  }
+  cta_sync();
+}
+
 // Features reversed, split: angle and rate adjoints to the joints of this warp; the rest (torso
 // sensors, target vector) to the pose adjoint by warp 3, when no other warp writes it.
 template <class AV>
@@ -1198,7 +1258,7 @@ __device__ __forceinline__ void blk_reverse_step(const DevTopo& T, const DevPtrs
   const TapeStep tp = tape_step(T, D, ts);
   const LaneT<SL> L{S, C.P, S, i};
   const BLaneT<SL> Bl{L, C.X, C.G, GC{tp.vminus, 32}};
-  rev_stage_first(T, tp);
+  rev_stage_first<Q::SEQ>(T, tp);
   if (load_x1)
     for (int f = warp; f < nf; f += blk_nw()) C.X[f] = x_t1[(size_t)f * Bp + i];
   if (T.grad_decay != 1.f) {  // section 3.2: the adjoint from later steps shrinks by alpha per step
@@ -1215,8 +1275,9 @@ __device__ __forceinline__ void blk_reverse_step(const DevTopo& T, const DevPtrs
 #pragma unroll
     for (int f = 0; f < 18; ++f) C.X[18 * b + f] = x_t[(size_t)(18 * b + f) * Bp + i];
     S[T.sm_invmb + b] = 0.f;
+    constexpr int n9 = Q::SEQ ? 9 : 6;
 #pragma unroll
-    for (int q = 0; q < 6; ++q) S[T.sm_iinvb + 6 * b + q] = 0.f;
+    for (int q = 0; q < n9; ++q) S[T.sm_iinvb + n9 * b + q] = 0.f;
   }
   for (int s = warp; s < T.nslots; s += blk_nw()) S[T.sm_lam + s] = 0.f;  // impulse adjoints
   inverse_inertia(T, L, C.X, mine);
@@ -1228,18 +1289,27 @@ __device__ __forceinline__ void blk_reverse_step(const DevTopo& T, const DevPtrs
   servo_targets(T, L, au, mine);
   blk_assemble<false>(T, S, C.P, C.X, VelTape{GS{tp.vminus}}, nullptr, warp);
   for (int j = warp; j < T.nj; j += blk_nw())
-    for (int q = 0; q < JA_N; ++q) joint_rec(T, S, j)[JR_N + q] = 0.f;
+    for (int q = 0; q < (Q::SEQ ? JX_N : JA_N); ++q) joint_rec(T, S, j)[JR_N + q] = 0.f;
   for (int c = warp; c < T.ns; c += blk_nw())
-    for (int q = 0; q < CA_N; ++q) contact_rec(T, S, c)[CR_N + q] = 0.f;
-  for (int c = warp; c < T.np; c += blk_nw())
-    for (int q = 0; q < PA_N; ++q) pair_rec(T, S, c)[PR_N + q] = 0.f;
+    for (int q = 0; q < (Q::SEQ ? CX_N : CA_N); ++q) contact_rec(T, S, c)[CR_N + q] = 0.f;
+  if constexpr (!Q::SEQ)
+    for (int c = warp; c < T.np; c += blk_nw())
+      for (int q = 0; q < PA_N; ++q) pair_rec(T, S, c)[PR_N + q] = 0.f;
   cta_sync();
   blk_stream(T, warp, true);
-  blk_sweeps_rev<!Q::SEQ>(T, S, tp, warp);
+  blk_sweeps_rev<Q::SEQ>(T, S, tp, warp);
   const bool ws = T.ws != 0;
-  for (int j = warp; j < T.nj; j += blk_nw()) joint_reverse(T, C, tp, ws, j);
-  for (int q = warp; q < T.ns; q += blk_nw()) contact_reverse(T, C, tp, ws, q);
-  for (int p = warp; p < T.np; p += blk_nw()) pair_reverse(T, C, tp, ws, p);
+  if constexpr (Q::SEQ) {
+    // the sweeps' staging buffers lay over x_t
+    for (int f = warp; f < nf; f += blk_nw()) C.X[f] = x_t[(size_t)f * Bp + i];
+    cta_sync();
+    for (int j = warp; j < T.nj; j += blk_nw()) rx_joint_item(T, C, tp, ws, j);
+    for (int q = warp; q < T.ns; q += blk_nw()) rx_contact_item(T, C, tp, ws, q);
+  } else {
+    for (int j = warp; j < T.nj; j += blk_nw()) joint_reverse(T, C, tp, ws, j);
+    for (int q = warp; q < T.ns; q += blk_nw()) contact_reverse(T, C, tp, ws, q);
+    for (int p = warp; p < T.np; p += blk_nw()) pair_reverse(T, C, tp, ws, p);
+  }
   // servo targets: the joint's warp has its adjoint
   const SL zb = S.at(T.sm_zb);
   const int nout = T.n_layers > 0 ? T.widths[T.n_layers] : 0;
@@ -1268,7 +1338,12 @@ __device__ __forceinline__ void blk_reverse_step(const DevTopo& T, const DevPtrs
     }
   }
   cta_sync();
-  for (int b = warp; b < T.nb; b += blk_nw()) body_reverse(T, C, b);
+  if constexpr (Q::SEQ) {
+    for (int b = warp; b < T.nb; b += blk_nw()) rx_body(T, C, ws, b);
+    external_reverse(T, Bl, C.XB, C.VB, mine);
+  } else {
+    for (int b = warp; b < T.nb; b += blk_nw()) body_reverse(T, C, b);
+  }
   if (T.ext_ctrl) {
     // wide controller: the output adjoint goes to the batched products; the features' adjoint comes
     // back into the next launch
@@ -1307,10 +1382,7 @@ __device__ __forceinline__ void blk_reverse_step(const DevTopo& T, const DevPtrs
   } else {
     cta_sync();
   }
-  for (int j = warp; j < T.nj; j += blk_nw()) hinge_reverse_item(T, C, j);
-  cta_sync();
-  for (int b = warp; b < T.nb; b += blk_nw()) hinge_reverse_body(T, C, b);
-  cta_sync();
+  blk_hinge_reverse<Q>(T, C, warp);
 }
 
 __device__ __forceinline__ void blk_loss_initial_reverse(const DevTopo& T, const DevPtrs& D, const RevCtx& C) {
@@ -1431,10 +1503,7 @@ __global__ void __launch_bounds__(32 * Q::NW, 1) k_backward_ext_blk(const __grid
     const GC sbar{D.sbar_ext + (size_t)i * T.ext_k0p, 1};
     features_reverse_joints(T, C.S, sbar, warp);
     if (warp == 3) features_reverse_rest(T, C, sbar);
-    for (int j = warp; j < T.nj; j += blk_nw()) hinge_reverse_item(T, C, j);
-    cta_sync();
-    for (int b = warp; b < T.nb; b += blk_nw()) hinge_reverse_body(T, C, b);
-    cta_sync();
+    blk_hinge_reverse<Q>(T, C, warp);
   }
   if (t >= 0) {
     blk_reverse_step<Q>(T, D, C, t, t, D.ckpt + (size_t)t * sb, D.state, tn >= Tw, warp);
@@ -1459,5 +1528,13 @@ static cudaError_t launch_backward_blk_t(const DevTopo& T, const DevTopo& Ts, co
     if (e != cudaSuccess) return e;
     k_backward_seg_blk<Q><<<T.Bp / 32, 32 * T.blk_nw, smem, s>>>(T, Ts, D);
   }
+  return cudaGetLastError();
+}
+template <class Q>
+static cudaError_t launch_backward_ext_blk_t(const DevTopo& T, const DevPtrs& D, int t, cudaStream_t s) {
+  const size_t smem = (size_t)T.sm_total * 128;
+  cudaError_t e = cudaFuncSetAttribute(k_backward_ext_blk<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_backward_ext_blk<Q><<<T.Bp / 32, 32 * T.blk_nw, smem, s>>>(T, D, t);
   return cudaGetLastError();
 }

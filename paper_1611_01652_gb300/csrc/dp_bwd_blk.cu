@@ -11,11 +11,8 @@ cudaError_t launch_backward_blk(const DevTopo& T, const DevTopo& Ts, const DevPt
   if (T.mlp_tc && T.widths[1] == BlkArm::CTRL_H) return launch_backward_blk_arm(T, Ts, D, s);
   return launch_backward_blk_quad(T, Ts, D, s);
 }
-// (the wide controller's launches run no network: one kernel for every robot)
+// (the wide controller's launches run no network: one kernel for every compiled topology)
 cudaError_t launch_backward_ext_blk(const DevTopo& T, const DevPtrs& D, int t, cudaStream_t s) {
-  const size_t smem = (size_t)T.sm_total * 128;
-  cudaError_t e = cudaFuncSetAttribute(k_backward_ext_blk<BlkQuad>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  k_backward_ext_blk<BlkQuad><<<T.Bp / 32, 32 * T.blk_nw, smem, s>>>(T, D, t);
-  return cudaGetLastError();
+  if (T.topo_id == 0) return launch_backward_ext_blk_dyn(T, D, t, s);
+  return launch_backward_ext_blk_t<BlkQuad>(T, D, t, s);
 }

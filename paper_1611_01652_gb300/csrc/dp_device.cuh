@@ -22,6 +22,10 @@
 #define DPK_ST_NAN_STATE 1
 #define DPK_ST_NAN_GRAD 2
 
+// Fields of a joint's and a contact's record in the reverse pass of a compiled topology (dp_blk_rows.cuh).
+#define RX_REC_J 86
+#define RX_REC_C 23
+
 // Warm-start group types (feature 15 of a group).
 enum { WSG_GROUND = 0, WSG_PAIR = 1, WSG_JOINT = 2, WSG_HINGE = 3 };
 
@@ -95,7 +99,8 @@ struct DevTopo {
   int blk_fwd, blk_bwd;  // 1: rollouts and steps / reverse passes of this world run on the four-warp step
   int rec_rows;          // 1: the tape records hold the constraint rows (read by the one-warp reverse)
   int rec_j, rec_c, rec_p;  // strides of the joints', contacts' and pairs' records
-  int sm_rlam, sm_rbr;   // four-warp reverse: staged tape lines (impulses, clamp branches)
+  int sm_rlam, sm_rbr;   // reverse on blocks: staged tape lines (impulses, clamp branches), and where the
+  int sm_rlam2, sm_vw2, sm_rbr2;  // third sweep's impulses and the second's velocities and branches go
   int sm_hbuf;           // controller buffers over the records (bfloat16 activations or delta planes, or ping-pong)
   int cslot;
   int16_t jslot[DPK_MAXJ], jlim[DPK_MAXJ], jmot[DPK_MAXJ];

@@ -34,6 +34,7 @@ cudaError_t launch_backward_blk(const DevTopo& T, const DevTopo& Ts, const DevPt
 cudaError_t launch_backward_blk_quad(const DevTopo& T, const DevTopo& Ts, const DevPtrs& D, cudaStream_t s);
 cudaError_t launch_backward_blk_arm(const DevTopo& T, const DevTopo& Ts, const DevPtrs& D, cudaStream_t s);
 cudaError_t launch_backward_blk_dyn(const DevTopo& T, const DevTopo& Ts, const DevPtrs& D, cudaStream_t s);
+cudaError_t launch_backward_ext_blk_dyn(const DevTopo& T, const DevPtrs& D, int t, cudaStream_t s);
 cudaError_t launch_backward_ext_blk(const DevTopo& T, const DevPtrs& D, int t, cudaStream_t s);
 cudaError_t launch_backward_ext(const DevTopo& T, const DevPtrs& D, int t, cudaStream_t s);
 cudaError_t launch_dw(const float* del, const float* act, int M, int C, size_t N, float* partial, int splits,
