@@ -25,7 +25,10 @@ enum { CA_RA = 0, CA_ME = 3, CA_BI = 6, CA_MU = 7, CA_N = 8 };
 enum { PA_LIN = 0, PA_ANGA = 9, PA_ANGB = 18, PA_ME = 27, PA_BI = 30, PA_MU = 31, PA_N = 32 };
 enum { JP_P = 0, JP_RA = 3, JP_RB = 12, JP_SA = 21, JP_SB = 27, JP_IA = 33, JP_IB = 34, JP_N = 35 };
 enum { CP_Z = 0, CP_R = 1, CP_S = 10, CP_I = 16, CP_V = 17, CP_W = 18, CP_N = 21 };
-enum { PP_P = 0, PP_RA = 3, PP_RB = 12, PP_SA = 21, PP_SB = 27, PP_IA = 33, PP_IB = 34, PP_V = 35, PP_WA = 38, PP_WB = 41, PP_N = 44 };
+enum { PP_P = 0, PP_RA = 3, PP_RB = 12, PP_SA = 21, PP_SB = 27, PP_IA = 33, PP_IB = 34, PP_V = 35, PP_WA = 38, PP_WB = 41, PP_GK = 44, PP_GL = 50, PP_N = 56 };
+// A pair's share of its two spheres' parameter gradients (at PP_GK and PP_GL): offset, radius, friction,
+// restitution.
+enum { PG_OFF = 0, PG_RAD = 3, PG_MU = 4, PG_E = 5 };
 enum { HP_W = 0, HP_RA = 3, HP_RB = 12, HP_N = 21 };
 
 // One body of a block: velocities, their adjoints, inverse mass and inertia, and the block's sums
@@ -757,7 +760,8 @@ static __device__ __noinline__ void pair_reverse(const DevTopo& T, const RevCtx&
   const SL Q = R.at(PR_N);
   float sa[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, sb[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, ima_b = 0.f, imb_b = 0.f;
   const float3 z3 = f3(0.f, 0.f, 0.f);
-  float3 dlb = z3, ckb = z3, clb = z3, vadd = z3, wadda = z3, waddb = z3;
+  float3 dlb = z3, ckb = z3, clb = z3, vadd = z3, wadda = z3, waddb = z3, goffk = z3, goffl = z3;
+  float rkb = 0.f, rlb = 0.f, muk_b = 0.f, mul_b = 0.f, ek_b = 0.f, el_b = 0.f;
   const float3 offk = C.P.v3(T.o_sph_off + 3 * k), offl = C.P.v3(T.o_sph_off + 3 * l);
   if (R[PF_ME] != 0.f) {
     float ia[6], ib[6];
@@ -774,7 +778,7 @@ static __device__ __noinline__ void pair_reverse(const DevTopo& T, const RevCtx&
     const float rk = C.P[T.o_sph_rad + k], rl = C.P[T.o_sph_rad + l];
     const float3 ra = ck - rk * n, rb = cl + rl * n;
     float3 nb = z3;
-    float distb = 0.f, rkb = 0.f, rlb = 0.f;
+    float distb = 0.f;
     for (int m = 0; m < 3; ++m) {
       const float me = R[PF_ME + m], Kb = -me * me * Q[PA_ME + m];
       const float3 lin = R.v3(PF_LIN + 3 * m), angA = R.v3(PF_ANGA + 3 * m), angB = R.v3(PF_ANGB + 3 * m);
@@ -808,7 +812,7 @@ static __device__ __noinline__ void pair_reverse(const DevTopo& T, const RevCtx&
         if (dist - rk - rl + T.slop < 0.f) distb += bh * biasb;
         if (vn < 0.f) {
           const float ek = C.P[T.o_sph_e + k], el = C.P[T.o_sph_e + l];
-          C.G.red(T.o_sph_e + (ek >= el ? k : l), vn * biasb);
+          (ek >= el ? ek_b : el_b) = vn * biasb;
           const float vnb = (ek >= el ? ek : el) * biasb;
           nb += vnb * (vma - vmb);
           vadd = vnb * n;
@@ -824,8 +828,8 @@ static __device__ __noinline__ void pair_reverse(const DevTopo& T, const RevCtx&
         const float muk = C.P[T.o_sph_mu + k], mul = C.P[T.o_sph_mu + l], mu = sqrtf(muk * mul);
         if (m == 1 && mu > 0.f) {
           const float mub = Q[PA_MU];
-          C.G.red(T.o_sph_mu + k, mub * mul / (2.f * mu));
-          C.G.red(T.o_sph_mu + l, mub * muk / (2.f * mu));
+          muk_b = mub * mul / (2.f * mu);
+          mul_b = mub * muk / (2.f * mu);
         }
       }
       const float3 rab = cross3(lin, angAb), rbb = -cross3(lin, angBb);
@@ -838,10 +842,8 @@ static __device__ __noinline__ void pair_reverse(const DevTopo& T, const RevCtx&
     dlb = deg ? z3 : distb * n + (1.f / dist) * (nb - dot3(n, nb) * n);
     ckb += dlb;
     clb -= dlb;
-    C.G.red3(T.o_sph_off + 3 * k, mtv(Ra, ckb));
-    C.G.red3(T.o_sph_off + 3 * l, mtv(Rb, clb));
-    C.G.red(T.o_sph_rad + k, rkb);
-    C.G.red(T.o_sph_rad + l, rlb);
+    goffk = mtv(Ra, ckb);
+    goffl = mtv(Rb, clb);
   }
   R.s3(PP_P, dlb);
   const float v[3] = {ckb.x, ckb.y, ckb.z}, c[3] = {offk.x, offk.y, offk.z};
@@ -853,6 +855,24 @@ static __device__ __noinline__ void pair_reverse(const DevTopo& T, const RevCtx&
   R.s3(PP_V, vadd);
   R.s3(PP_WA, wadda);
   R.s3(PP_WB, waddb);
+  R.s3(PP_GK + PG_OFF, goffk);
+  R[PP_GK + PG_RAD] = rkb; R[PP_GK + PG_MU] = muk_b; R[PP_GK + PG_E] = ek_b;
+  R.s3(PP_GL + PG_OFF, goffl);
+  R[PP_GL + PG_RAD] = rlb; R[PP_GL + PG_MU] = mul_b; R[PP_GL + PG_E] = el_b;
+}
+
+// The pairs' shares of sphere q's parameter gradients, in pair order (the sphere's contact has added its
+// own, before the barrier). Several pairs and the ground contact of a sphere belong to different warps:
+// added where they are formed, their order, and the sums' last bits, would change from run to run.
+__device__ __forceinline__ void sphere_reverse(const DevTopo& T, const RevCtx& C, int q) {
+  for (int p = 0; p < T.np; ++p) {
+    if (!blk_live(T)[T.nj + T.ns + p] || (T.pk[p] != q && T.pl[p] != q)) continue;
+    const SL R = pair_rec(T, C.S, p).at(T.pk[p] == q ? PP_GK : PP_GL);
+    C.G.red3(T.o_sph_off + 3 * q, R.v3(PG_OFF));
+    C.G.red(T.o_sph_rad + q, R[PG_RAD]);
+    C.G.red(T.o_sph_mu + q, R[PG_MU]);
+    C.G.red(T.o_sph_e + q, R[PG_E]);
+  }
 }
 
 // Body b: the packages of its items (slot order) into the pose adjoint and the adjoints of the
@@ -1343,6 +1363,8 @@ __device__ __forceinline__ void blk_reverse_step(const DevTopo& T, const DevPtrs
     external_reverse(T, Bl, C.XB, C.VB, mine);
   } else {
     for (int b = warp; b < T.nb; b += blk_nw()) body_reverse(T, C, b);
+    if (T.np)
+      for (int q = warp; q < T.ns; q += blk_nw()) sphere_reverse(T, C, q);
   }
   if (T.ext_ctrl) {
     // wide controller: the output adjoint goes to the batched products; the features' adjoint comes
