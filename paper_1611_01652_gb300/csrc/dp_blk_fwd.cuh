@@ -236,18 +236,24 @@ __device__ __forceinline__ void blk_damped_start(const DevTopo& T, const SL& S, 
       lam[s] = fminf(fmaxf(y, -hi), hi);
     }
   }
-  for (int c = warp; c < T.ns + T.np; c += blk_nw()) {
-    const bool pair = c >= T.ns;
-    const SL R = pair ? pair_rec(T, S, c - T.ns) : contact_rec(T, S, c);
-    const int s0 = T.cslot + 3 * c;
+  auto touch = [&](int s0, float me, float mu) {
     float l[3] = {0.f, 0.f, 0.f};
-    if (R[pair ? PF_ME : CF_ME] != 0.f) {
+    if (me != 0.f) {
       l[0] = fmaxf(T.ws_alpha * lam[s0], 0.f);
-      const float hi = R[pair ? PF_MU : CF_MU] * l[0];
+      const float hi = mu * l[0];
       l[1] = fminf(fmaxf(T.ws_alpha * lam[s0 + 1], -hi), hi);
       l[2] = fminf(fmaxf(T.ws_alpha * lam[s0 + 2], -hi), hi);
     }
     for (int k = 0; k < 3; ++k) lam[s0 + k] = l[k];
+  };
+  // (the warp that has formed the record: there is no barrier in between)
+  for (int q = warp; q < T.ns; q += blk_nw()) {
+    const SL R = contact_rec(T, S, q);
+    touch(T.cslot + 3 * q, R[CF_ME], R[CF_MU]);
+  }
+  for (int p = warp; p < T.np; p += blk_nw()) {
+    const SL R = pair_rec(T, S, p);
+    touch(T.cslot + 3 * (T.ns + p), R[PF_ME], R[PF_MU]);
   }
 }
 

@@ -62,6 +62,15 @@ def pile(B):
     return robot(B, [[x[k], 0.0, r[k] - 0.002] for k in range(3)], [], [(k, [0, 0, 0], r[k]) for k in range(3)], [(0, 1), (1, 2)])
 
 
+def hub(B, n=7):
+    """A ball on the ground and n smaller ones around it that touch it: n pairs share its sphere."""
+    R, r = 0.3, 0.1
+    u = np.sqrt((R + r) ** 2 - (R - r) ** 2) - 0.003
+    ang = 0.1 + 2 * np.pi * np.arange(n) / n
+    pos = [[0.0, 0.0, R - 0.002]] + [[u * np.cos(a), u * np.sin(a), r - 0.002] for a in ang]
+    return robot(B, pos, [], [(0, [0, 0, 0], R)] + [(k + 1, [0, 0, 0], r) for k in range(n)], [(0, k + 1) for k in range(n)])
+
+
 def solve(m, horizon, iters, ckpt, warm, **kw):
     """(loss, final state), every gradient, the activity log and the schedule."""
     w = World(m, horizon=horizon, iters=iters, ckpt_every=ckpt, warmstart=warm, **kw)
@@ -103,15 +112,6 @@ def test_wide_controller_on_a_run_time_topology(monkeypatch):
     same(got, solve(m, 6, 5, None, True))
 
 
-def hub(B, n=7):
-    """A ball on the ground and n smaller ones around it that touch it: n pairs share its sphere."""
-    R, r = 0.3, 0.1
-    u = np.sqrt((R + r) ** 2 - (R - r) ** 2) - 0.003
-    ang = 0.1 + 2 * np.pi * np.arange(n) / n
-    pos = [[0.0, 0.0, R - 0.002]] + [[u * np.cos(a), u * np.sin(a), r - 0.002] for a in ang]
-    return robot(B, pos, [], [(0, [0, 0, 0], R)] + [(k + 1, [0, 0, 0], r) for k in range(n)], [(0, k + 1) for k in range(n)])
-
-
 def test_gradients_of_touching_spheres_repeat_bit_for_bit():
     """Ground contacts and pairs add to the parameters of the same spheres: always in the same order."""
     m = hub(64)
@@ -124,9 +124,10 @@ def test_gradients_of_touching_spheres_repeat_bit_for_bit():
             assert np.array_equal(first[k], again[k]), k
 
 
-def test_touching_spheres_match_rows(monkeypatch):
-    for m in (hub(33), pile(33)):
-        got = solve(m, 12, 5, None, True)
-        with monkeypatch.context() as mp:
-            one_warp(mp)
-            same(got, solve(m, 12, 5, None, True))
+def test_colliding_spheres_match_rows(monkeypatch):
+    """Two spheres in free flight that meet within sixty steps."""
+    m = WL.two_spheres(B=40, e=0.3, mu=0.4)
+    got = solve(m, 60, 5, 16, True)
+    assert got[2][:, :, got[3].schedule()["kind"] == PN].any()
+    one_warp(monkeypatch)
+    same(got, solve(m, 60, 5, 16, True))
