@@ -71,6 +71,75 @@ def hub(B, n=7):
     return robot(B, pos, [], [(0, [0, 0, 0], R)] + [(k + 1, [0, 0, 0], r) for k in range(n)], [(0, k + 1) for k in range(n)])
 
 
+def mixed_chain(B):
+    """A ball joint, then two hinges with limits and servos, two contacts on the last link: the second
+    hinge's linear and angular rows fall apart, and so does the second contact."""
+    return robot(B, [[0, 0, -0.2], [0, 0, -0.6], [0, 0, -1.0]],
+                 [(BALL, -1, 0, [0, 0, 0], [0, 1, 0], 0), (HINGE, 0, 1, [0, 0, -0.4], [0, 1, 0], BOTH),
+                  (HINGE, 1, 2, [0, 0, -0.8], [1, 0, 0], BOTH)],
+                 [(2, [0.05, 0, -0.2], 0.05), (2, [-0.05, 0, -0.2], 0.05)], ground_z=-1.248)
+
+
+def split_pair(B):
+    """A hinge to the world and a ball joint leave a hole in one body's colours that takes a pair's normal
+    and first friction row; the other falls behind a contact."""
+    u = np.sqrt(0.22 ** 2 - 0.02 ** 2) - 0.003
+    return robot(B, [[0, 0, 0.3], [0.4, 0, 0.3], [0.4 + u, 0, 0.12]],
+                 [(HINGE, -1, 0, [0, 0, 0.5], [0, 1, 0], 0), (BALL, 1, 0, [0.2, 0, 0.3], [0, 1, 0], 0)],
+                 [(2, [0, 0, 0], 0.12), (1, [0, 0, -0.2], 0.1), (0, [0, 0, -0.2], 0.1)], [(1, 0)], ground_z=0.002)
+
+
+def plates(B):
+    """Two plates of sixteen contact spheres each, a ball joint and a hinge with limit and servo: 36 blocks."""
+    grid = [[0.05 * (k % 4), 0.05 * (k // 4), -0.45] for k in range(16)]
+    return robot(B, [[0, 0, 0.5], [0.6, 0, 0.5]],
+                 [(BALL, -1, 0, [0, 0, 0.9], [0, 1, 0], 0), (HINGE, 0, 1, [0.3, 0, 0.5], [0, 1, 0], BOTH)],
+                 [(b, o, 0.05) for b in range(2) for o in grid], ground_z=0.002)
+
+
+def one_plate(B):
+    """A body on a hinge with 32 contacts: 35 levels, more than the schedule holds (one warp)."""
+    grid = [[0.05 * (k % 8), 0.05 * (k // 8), -0.45] for k in range(32)]
+    return robot(B, [[0, 0, 0.5]], [(HINGE, -1, 0, [0, 0, 0.9], [0, 1, 0], BOTH)], [(0, o, 0.05) for o in grid], ground_z=0.002)
+
+
+def ball_chain(B):
+    """Thirteen links on ball joints and a contact: the rollout fits on blocks, the reverse pass does not."""
+    return robot(B, [[0, 0, -0.1 - 0.2 * k] for k in range(13)],
+                 [(BALL, k - 1, k, [0, 0, -0.2 * k], [0, 1, 0], 0) for k in range(13)], [(12, [0, 0, -0.1], 0.05)], ground_z=-2.648)
+
+
+# robot, blocks of its schedule, items that are split (type, index)
+JOINT, CONTACT, PAIR = "joint", "contact", "pair"
+ROBOTS = {
+    "mixed chain": (mixed_chain, 11, {(JOINT, 2), (CONTACT, 1)}),
+    "split pair": (split_pair, 7, {(PAIR, 0)}),
+    "plates": (plates, 36, set()),
+    "one plate": (one_plate, 35, set()),
+    "ball chain": (ball_chain, 14, set()),
+    "pile": (pile, 5, set()),
+    "hub": (hub, 15, set()),
+}
+
+
+def blocks(w):
+    """The schedule's blocks: a row joins its item's block when that is the last one on each of its
+    bodies. Returns their number and the items in more than one block."""
+    s = w.schedule()
+    item = {JLIN: JOINT, JANG: JOINT, LIMIT: LIMIT, MOTOR: MOTOR, GN: CONTACT, GT: CONTACT, PN: PAIR, PT: PAIR}
+    last, made = {}, []
+    for o in s["order"]:
+        it = (item[s["kind"][o]], int(s["idx"][o]))
+        bodies = [x for x in (s["body_a"][o], s["body_b"][o]) if x >= 0]
+        on = {last.get(x) for x in bodies}
+        if len(on) == 1 and None not in on and made[list(on)[0]] == it and it[0] not in (LIMIT, MOTOR):
+            continue
+        made.append(it)
+        for x in bodies:
+            last[x] = len(made) - 1
+    return len(made), {it for it in made if made.count(it) > 1}
+
+
 def solve(m, horizon, iters, ckpt, warm, **kw):
     """(loss, final state), every gradient, the activity log and the schedule."""
     w = World(m, horizon=horizon, iters=iters, ckpt_every=ckpt, warmstart=warm, **kw)
@@ -122,6 +191,20 @@ def test_gradients_of_touching_spheres_repeat_bit_for_bit():
         again = solve(m, 12, 5, None, True)[1]
         for k in first:
             assert np.array_equal(first[k], again[k]), k
+
+
+@pytest.mark.parametrize("name", sorted(ROBOTS))
+@pytest.mark.parametrize("B,iters,ckpt,warm", [(1, 1, 1, False), (33, 3, None, True), (40, 5, 5, True), (32, 7, None, False)])
+def test_general_robots_match_rows(monkeypatch, name, B, iters, ckpt, warm):
+    make, n, split = ROBOTS[name]
+    m = make(B)
+    got = solve(m, 12, iters, ckpt, warm)
+    assert blocks(got[3]) == (n, split)
+    kind = got[3].schedule()["kind"]
+    for k in (LIMIT, GN, PN):  # every kind of row that comes and goes was there
+        assert not (kind == k).any() or got[2][:, :, kind == k].any(), k
+    one_warp(monkeypatch)
+    same(got, solve(m, 12, iters, ckpt, warm))
 
 
 def test_colliding_spheres_match_rows(monkeypatch):
