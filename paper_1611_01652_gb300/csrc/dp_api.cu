@@ -539,6 +539,7 @@ dp_status dp_create_world(const dp_batch_desc* d, void* stream, dp_world** out) 
   CU(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   plan_smem(w->Tf, false, smem_max / (int)sizeof(float), d->rows_global == 0);
   plan_smem(w->Tb, true, smem_max / (int)sizeof(float));
+  const DevTopo one = w->Tf;  // the one-warp layout
   // The four-warp step, unless the world asks for one warp per group or rows in global memory (or
   // the environment forces the one-warp kernels, for comparison).
   std::vector<int32_t> prog;
@@ -558,7 +559,7 @@ dp_status dp_create_world(const dp_batch_desc* d, void* stream, dp_world** out) 
     }
   }
   // only the one-warp reverse reads the rows from the tape
-  w->Tf.rec_rows = w->Tb.rec_rows = w->Ts.rec_rows = T.rec_rows = !w->Tb.blk_bwd;
+  T.rec_rows = !w->Tb.blk_bwd;
   size_t need = (size_t)std::max(w->Tf.sm_total, w->Tb.sm_total) * 32 * sizeof(float);
   if (need > (size_t)smem_max) {
     dp_status s = fail(DP_EINVAL, "robot too large: needs " + std::to_string(need) + " bytes of shared memory per warp, the device offers " +
@@ -587,15 +588,17 @@ dp_status dp_create_world(const dp_batch_desc* d, void* stream, dp_world** out) 
     T.rec_lam0 = o;
     if (d->warmstart) o += (long long)T.nslots * 32 * 4;
     T.rec_bytes = (o + 255) / 256 * 256;
-    for (DevTopo* t2 : {&w->Tf, &w->Tb, &w->Ts}) {
-      t2->rec_lam = T.rec_lam;
-      t2->rec_viter = T.rec_viter;
-      t2->rec_vminus = T.rec_vminus;
-      t2->rec_br = T.rec_br;
-      t2->rec_lam0 = T.rec_lam0;
-      t2->rec_bytes = T.rec_bytes;
-    }
   }
+  auto set_record = [&](DevTopo& t) {
+    t.rec_rows = T.rec_rows;
+    t.rec_lam = T.rec_lam;
+    t.rec_viter = T.rec_viter;
+    t.rec_vminus = T.rec_vminus;
+    t.rec_br = T.rec_br;
+    t.rec_lam0 = T.rec_lam0;
+    t.rec_bytes = T.rec_bytes;
+  };
+  for (DevTopo* t : {&w->Tf, &w->Tb, &w->Ts}) set_record(*t);
   const size_t tape_step_bytes = (size_t)T.rec_bytes * (Bp / 32);
   const size_t dump_bytes = (size_t)T.dump_rows * T.horizon * Bp * sizeof(float);
   size_t free_b = 0, total_b = 0;
@@ -632,6 +635,24 @@ dp_status dp_create_world(const dp_batch_desc* d, void* stream, dp_world** out) 
   D.n_ckpt = n_ckpt;
   D.tape_steps = tape_steps;
   D.tape_full = full ? 1 : 0;
+  // Recorded rollouts of robots without joints: a step is a few contact rows, and a warp that takes all of
+  // it needs 2.5 to 2.9 times as long as blocks do, but an SM holds seven or eight such groups and two on
+  // blocks. Which is faster goes by the waves. Measured, ms, one warp and blocks, at groups an SM: a ball,
+  // 60 steps of 20 sweeps, 4: 1.24, 0.93; 8: 1.34, 1.83; 10: 2.52, 2.29; 16: 2.66, 3.65; two spheres,
+  // 40 steps, 4: 1.31, 1.08; 7: 1.45, 2.07; 10: 2.78, 2.66; 14: 2.88, 3.71. (With joints blocks are faster
+  // by 2 to 6 at any size, but for a lone hinge: within an eighth of one warp from 8 groups an SM on.)
+  w->Tr = w->Tf;
+  if (full && w->Tf.blk_fwd && T.nj == 0 && one.sm_rows >= 0) {
+    int n1 = 0, n4 = 0, sms = 0;
+    CU(forward_groups_one_warp(one, &n1));
+    CU(forward_groups_blk_dyn(w->Tf, &n4));
+    CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    auto waves = [&](int n) { return (Bp / 32 + std::max(n, 1) * sms - 1) / (std::max(n, 1) * sms); };
+    if (11 * waves(n1) < 4 * waves(n4)) {
+      w->Tr = one;
+      set_record(w->Tr);
+    }
+  }
   // device buffers
   float* prm = nullptr;
   if (dalloc(w, &prm, (size_t)T.n_pfields * Bp)) return cleanup(DP_ENOMEM);
@@ -888,7 +909,7 @@ dp_status dp_rollout(dp_world* w, const float* W, float* loss, float* traj, uint
   if (w->Tf.ext_ctrl)
     CU(ext_forward(w, w->Tf, D, 0, w->Tf.horizon, 1, D.tape_full));
   else
-    CU(launch_forward(w->Tf, D, w->x0, 0, w->Tf.horizon, 1, D.tape_full, w->stream));
+    CU(launch_forward(D.tape_full ? w->Tr : w->Tf, D, w->x0, 0, w->Tf.horizon, 1, D.tape_full, w->stream));
   if (loss) CU(cudaMemcpyAsync(loss, D.loss, sizeof(float) * w->B, cudaMemcpyDefault, w->stream));
   w->t_now = w->Tf.horizon;
   w->have_rollout = true;
@@ -900,21 +921,21 @@ dp_status dp_set_warmstart(dp_world* w, const float* W, float alpha) {
   if (!w->ws_capable) return fail(DP_EINVAL, "the world was created without warm-start support (desc.warmstart = 0)");
   if (!(alpha >= 0.f && alpha <= 1.f)) return fail(DP_EINVAL, "alpha must lie in [0, 1]");
   if (w->have_rollout) w->have_rollout = false;  // the recorded tape belongs to the other solver
-  w->Tf.ws_alpha = w->Tb.ws_alpha = w->Ts.ws_alpha = alpha;
+  w->Tf.ws_alpha = w->Tb.ws_alpha = w->Ts.ws_alpha = w->Tr.ws_alpha = alpha;
   if (!W) {
-    w->Tf.ws = w->Tb.ws = w->Ts.ws = 0;
+    w->Tf.ws = w->Tb.ws = w->Ts.ws = w->Tr.ws = 0;
     return DP_OK;
   }
   CU(cudaMemcpyAsync(w->ws_master, W, sizeof(float) * WsTC::PARAMS, cudaMemcpyDefault, w->stream));
   CU(launch_ws_prep(w->ws_master, w->ws_tc, w->ws_b, w->stream));
-  w->Tf.ws = w->Tb.ws = w->Ts.ws = 1;
+  w->Tf.ws = w->Tb.ws = w->Ts.ws = w->Tr.ws = 1;
   {  // an identically zero network is the damped start: the kernels skip its evaluation
     std::vector<float> hw(WsTC::PARAMS);
     CU(cudaMemcpyAsync(hw.data(), w->ws_master, sizeof(float) * WsTC::PARAMS, cudaMemcpyDeviceToHost, w->stream));
     CU(cudaStreamSynchronize(w->stream));
     int nz = 0;
     for (float x : hw) nz |= x != 0.f;
-    w->Tf.ws_net = w->Tb.ws_net = w->Ts.ws_net = nz;
+    w->Tf.ws_net = w->Tb.ws_net = w->Ts.ws_net = w->Tr.ws_net = nz;
   }
   return DP_OK;
 }

@@ -12,6 +12,12 @@ static cudaError_t launch_forward_t(const DevTopo& T, const DevPtrs& D, const fl
   k_forward<RV, REC, Q><<<T.Bp / 32, 32, smem, s>>>(T, D, x0, t0, nsteps, rollout);
   return cudaGetLastError();
 }
+cudaError_t forward_groups_one_warp(const DevTopo& T1, int* n) {
+  const size_t smem = SM_BYTES(T1);
+  cudaError_t e = cudaFuncSetAttribute(k_forward<SL, true, DynTopo>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_forward<SL, true, DynTopo>, 32, smem);
+}
 cudaError_t launch_forward(const DevTopo& T, const DevPtrs& D, const float* x0, int t0, int nsteps, int rollout,
                            int record, cudaStream_t s) {
   // robots whose blocks are scheduled and fit on chip run on four warps per group; the one-warp

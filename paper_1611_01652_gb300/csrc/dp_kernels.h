@@ -19,6 +19,10 @@ cudaError_t launch_param_in(int B, int Bp, int o, int n, const float* src, float
 cudaError_t launch_pad_scalar(int B, int Bp, const float* src, float* dst, cudaStream_t s);
 cudaError_t launch_forward(const DevTopo& T, const DevPtrs& D, const float* x0, int t0, int nsteps, int rollout,
                            int record, cudaStream_t s);
+// CTAs (groups of 32 instances) an SM holds of a recorded rollout of a robot without a compiled topology,
+// on one warp a group (layout T1) and on blocks (layout T4).
+cudaError_t forward_groups_one_warp(const DevTopo& T1, int* n);
+cudaError_t forward_groups_blk_dyn(const DevTopo& T4, int* n);
 cudaError_t launch_forward_blk(const DevTopo& T, const DevPtrs& D, const float* x0, int t0, int nsteps, int rollout,
                                int record, cudaStream_t s);
 cudaError_t launch_forward_blk_arm(const DevTopo& T, const DevPtrs& D, const float* x0, int t0, int nsteps, int rollout,

@@ -17,7 +17,8 @@ struct ExtLayout {
 
 struct dp_world {
   DevTopo Tf, Tb;  // same topology; forward / backward shared-memory layouts
-  DevTopo Ts;      // forward layout of the four-warp reverse pass's segment recompute
+  DevTopo Ts;      // forward layout of the block reverse pass's segment recompute
+  DevTopo Tr;      // forward layout of recorded rollouts
   DevPtrs D;
   cudaStream_t stream = nullptr;
   int device = 0;  // the CUDA device current at creation (the world's buffers live there)

@@ -214,3 +214,15 @@ def test_colliding_spheres_match_rows(monkeypatch):
     assert got[2][:, :, got[3].schedule()["kind"] == PN].any()
     one_warp(monkeypatch)
     same(got, solve(m, 60, 5, 16, True))
+
+
+def test_many_balls_record_on_one_warp():
+    """At seven groups an SM and above, recorded rollouts of robots without joints take one warp a group,
+    their reverse pass blocks: against the one-warp kernels."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    few = WL.ball(B=64, horizon=20)
+    m = few.subset(np.arange(32 * (7 * sms + 1) - 5) % few.B)
+    m.state0[:, :, 14] = np.where(np.arange(m.B) % 3 == 0, -1.0, m.state0[:, 0, 14])[:, None]  # a third hits the ground at once
+    got = solve(m, 20, 3, None, True)
+    assert got[2].any()
+    same(got, solve(m, 20, 3, None, True, one_warp=True))
