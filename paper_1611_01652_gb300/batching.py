@@ -4,7 +4,7 @@ Instances are binned by topology (one World per bin, since a world's kernels are
 to one topology); inside a bin they are ordered by horizon, longest first, so that the 32
 instances of a warp have similar horizons and each warp steps only to its own longest one. Each
 bin gets the launch configuration an autotuner picked by timing short rollouts: the mapping of
-a group of 32 instances (four warps, with the compiled topology's kernels, or one warp),
+a group of 32 instances (the solver-block kernels on several warps, or one warp),
 constraint rows on chip or in global memory, whole solver tape or checkpoint segments, split
 count of the controller-gradient reduction. All bins run concurrently, each on its own stream, and the
 whole pass (every bin's rollout and reverse pass, and the sum of the controller gradients) can
@@ -28,8 +28,8 @@ def _order_by_horizon(m):
     return m.subset(perm), perm
 
 
-# one warp per group of 32 instances with every row/tape/split choice; four warps per group (the
-# compiled topologies' kernels, which keep the rows on chip and the whole tape) with each split
+# one warp per group of 32 instances with every row/tape/split choice; the solver-block kernels (several
+# warps per group, records on chip, here with the whole tape) with each split
 CANDIDATES = ([dict(rows_global=rg, ckpt_every=ck, dw_splits=sp, one_warp=True)
                for rg, ck, sp in itertools.product((False, True), (0, 16), (64, 256))] +
               [dict(rows_global=False, ckpt_every=0, dw_splits=sp, one_warp=False) for sp in (64, 256)])

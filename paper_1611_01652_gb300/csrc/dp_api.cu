@@ -232,7 +232,7 @@ void plan_smem(DevTopo& T, bool backward, int smem_floats_max, bool rows_on_chip
   T.sm_total = o;
 }
 
-// Shared-memory plans of the four-warp step (units of 32 floats). Forward; the first `keep` units stay
+// Shared-memory plans of the kernels on blocks (units of 32 floats). Forward; the first `keep` units stay
 // free (the reverse pass's segment recompute leaves its state adjoint there).
 void plan_smem_blk_fwd(DevTopo& T, int keep = 0) {
   int o = keep;
@@ -540,7 +540,7 @@ dp_status dp_create_world(const dp_batch_desc* d, void* stream, dp_world** out) 
   plan_smem(w->Tf, false, smem_max / (int)sizeof(float), d->rows_global == 0);
   plan_smem(w->Tb, true, smem_max / (int)sizeof(float));
   const DevTopo one = w->Tf;  // the one-warp layout
-  // The four-warp step, unless the world asks for one warp per group or rows in global memory (or
+  // The kernels on blocks, unless the world asks for one warp per group or rows in global memory (or
   // the environment forces the one-warp kernels, for comparison).
   std::vector<int32_t> prog;
   if (!T.one_warp && d->rows_global == 0 && plan_blocks(T, prog)) {

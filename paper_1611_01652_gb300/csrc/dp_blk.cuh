@@ -1,16 +1,17 @@
-// One step of the engine on the four warps of a CTA that share a group of 32 instances (a lane is
-// an instance in every warp), for any robot whose constraint rows fit on chip.
+// One step of the engine on the warps of a CTA that share a group of 32 instances (a lane is an instance
+// in every warp; eight warps for the compiled topologies, four else: plan_blocks), for any robot whose constraint rows fit on chip.
 //
 // The work of a step is cut into items: joints (the up to seven rows of one hinge or ball joint)
-// and contacts (the three rows of one sphere). Outside the solver, item k belongs to warp k % 4 and
-// body b to warp b % 4; every quantity of an item (its lever arms, axes, effective masses) is
+// and contacts (the three rows of one sphere). Outside the solver, item k (joints,
+// contacts and pairs each counted from 0) belongs to warp k % blk_nw() and body b to warp b % blk_nw(); every quantity of an item (its lever arms, axes, effective masses) is
 // formed once and kept in a compact record, from which the Jacobian of each row is a sign and a
 // permutation. In the solver the rows of one item that are adjacent in the sweep order of both of
 // its bodies form a block; the host schedules the blocks into levels of independent ones
 // (plan_blocks in dp_plan.cu), a warp loads the two bodies' velocities from shared memory, runs
 // the block's rows in registers and stores them back, and the warps meet at one CTA barrier per
-// level that has a live block. Every body sees its rows in the order (colour, slot), so the
-// result is that of the sequential sweep, bit for bit.
+// level that has a live block. Every body sees its rows in the order (colour, slot) of the sequential
+// sweep. The compiled topologies' rollouts are its rollouts bit for bit; a row of another robot may be
+// rounded otherwise in a last place.
 //
 // Why: one warp running the whole sweep (unrolled over the slots, velocities in registers) spent
 // about 125 cycles per row update on one scheduler of four, with a straight-line body of some 70 KB
@@ -119,7 +120,7 @@ __device__ __forceinline__ void blk_load(const DevTopo& T, const DevPtrs& D) {
 
 // This warp's stream of the step: the live blocks of each level in order, a barrier after every
 // level that has a live block on some warp, and a zero at the end. Lane l handles level l; the
-// streams of the four warps hold the same number of barriers, so they cannot deadlock. reverse: the
+// streams of all warps hold the same number of barriers, so they cannot deadlock. reverse: the
 // levels and the blocks of a level last first (the reverse sweeps).
 __device__ __forceinline__ void blk_stream(const DevTopo& T, int warp, bool reverse = false) {
   const int lane = threadIdx.x & 31;
@@ -366,7 +367,7 @@ __device__ __forceinline__ void pair_assemble(const DevTopo& T, const SL& S, con
   R[PF_MU] = sqrtf(P[T.o_sph_mu + k] * P[T.o_sph_mu + l]);
 }
 
-// Every record, item k by warp k % 4 (V: velocities after the external impulses; ao: the step's
+// Every record, item k by warp k % blk_nw() (V: velocities after the external impulses; ao: the step's
 // activity flags of this instance, or NULL; INV: with the I^-1 J_w fields).
 template <bool INV, class G, class VV>
 __device__ __forceinline__ void blk_assemble(const DevTopo& T, const SL& S, const G& P, const SL& X, const VV& V, uint8_t* ao,

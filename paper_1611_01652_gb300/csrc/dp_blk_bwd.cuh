@@ -1,4 +1,4 @@
-// The reverse-mode kernels on four warps per group of 32 instances (items, blocks and records of
+// The reverse-mode kernels on blocks, one CTA per group of 32 instances (items, blocks and records of
 // dp_blk.cuh). A reverse step
 //   - reverses the loss term and the integrator (bodies),
 //   - re-forms the step's records from x_t (items), bit for bit those of the rollout,
@@ -10,7 +10,7 @@
 //   - pushes every item's adjoints to its bodies: the item's warp writes one package per side over
 //     its record, and the bodies' warps add the packages of their items in slot order,
 //   - reverses the external impulses (bodies), the controller (tensor-core layers split over the
-//     four warps) and the hinge kinematics (items, packages again).
+//     warps) and the hinge kinematics (items, packages again).
 // A body belongs to one block at a time (levels), one warp outside the sweeps, so every sum has one
 // writer and a fixed order.
 // The compiled topologies (kernels with SEQ) form the same adjoints row by row: their blocks, items and
@@ -1124,7 +1124,7 @@ __device__ __forceinline__ void mask_delta(float (&d)[NT][4], int mt, int n1, co
     if (!(act[(size_t)(c + 1) * N + r0 + 8] > 0.f)) d[nt][3] = 0.f;
   }
 }
-// The tensor-core controller reversed on the four warps: ub the output adjoint, sbar receives the
+// The tensor-core controller reversed on the CTA's warps: ub the output adjoint, sbar receives the
 // input adjoint, col the step's dump column of lane 0. The planes (four of [32][H + 8] bfloat16) lie
 // over the records, whose packages have been added up by then. Ends before a barrier.
 template <int H, int NW>
@@ -1504,7 +1504,7 @@ __global__ void __launch_bounds__(32 * Q::NW, 1) k_backward_ext_blk(const __grid
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int i = blockIdx.x * 32 + lane, Bp = T.Bp, nf = 18 * T.nb;
   const RevCtx C = rev_ctx(T, D, g_smem + lane, i);
-  const int Tw = warp_horizon(D, i);  // the same for the CTA's four warps
+  const int Tw = warp_horizon(D, i);  // the same for the CTA's warps
   if (t >= Tw) return;                // this group's rollout ended before step t
   blk_load(T, D);
   const size_t sb = (size_t)nf * Bp;

@@ -1,4 +1,4 @@
-// The rollout kernel on four warps per group of 32 instances (stages of dp_blk.cuh).
+// The rollout kernel on blocks, one CTA per group of 32 instances (stages of dp_blk.cuh).
 #pragma once
 #include "dp_blk.cuh"
 
@@ -7,7 +7,7 @@
 // SEQ the parent's share of J v is one chain of multiply-adds from the linear velocity on and the
 // linear update is fused (the quadruped's and the arms' worlds); without it the angular product is
 // summed by itself and the linear impulse is rounded first (every other robot). Each keeps the
-// rounding its worlds have always had. NW: the warps of a CTA (blk_warps in dp_plan.cu).
+// rounding its worlds have always had. NW: the warps of a CTA (plan_blocks in dp_plan.cu).
 struct BlkQuad {
   static constexpr int CTRL_H = 128, NW = 8;
   static constexpr bool SEQ = true;
@@ -60,7 +60,7 @@ __device__ __forceinline__ void store_hidden(const float (&acc)[NT][4], int mt, 
   }
 }
 
-// The tensor-core controller on the CTA's four warps: each hidden layer's columns are split over
+// The tensor-core controller on the CTA's warps: each hidden layer's columns are split over
 // the warps (both 16-row tiles of a weight fragment are multiplied with one load of it), the
 // output layer's two row tiles over warps 0 and 1. Every output's sum runs over k in increasing
 // order. in: the features, out: the outputs, dump: the step's dump column of lane 0 (or NULL).
@@ -155,7 +155,7 @@ __device__ __forceinline__ void ctrl_forward_blk(const DevTopo& T, const DevPtrs
   }
 }
 
-// The fp32-arithmetic controller on the four warps: 8 outputs of a layer per warp and pass.
+// The fp32-arithmetic controller on the CTA's warps: 8 outputs of a layer per warp and pass.
 __device__ __forceinline__ void controller_forward_nw(const DevTopo& T, const DevPtrs& D, const SL* act, int warp) {
   for (int l = 0; l < T.n_layers; ++l) {
     dense_fwd(D.Wt + T.w_off[l], D.bias + T.w_off[l], T.widths[l], T.widths[l + 1], act[l], act[l + 1],
@@ -573,8 +573,8 @@ __device__ __forceinline__ void blk_step(const DevTopo& T, const DevPtrs& D, con
   cta_sync();
 }
 
-// Rollouts and steps (see k_forward in dp_steps.cuh for rollout's values) on four warps per group of
-// 32 instances, one CTA per group.
+// Rollouts and steps (see k_forward in dp_steps.cuh for rollout's values) on blocks, one CTA per group of
+// 32 instances.
 template <bool REC, class Q>
 __global__ void __launch_bounds__(32 * Q::NW, 1) k_forward_blk(const __grid_constant__ DevTopo T, const __grid_constant__ DevPtrs D,
                                                         const float* __restrict__ x0, int t0, int nsteps, int rollout) {

@@ -1,5 +1,5 @@
 // Launchers of the one-warp reverse-mode kernel k_backward, and the choice between it and the
-// four-warp kernels of dp_bwd_blk.cu.
+// kernels on blocks (dp_bwd_blk.cu).
 #include "dp_steps.cuh"
 #include "dp_kernels.h"
 
@@ -12,7 +12,7 @@ static cudaError_t launch_backward_q(const DevTopo& T, const DevPtrs& D, cudaStr
   return cudaGetLastError();
 }
 cudaError_t launch_backward(const DevTopo& T, const DevTopo& Ts, const DevPtrs& D, cudaStream_t s) {
-  if (T.blk_bwd) return launch_backward_blk(T, Ts, D, s);  // four warps per group
+  if (T.blk_bwd) return launch_backward_blk(T, Ts, D, s);
   if (T.topo_id == QuadrupedTopo::id) return launch_backward_q<QuadrupedTopo>(T, D, s);
   return launch_backward_q<DynTopo>(T, D, s);
 }

@@ -1,4 +1,4 @@
-// Launchers of the four-warp reverse kernels for the quadruped's worlds, and the choice
+// Launchers of the reverse kernels on blocks for the quadruped's worlds, and the choice
 // between the kernels.
 #include "dp_blk_bwd.cuh"
 #include "dp_kernels.h"

@@ -1,4 +1,4 @@
-// Launchers of the four-warp reverse kernels for the uneven batch's arms.
+// Launchers of the reverse kernels on blocks for the uneven batch's arms.
 #include "dp_blk_bwd.cuh"
 #include "dp_kernels.h"
 

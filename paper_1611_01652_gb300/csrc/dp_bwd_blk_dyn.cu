@@ -1,4 +1,4 @@
-// Launchers of the four-warp reverse kernels for every other robot.
+// Launchers of the reverse kernels on blocks for every other robot.
 #include "dp_blk_bwd.cuh"
 #include "dp_kernels.h"
 

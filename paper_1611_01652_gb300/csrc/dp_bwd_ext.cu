@@ -1,5 +1,5 @@
 // Launchers of the per-step reverse kernel of the wide controller's path, one warp per group of 32
-// instances (the four-warp kernel's launcher is in dp_bwd_blk.cu).
+// instances (the block kernel's launcher is in dp_bwd_blk.cu).
 #include "dp_steps.cuh"
 #include "dp_kernels.h"
 

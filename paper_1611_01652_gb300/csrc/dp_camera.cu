@@ -371,8 +371,7 @@ __global__ void __launch_bounds__(kThreads, DPK_RENDER_BLOCKS) k_render(const __
   }
 }
 
-// Adds six consecutive values (two texels) at D + i, which starts at a multiple of four floats below
-// n: with 16-byte reductions over the aligned window of eight or twelve floats around them, the rest
+// Adds six consecutive values (two texels) at D + i of a buffer of n floats: with 16-byte reductions over the aligned window of eight or twelve floats around them, the rest
 // of the window zeros; one by one where the window would leave the buffer (or it is not aligned).
 __device__ __forceinline__ void red_texels(float* D, size_t i, size_t n, bool vec, const float (&w)[6]) {
   const size_t b = i & ~(size_t)3;

@@ -52,7 +52,7 @@ struct DevTopo {
   int iters, horizon, features, imu_body, loss_kind, loss_mode, loss_body;
   int n_layers, skip, n_params, n_motors, ctrl_round;  // ctrl_round: 1 = bfloat16 storage points
   int topo_id;  // 0: run-time topology loops; otherwise the compiled topology with this id
-  int one_warp;  // 1: every launch on one warp per group (no four-warp kernels)
+  int one_warp;  // 1: every launch on one warp per group (no block kernels)
   int mlp_tc;   // 1: the controller is the 24-128-128-8 bfloat16 network, run on the tensor cores
   // 1: the controller is evaluated between step launches by batched tensor-core products over all
   // instances (wide bfloat16 networks); the step kernels read its output u_t and write the next
@@ -89,14 +89,13 @@ struct DevTopo {
   int sm_x0, sm_x, sm_xb, sm_vb, sm_iinv, sm_invm, sm_th, sm_thd, sm_ua, sm_wst, sm_wbr, sm_lam, sm_u;
   int sm_thb, sm_thdb, sm_uab, sm_wstb, sm_iinvb, sm_invmb, sm_rc, sm_sbar, sm_vw, sm_zb, sm_act[DPK_MAXL + 1], sm_rows,
       sm_total;
-  // four-warp step (dp_blk.cuh; laid out by plan_blocks): blk = 1 when the robot's solver blocks
-  // are scheduled and its records fit on chip; byte offsets in the program's region of shared
+  // solver blocks (dp_blk.cuh; laid out by plan_blocks): byte offsets in the program's region of shared
   // memory (sm_prog): level table, bodies' item lists (first index per body, entries), live flags,
   // streams; slots of each joint's first linear row, limit row and servo row, and of the contacts
   int blk_nw;  // warps of a CTA
-  int blk, blk_nops, blk_nlev, blk_single, blk_words, blk_bytes_total;
+  int blk_nops, blk_nlev, blk_single, blk_words, blk_bytes_total;
   int blk_lev, blk_inc0, blk_inc, blk_live, blk_stream, blk_stream_len, sm_prog;
-  int blk_fwd, blk_bwd;  // 1: rollouts and steps / reverse passes of this world run on the four-warp step
+  int blk_fwd, blk_bwd;  // 1: rollouts and steps / reverse passes of this world run on blocks
   int rec_rows;          // 1: the tape records hold the constraint rows (read by the one-warp reverse)
   int rec_j, rec_c, rec_p;  // strides of the joints', contacts' and pairs' records
   int sm_rlam, sm_rbr;   // reverse on blocks: staged tape lines (impulses, clamp branches), and where the

@@ -317,17 +317,15 @@ struct RowGeo {
   bool active;
 };
 
-// Assemble constraint slots s0, s0 + sstep, ... of this instance into rows (every slot by
-// default; each slot's row depends on the state alone, so the slots may be split over warps).
+// Assemble this instance's constraint slots into rows.
 template <class RV>
-__device__ void assemble_rows(const DevTopo& T, const LaneT<RV>& L, const SL& X, uint8_t* active_out, int s0 = 0,
-                              int sstep = 1) {
+__device__ void assemble_rows(const DevTopo& T, const LaneT<RV>& L, const SL& X, uint8_t* active_out) {
   const SL& S = L.S;
   const float h = T.dt;
   const float bh = T.beta / h;
   const float INF = __int_as_float(0x7f800000);
   const float3 ez = f3(0.f, 0.f, 1.f);
-  for (int s = s0; s < T.nslots; s += sstep) {
+  for (int s = 0; s < T.nslots; ++s) {
     const int kind = T.skind[s], idx = T.sidx[s], sub = T.ssub[s], a = T.sa[s], b = T.sb[s];
     float3 lin = f3(0.f, 0.f, 0.f), angA = lin, angB = lin;
     float bias = 0.f, bnd = 0.f;

@@ -20,7 +20,7 @@ cudaError_t forward_groups_one_warp(const DevTopo& T1, int* n) {
 }
 cudaError_t launch_forward(const DevTopo& T, const DevPtrs& D, const float* x0, int t0, int nsteps, int rollout,
                            int record, cudaStream_t s) {
-  // robots whose blocks are scheduled and fit on chip run on four warps per group; the one-warp
+  // robots whose blocks are scheduled and fit on chip run on blocks; the one-warp
   // kernels take larger robots, worlds that keep their rows in global memory, and those that ask
   // for one warp
   if (T.blk_fwd) return launch_forward_blk(T, D, x0, t0, nsteps, rollout, record, s);

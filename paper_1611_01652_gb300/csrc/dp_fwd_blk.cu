@@ -1,4 +1,4 @@
-// Launcher of the four-warp rollout kernel k_forward_blk for the quadruped's worlds, and the choice
+// Launcher of the rollout kernel k_forward_blk for the quadruped's worlds, and the choice
 // between the kernels.
 #include "dp_blk_fwd.cuh"
 #include "dp_kernels.h"

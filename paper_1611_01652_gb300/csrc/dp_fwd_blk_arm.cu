@@ -1,4 +1,4 @@
-// Launcher of the four-warp rollout kernel k_forward_blk for the uneven batch's arms.
+// Launcher of the rollout kernel k_forward_blk for the uneven batch's arms.
 #include "dp_blk_fwd.cuh"
 #include "dp_kernels.h"
 

@@ -1,4 +1,4 @@
-// Launcher of the four-warp rollout kernel k_forward_blk for every other robot.
+// Launcher of the rollout kernel k_forward_blk for every other robot.
 #include "dp_blk_fwd.cuh"
 #include "dp_kernels.h"
 

@@ -1,5 +1,5 @@
 // The persistent rollout (forward) and reverse-mode kernel templates on one warp per group of 32
-// instances: robots too large for the four-warp step, worlds that keep rows in global memory, and
+// instances: robots too large for the block kernels, worlds that keep rows in global memory, and
 // those that ask for one warp.
 #pragma once
 #include <cuda_runtime.h>
