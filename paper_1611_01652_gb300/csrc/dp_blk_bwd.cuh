@@ -451,8 +451,7 @@ __device__ __forceinline__ void blk_sweeps_rev(const DevTopo& T, const SL& S, co
     if constexpr (ROWS) {  // (a compiled topology has no sphere pairs)
       if (type == BT_GROUND) rx_contact(T, S, rt, op, contact_rec(T, S, idx), A, ready);
       else if (type == BT_JOINT) {
-        if (op.mask() == 31) rx_joint<true>(T, S, rt, op, joint_rec(T, S, idx), A, B, ready);
-        else rx_joint<false>(T, S, rt, op, joint_rec(T, S, idx), A, B, ready);
+        rx_joint(T, S, rt, op, joint_rec(T, S, idx), A, B, ready);
       } else rx_hinge(T, S, rt, op, joint_rec(T, S, idx), A, B, ready);
     } else if (type == BT_GROUND) rev_contact(T, S, rt, op, contact_rec(T, S, idx), A, ready);
     else if (type == BT_JOINT) {

@@ -189,74 +189,70 @@ __device__ __forceinline__ float rx_ang(const DevTopo& T, bool world, float la, 
   return jvb;
 }
 
-// Blocks, last row first (see rev_joint and its neighbours in dp_blk_bwd.cuh for what is loaded when).
-template <bool FULL, class TP, class RD>
+// Blocks, last row first (see rev_joint and its neighbours in dp_blk_bwd.cuh for what is loaded when). A
+// joint's five rows and a contact's three are one block each (plan_blocks sees to it).
+template <class TP, class RD>
 __device__ __forceinline__ void rx_joint(const DevTopo& T, const SL& S, const TP& tp, const BlkOp& op, const SL& R, RowBody& A,
                                          RowBody& B, const RD& ready) {
-  const int mask = FULL ? 31 : op.mask(), s0 = op.slot();
+  const int s0 = op.slot();
   const bool world = op.a() < 0;
   const SL Q = R.at(JR_N);
   const float3 ra = R.v3(JF_RA), rb = R.v3(JF_RB);
   float la[5], lb[5], lam[5], me[5], bi[5], mea[5], meb[5], acc[3][5], bia[2];
   float3 t[2], ca[2], cb[2];
 #pragma unroll
-  for (int k = 0; k < 5; ++k)
-    if (mask >> k & 1) {
-      const int f = k < 3 ? JX_LIN + 7 * k + LX_ME : JX_ANG + 9 * (k - 3) + AX_ME;
-      la[k] = tp.la[s0 + k];
-      lb[k] = tp.lb[s0 + k];
-      lam[k] = S[T.sm_lam + s0 + k];
-      me[k] = R[JF_ME + k];
-      bi[k] = R[JF_BI + k];
-      mea[k] = Q[f];
-      meb[k] = Q[f + 1];
-      if (k >= 3) t[k - 3] = R.v3(JF_T + 3 * (k - 3));
-    }
+  for (int k = 0; k < 5; ++k) {
+    const int f = k < 3 ? JX_LIN + 7 * k + LX_ME : JX_ANG + 9 * (k - 3) + AX_ME;
+    la[k] = tp.la[s0 + k];
+    lb[k] = tp.lb[s0 + k];
+    lam[k] = S[T.sm_lam + s0 + k];
+    me[k] = R[JF_ME + k];
+    bi[k] = R[JF_BI + k];
+    mea[k] = Q[f];
+    meb[k] = Q[f + 1];
+    if (k >= 3) t[k - 3] = R.v3(JF_T + 3 * (k - 3));
+  }
   ready();
   float unused;
 #pragma unroll
   for (int k = 4; k >= 3; --k)
-    if (mask >> k & 1)
-      bia[k - 3] = rx_ang(T, world, la[k], lb[k], me[k], bi[k], 0, -t[k - 3], A, B, lam[k], mea[k], meb[k], unused, ca[k - 3], cb[k - 3]);
-  if (mask & 4) rx_lin<2>(T, world, la[2], lb[2], me[2], bi[2], ra, rb, A, B, lam[2], mea[2], meb[2], acc[2]);
-  if (mask & 2) rx_lin<1>(T, world, la[1], lb[1], me[1], bi[1], ra, rb, A, B, lam[1], mea[1], meb[1], acc[1]);
-  if (mask & 1) rx_lin<0>(T, world, la[0], lb[0], me[0], bi[0], ra, rb, A, B, lam[0], mea[0], meb[0], acc[0]);
+    bia[k - 3] = rx_ang(T, world, la[k], lb[k], me[k], bi[k], 0, -t[k - 3], A, B, lam[k], mea[k], meb[k], unused, ca[k - 3], cb[k - 3]);
+  rx_lin<2>(T, world, la[2], lb[2], me[2], bi[2], ra, rb, A, B, lam[2], mea[2], meb[2], acc[2]);
+  rx_lin<1>(T, world, la[1], lb[1], me[1], bi[1], ra, rb, A, B, lam[1], mea[1], meb[1], acc[1]);
+  rx_lin<0>(T, world, la[0], lb[0], me[0], bi[0], ra, rb, A, B, lam[0], mea[0], meb[0], acc[0]);
   // (every row's accumulators are its own block's: the loads here wait for nothing)
 #pragma unroll
-  for (int k = 0; k < 3; ++k)
-    if (mask >> k & 1) {
-      const SL q = Q.at(JX_LIN + 7 * k);
+  for (int k = 0; k < 3; ++k) {
+    const SL q = Q.at(JX_LIN + 7 * k);
 #pragma unroll
-      for (int c = 0; c < 4; ++c) acc[k][c] += q[c];
-      acc[k][4] += q[LX_BI];
+    for (int c = 0; c < 4; ++c) acc[k][c] += q[c];
+    acc[k][4] += q[LX_BI];
+  }
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const SL q = Q.at(JX_ANG + 9 * k);
+    ca[k] = q.v3(AX_A) + ca[k];
+    cb[k] = q.v3(AX_B) + cb[k];
+    bia[k] += q[AX_BI];
+  }
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const SL q = Q.at(k < 3 ? JX_LIN + 7 * k : JX_ANG + 9 * (k - 3));
+    S[T.sm_lam + s0 + k] = lam[k];
+    if (k < 3) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) q[c] = acc[k][c];
+      q[LX_ME] = mea[k];
+      q[LX_MEB] = meb[k];
+      q[LX_BI] = acc[k][4];
+    } else {
+      q.s3(AX_A, ca[k - 3]);
+      q.s3(AX_B, cb[k - 3]);
+      q[AX_ME] = mea[k];
+      q[AX_MEB] = meb[k];
+      q[AX_BI] = bia[k - 3];
     }
-#pragma unroll
-  for (int k = 0; k < 2; ++k)
-    if (mask >> (3 + k) & 1) {
-      const SL q = Q.at(JX_ANG + 9 * k);
-      ca[k] = q.v3(AX_A) + ca[k];
-      cb[k] = q.v3(AX_B) + cb[k];
-      bia[k] += q[AX_BI];
-    }
-#pragma unroll
-  for (int k = 0; k < 5; ++k)
-    if (mask >> k & 1) {
-      const SL q = Q.at(k < 3 ? JX_LIN + 7 * k : JX_ANG + 9 * (k - 3));
-      S[T.sm_lam + s0 + k] = lam[k];
-      if (k < 3) {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) q[c] = acc[k][c];
-        q[LX_ME] = mea[k];
-        q[LX_MEB] = meb[k];
-        q[LX_BI] = acc[k][4];
-      } else {
-        q.s3(AX_A, ca[k - 3]);
-        q.s3(AX_B, cb[k - 3]);
-        q[AX_ME] = mea[k];
-        q[AX_MEB] = meb[k];
-        q[AX_BI] = bia[k - 3];
-      }
-    }
+  }
 }
 template <class TP, class RD>
 __device__ __forceinline__ void rx_hinge(const DevTopo& T, const SL& S, const TP& tp, const BlkOp& op, const SL& R, RowBody& A,
@@ -285,7 +281,7 @@ __device__ __forceinline__ void rx_hinge(const DevTopo& T, const SL& S, const TP
 template <class TP, class RD>
 __device__ __forceinline__ void rx_contact(const DevTopo& T, const SL& S, const TP& tp, const BlkOp& op, const SL& R, RowBody& A,
                                            const RD& ready) {
-  const int mask = op.mask(), s0 = op.slot();
+  const int s0 = op.slot();
   const SL Q = R.at(CR_N);
   float la[3], lb[3], lam[3], me[3], mea[3], acc[3][3];
   int br[3];
@@ -301,11 +297,6 @@ __device__ __forceinline__ void rx_contact(const DevTopo& T, const SL& S, const 
   const float3 ra = R.v3(CF_RA);
   const float mu = R[CF_MU], bias0 = R[CF_BI];
   ready();
-  if (mask != 7)  // another block of this contact changes their adjoints and sums too
-    for (int m = 0; m < 3; ++m) {
-      lam[m] = S[T.sm_lam + s0 + m];
-      mea[m] = Q[4 * m + CX_ME];
-    }
   const float lnrm = la[0];  // the normal impulse a friction row saw (the normal row comes first)
   auto row = [&](auto MI, auto AI, float bias) {
     constexpr int m = decltype(MI)::value, K = decltype(AI)::value;
@@ -337,24 +328,21 @@ __device__ __forceinline__ void rx_contact(const DevTopo& T, const SL& S, const 
   using I0 = std::integral_constant<int, 0>;
   using I1 = std::integral_constant<int, 1>;
   using I2 = std::integral_constant<int, 2>;
-  if (mask & 4) row(I2{}, I1{}, 0.f);
-  if (mask & 2) row(I1{}, I0{}, 0.f);
-  if (mask & 1) row(I0{}, I2{}, bias0);
+  row(I2{}, I1{}, 0.f);
+  row(I1{}, I0{}, 0.f);
+  row(I0{}, I2{}, bias0);
 #pragma unroll
   for (int m = 0; m < 3; ++m)
-    if (mask >> m & 1)
 #pragma unroll
-      for (int c = 0; c < 3; ++c) acc[m][c] += Q[4 * m + (c < 2 ? c : CX_BI)];
-  S[T.sm_lam + s0] = lam[0];  // (also from a block of friction rows alone)
+    for (int c = 0; c < 3; ++c) acc[m][c] += Q[4 * m + (c < 2 ? c : CX_BI)];
 #pragma unroll
-  for (int m = 0; m < 3; ++m)
-    if (mask >> m & 1) {
-      S[T.sm_lam + s0 + m] = lam[m];
-      Q[4 * m + CX_A] = acc[m][0];
-      Q[4 * m + CX_A + 1] = acc[m][1];
-      Q[4 * m + CX_ME] = mea[m];
-      Q[4 * m + CX_BI] = acc[m][2];
-    }
+  for (int m = 0; m < 3; ++m) {
+    S[T.sm_lam + s0 + m] = lam[m];
+    Q[4 * m + CX_A] = acc[m][0];
+    Q[4 * m + CX_A + 1] = acc[m][1];
+    Q[4 * m + CX_ME] = mea[m];
+    Q[4 * m + CX_BI] = acc[m][2];
+  }
 }
 
 // ------------------------------------------------------------------------------ items

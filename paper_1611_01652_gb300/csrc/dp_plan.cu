@@ -80,6 +80,9 @@ bool plan_blocks(DevTopo& T, std::vector<int32_t>& blob) {
   }
   const int n = (int)ops.size();
   if (n > 63 || n == 0) return false;
+  if (T.topo_id != 0)  // (true of every compiled topology: their reverse blocks are written for whole items)
+    for (const Op& o : ops)
+      if ((o.type == 0 && o.mask != 31) || o.type == 4 || (o.type == 3 && o.mask != 7)) return false;
   for (int k = n - 1; k >= 0; --k) {
     for (int u : ops[k].users) ops[k].path = std::max(ops[k].path, ops[u].path);
     ops[k].path += ops[k].weight;
