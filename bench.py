@@ -42,9 +42,9 @@ RESID_TOL = 0.02
 WS_ITERS = (5, 7, 10, 14)
 # DRAM bytes (read + written) per instance-step of k_backward_blk, damped start at 10 sweeps:
 # dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture of one launch at B = 1024,
-# T = 20 (176.9 MB + 15.8 MB, the kernel as built now) / (B T). The tape is read once per
+# T = 20 (176.5 MB + 15.5 MB, the kernel as built now) / (B T). The tape is read once per
 # launch, so the traffic of the full launch scales with B T.
-BWD_TRAFFIC_PER_INST_STEP = {10: (176907264 + 15763456) / (1024 * 20)}
+BWD_TRAFFIC_PER_INST_STEP = {10: (176489728 + 15459584) / (1024 * 20)}
 
 
 def parse():

@@ -11,8 +11,8 @@
 // were more than 2e-5 of the adjoint's norm away, up to 4.6e-4. Here every sum is that of the sequential
 // walk, so schedules, warps and layouts do not show in it; state, weight, mass and inertia gradients of
 // 138 batches (recurrent, feed-forward and wide quadrupeds, arms) have its bits.
-// What it costs, us with rollout, against the sums by items: quadruped 100 steps 27331 -> 29488, 1000
-// steps warm 166007 -> 180559, recurrent 19418 -> 20957, wide 17199 -> 17675, arms 227453 -> 240750.
+// What it costs, us with rollout, against the sums by items: quadruped 100 steps 27487 -> 28748, 1000
+// steps warm 165907 -> 176146, recurrent 19462 -> 20427, wide 17182 -> 17600, arms 227721 -> 235395.
 // Bound: issue and latency of the blocks' chains, as in dp_blk_bwd.cuh.
 //
 // Products with a coordinate axis' zeros are left out (exact zeros); where a sum's order of rounding
