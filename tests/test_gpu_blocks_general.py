@@ -140,11 +140,11 @@ def blocks(w):
     return len(made), {it for it in made if made.count(it) > 1}
 
 
-def solve(m, horizon, iters, ckpt, warm, **kw):
+def solve(m, horizon, iters, ckpt, warm, net=None, **kw):
     """(loss, final state), every gradient, the activity log and the schedule."""
     w = World(m, horizon=horizon, iters=iters, ckpt_every=ckpt, warmstart=warm, **kw)
     if warm:
-        w.set_warmstart(torch.zeros(WS_PARAMS, device="cuda"), 0.7)
+        w.set_warmstart(torch.zeros(WS_PARAMS, device="cuda") if net is None else net, 0.7)
     W = torch.tensor(m.W, device="cuda") if m.W is not None and len(m.W) else None
     loss = torch.zeros(m.B, device="cuda")
     act = torch.zeros(horizon, m.B, w.n_slots, dtype=torch.uint8, device="cuda")
@@ -226,3 +226,14 @@ def test_many_balls_record_on_one_warp():
     got = solve(m, 20, 3, None, True)
     assert got[2].any()
     same(got, solve(m, 20, 3, None, True, one_warp=True))
+
+
+@pytest.mark.parametrize("name", sorted(ROBOTS))
+def test_learned_start_matches_rows(monkeypatch, name):
+    """A warm-start network that is not zero, two steps (a bfloat16 rounding of its features or hidden units
+    that falls the other way shows later)."""
+    net = torch.tensor(0.05 * WL.xavier_weights([16, 64, 64, 3], 0, np.random.default_rng(2)), device="cuda")
+    m = ROBOTS[name][0](33)
+    got = solve(m, 2, 3, None, True, net)
+    one_warp(monkeypatch)
+    same(got, solve(m, 2, 3, None, True, net))
